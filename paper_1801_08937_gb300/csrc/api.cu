@@ -64,6 +64,8 @@ struct Plan {
     int whole = 0;     // FFT: 1 one transform per whole block (no overlap-save halo), two blocks
                        // per CTA; 2 one block per CTA as an L/2-point complex transform
     FftPasses fp{};
+    bool three = false;   // whole = 2, float32: the three-pass transform
+    bool even = true;     // every segment starts at an even sample
     int f64 = 0;
     int nrhs = 0;
     std::vector<int64_t> lens;
@@ -108,6 +110,8 @@ struct mm_ctx {
     std::vector<double> band;
     DevBuf d_pix, d_psi, d_cs64, d_block_off, d_block_band, d_band64, d_band32, d_banddf, d_csdf;
     bool have_csdf = false;
+    DevBuf w_off, w_win;     // scratch of the pointing check
+    std::vector<int2> win;   // pixel window (smallest, largest) of each block
     int p64 = 1;   // precision of the float64-accurate products: 1 native, 2 double-float
     std::vector<std::unique_ptr<Plan>> plans;
 
@@ -180,6 +184,9 @@ struct mm_ctx {
     DevBuf d_Z32, d_AZ32;              // float32 copies of Z and AZ for mixed-precision M_2l
     bool z32_valid = false;
     int coarse_rank_min = 0;           // smallest coarse rank a right-hand side of the last uneven batch kept
+    // set by a bounded wait of a filter kernel that gave up (pinned host memory the kernels write to)
+    int* h_fault = nullptr;
+    int* d_fault = nullptr;
     // asynchronous stepping
     RhsState* h_st_pinned = nullptr;
     int h_st_pinned_n = 0;
@@ -472,23 +479,17 @@ std::vector<int> dif_frequency(const FftPasses& fp) {
     return k;
 }
 
-// Tables of a whole-block plan run as an M = N/2 point complex transform:
-// twiddles of length M, the pair positions (k, M - k) and, per band, the
-// coefficients (alpha_k, alpha_{M-k}, beta_k) of the paired real-spectrum
-// filter, from the band's length-N spectrum, with 1/M folded in.
-mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, int N, int f64) {
-    const int M = fpM.L;
-    if (ft.L == M && ft.pairs.p) return MM_OK;
+// Spectra of the bands for circular products of N points, in natural order of
+// the frequency and scaled by 1/N: [n_bands][N].
+mm_status band_spectra(mm_ctx* ctx, int N, std::vector<double>& H) {
     FftPasses fpN;
     if (!fft_passes(N, &fpN, 16)) return fail(ctx, MM_ERR_ARG, "no transform plan for the block spectrum");
-    // length-N spectra of the bands (digit-reversed, scaled by 1/N) on the device
-    std::vector<double> twN(2 * (size_t)N);
+    std::vector<double> twN(2 * (size_t)N), h((size_t)ctx->n_bands * N, 0.0);
     for (int e = 0; e < N; ++e) {
         const double ang = -2.0 * M_PI * (double)e / (double)N;
         twN[2 * e] = std::cos(ang);
         twN[2 * e + 1] = std::sin(ang);
     }
-    std::vector<double> h((size_t)ctx->n_bands * N, 0.0);
     for (int b = 0; b < ctx->n_bands; ++b) {
         const double* c = &ctx->band[(size_t)b * (ctx->lam + 1)];
         double* hb = &h[(size_t)b * N];
@@ -499,21 +500,89 @@ mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, in
         }
     }
     std::vector<double> Hp(h.size());
-    {
-        DevBuf d_tw, d_h, d_H, d_work;
-        CK(d_tw.ensure(twN.size() * 8));
-        CK(d_h.ensure(h.size() * 8));
-        CK(d_H.ensure(h.size() * 8));
-        CK(d_work.ensure((size_t)ctx->n_bands * (N + (N >> 4)) * 16));
-        CK(cudaMemcpyAsync(d_tw.p, twN.data(), twN.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-        CK(cudaMemcpyAsync(d_h.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-        launch_fft_spectrum(d_h.as<double>(), d_H.as<double>(), d_work.as<double2>(), d_tw.as<double2>(),
-                            ctx->n_bands, fpN, ctx->stream);
-        CKL();
-        CK(cudaMemcpyAsync(Hp.data(), d_H.p, Hp.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
+    DevBuf d_tw, d_h, d_H, d_work;
+    CK(d_tw.ensure(twN.size() * 8));
+    CK(d_h.ensure(h.size() * 8));
+    CK(d_H.ensure(h.size() * 8));
+    CK(d_work.ensure((size_t)ctx->n_bands * (N + (N >> 4)) * 16));
+    CK(cudaMemcpyAsync(d_tw.p, twN.data(), twN.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(d_h.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    launch_fft_spectrum(d_h.as<double>(), d_H.as<double>(), d_work.as<double2>(), d_tw.as<double2>(), ctx->n_bands, fpN,
+                        ctx->stream);
+    CKL();
+    CK(cudaMemcpyAsync(Hp.data(), d_H.p, Hp.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    const std::vector<int> kN = dif_frequency(fpN);
+    H.resize(h.size());
+    for (int b = 0; b < ctx->n_bands; ++b)
+        for (int p = 0; p < N; ++p) H[(size_t)b * N + kN[p]] = Hp[(size_t)b * N + p];
+    return MM_OK;
+}
+
+// Tables of the three-pass whole-block transform (filter_half3.cuh): twiddles
+// of its passes and, per band, the coefficients of the paired spectrum step in
+// the order of its items.
+mm_status build_half3_tables(mm_ctx* ctx, FftTables& ft, int N) {
+    const int M = N / 2;
+    int r0 = 0, r1 = 0;
+    if (!half3_shape(M, &r0, &r1)) return fail(ctx, MM_ERR_STATE, "not a three-pass length");
+    if (ft.L == M) return MM_OK;
+    std::vector<double> H;
+    TRY(band_spectra(ctx, N, H));
+    const int sr = 9 * r1, nb = r0 * r1, ni = nb / 2 + 1, ra = r0 / 4;
+    std::vector<float> t1, t2;
+    auto put = [](std::vector<float>& t, int64_t e, int64_t n) {
+        const double ang = -2.0 * M_PI * (double)(e % n) / (double)n;
+        t.push_back((float)std::cos(ang));
+        t.push_back((float)std::sin(ang));
+    };
+    for (int q = 1; q < ra + 3; ++q)
+        for (int j = 0; j < sr; ++j) put(t1, (int64_t)j * (q < ra ? q : (q - ra + 1) * ra), M);
+    for (int j = 0; j < 9; ++j)
+        for (int q = 0; q < r1; ++q) put(t2, (int64_t)j * q, sr);
+    std::vector<float> C((size_t)ctx->n_bands * 9 * ni * 4, 0.0f);
+    for (int t = 0; t < ni; ++t) {
+        int g = t / r1, r = t % r1;
+        if (t == nb / 2) {
+            g = 0;
+            r = r1 / 2;
+        } else if (g == 0) {
+            if (r < r1 / 2) g = r0 / 2;
+            else r -= r1 / 2;
+        }
+        for (int q = 0; q < 9; ++q) {
+            const int k = g + r0 * r + nb * q;
+            const double th = 2.0 * M_PI * (double)k / (double)N, sn = std::sin(th), cs = std::cos(th);
+            for (int b = 0; b < ctx->n_bands; ++b) {
+                const double h1 = 2.0 * H[(size_t)b * N + k], h2 = 2.0 * H[(size_t)b * N + M - k];
+                float* o = &C[(((size_t)b * 9 + q) * ni + t) * 4];
+                o[0] = (float)(0.5 * ((h1 + h2) + (h2 - h1) * sn));
+                o[1] = (float)(0.5 * ((h1 + h2) - (h2 - h1) * sn));
+                o[2] = (float)(-0.5 * (h2 - h1) * cs);
+            }
+        }
     }
-    const std::vector<int> kN = dif_frequency(fpN), kM = dif_frequency(fpM);
+    CK(ft.twp.ensure(t1.size() * 4));
+    CK(ft.tw.ensure(t2.size() * 4));
+    CK(ft.Hi.ensure(C.size() * 4));
+    CK(cudaMemcpyAsync(ft.twp.p, t1.data(), t1.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(ft.tw.p, t2.data(), t2.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(ft.Hi.p, C.data(), C.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    ft.L = M;
+    return MM_OK;
+}
+
+// Tables of a whole-block plan run as an M = N/2 point complex transform:
+// twiddles of length M, the pair positions (k, M - k) and, per band, the
+// coefficients (alpha_k, alpha_{M-k}, beta_k) of the paired real-spectrum
+// filter, from the band's length-N spectrum, with 1/M folded in.
+mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, int N, int f64) {
+    const int M = fpM.L;
+    if (ft.L == M && ft.pairs.p) return MM_OK;
+    std::vector<double> Hp;
+    TRY(band_spectra(ctx, N, Hp));
+    const std::vector<int> kM = dif_frequency(fpM);
     std::vector<int> posM(M);
     for (int p = 0; p < M; ++p) posM[kM[p]] = p;
     const int np = M / 2 + 1;
@@ -562,9 +631,9 @@ mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, in
     }
     // coefficients in float64: H_k / M = 2 (H_k / N)
     std::vector<double> coef((size_t)ctx->n_bands * np * 3), coefi((size_t)ctx->n_bands * std::max(ni, 1) * R * 3);
-    std::vector<double> Hn(N);
+    const double* Hn = nullptr;
     auto pair_coef = [&](int k, double* o) {
-        const double h1 = Hn[k], h2 = Hn[M - k];
+        const double h1 = 2.0 * Hn[k], h2 = 2.0 * Hn[M - k];
         const double th = 2.0 * M_PI * (double)k / (double)N;
         const double sn = std::sin(th), cs = std::cos(th);
         o[0] = 0.5 * ((h1 + h2) + (h2 - h1) * sn);
@@ -572,7 +641,7 @@ mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, in
         o[2] = -0.5 * (h2 - h1) * cs;
     };
     for (int b = 0; b < ctx->n_bands; ++b) {
-        for (int p = 0; p < N; ++p) Hn[kN[p]] = 2.0 * Hp[(size_t)b * N + p];
+        Hn = &Hp[(size_t)b * N];
         for (int e = 0; e < np; ++e) pair_coef(order[e], &coef[((size_t)b * np + e) * 3]);
         for (int i = 0; i < ni; ++i)
             for (int q = 0; q < R; ++q) pair_coef(item_kc[i] + NB * q, &coefi[(((size_t)b * ni + i) * R + q) * 3]);
@@ -729,6 +798,8 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
                 s.n_out = (int32_t)std::min<int64_t>(step, hi - c0);
                 s.band = ctx->block_band[b];
                 s.shift = whole ? 0 : ctx->lam;
+                s.win0 = std::max(0, std::min(ctx->win[b].x, ctx->n_pix - 1));
+                s.nwin = ctx->win[b].y < 0 ? 0 : ctx->win[b].y - ctx->win[b].x + 1;
                 push(s);
             }
         }
@@ -750,12 +821,16 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     p->nrhs = nrhs;
     p->lens = lens;
     p->starts = starts;
+    int r0 = 0, r1 = 0;
+    p->three = single && f64 == 0 && half3_shape(L / 2, &r0, &r1);
+    for (const Seg& sg : segs) p->even = p->even && sg.out0 % 2 == 0;
     p->n_work = (int)(single ? segs.size() : segs.size() / 2);
     CK(p->segs.ensure(std::max<size_t>(1, segs.size()) * sizeof(Seg)));
     if (!segs.empty())
         CK(cudaMemcpyAsync(p->segs.p, segs.data(), segs.size() * sizeof(Seg), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    if (variant == 2 && whole == 2) TRY(build_half_tables(ctx, p->ft, fp, L, f64));
+    if (p->three) TRY(build_half3_tables(ctx, p->ft, L));
+    else if (variant == 2 && whole == 2) TRY(build_half_tables(ctx, p->ft, fp, L, f64));
     else if (variant == 2) TRY(build_fft_tables(ctx, p->ft, fp, f64));
     if (f64 == 2 && !ctx->have_csdf) {
         CK(ctx->d_csdf.ensure((size_t)ctx->n_samples * 16));
@@ -856,13 +931,16 @@ void tune_record(const TuneKey& k, const TuneVal& v) {
 
 // Time each candidate plan once (after one warm-up launch) on the current
 // pointing and keep the fastest.  Candidates: the six cheapest FFT plans of
-// the cost model and, for narrow bands, the direct band at two tile sizes.
+// the cost model, every three-pass whole-block plan that fits and, for narrow bands, the direct band at two tile sizes.
 mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& lens, TuneVal* best) {
     struct Opt { int variant, L, whole, V; };
     std::vector<Opt> opts;
     auto cands = fft_candidates(ctx, f64, 0, 0);
-    for (size_t i = 0; i < cands.size() && i < 6; ++i)
-        opts.push_back({2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
+    int r0 = 0, r1 = 0;
+    for (size_t i = 0; i < cands.size(); ++i)   // the three-pass whole blocks are cheaper than the model says
+        if (i < 6 || (f64 == 0 && cands[i].whole == 2 && half3_shape(cands[i].L / 2, &r0, &r1)))
+            opts.push_back(
+                {2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
     if (ctx->lam <= 256)
         for (int tile : {1024, 2048})
             if (direct_smem_bytes(tile, ctx->lam, f64 != 0) <= 200 * 1024) opts.push_back({1, 0, 0, tile});
@@ -974,6 +1052,7 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
         e1 = pr.second;
     }
     a.csdf = ctx->d_csdf.as<float4>();
+    a.fault = ctx->d_fault;
     if (ctx->tmpl_on) {
         if (!plan->lens.empty() || !plan->starts.empty())
             return fail(ctx, MM_ERR_ARG, "template filters: right-hand sides of uneven length are not supported");
@@ -996,6 +1075,8 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
         a.tw = ft.tw.p;
         if (plan->whole == 2) {
             a.half = 1;
+            a.three = plan->three ? 1 : 0;
+            a.even = plan->even ? 1 : 0;
             a.L = plan->L / 2;
             a.pairs = ft.pairs.as<uint32_t>();
             a.items = ft.items.as<uint32_t>();
@@ -1174,6 +1255,13 @@ mm_status pcg_start(mm_ctx* ctx, const V4<double>* b, const std::vector<double>&
     return MM_OK;
 }
 
+// After the stream is synchronised: whether a bounded wait of a filter kernel gave up.
+mm_status filter_fault_check(mm_ctx* ctx) {
+    if (*static_cast<volatile int*>(ctx->h_fault) == 0) return MM_OK;
+    *ctx->h_fault = 0;
+    return fail(ctx, MM_ERR_TIMEOUT, "filter: a bounded wait for a copy to shared memory gave up");
+}
+
 mm_status tc_fault_check(mm_ctx* ctx) {
     int fault = 0;
     CK(m2l_tc_fault_take(ctx->stream, &fault));
@@ -1187,6 +1275,7 @@ mm_status read_state(mm_ctx* ctx) {
     ctx->h_st.resize(ctx->nrhs);
     CK(cudaMemcpyAsync(ctx->h_st.data(), ctx->s_st.p, ctx->nrhs * sizeof(RhsState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    TRY(filter_fault_check(ctx));
     if (ctx->precond == MM_PRECOND_2L) TRY(tc_fault_check(ctx));
     return MM_OK;
 }
@@ -1222,7 +1311,7 @@ mm_status true_residual(mm_ctx* ctx, const V4<double>* x, std::vector<double>& r
     CK(cudaMemcpyAsync(rr.data(), ctx->w_norms.p, ctx->nrhs * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     for (auto& v : rr) v = std::sqrt(std::max(0.0, v));
-    return MM_OK;
+    return filter_fault_check(ctx);
 }
 
 void destroy_graph(mm_ctx* ctx) {
@@ -1610,6 +1699,12 @@ mm_status mm_create(mm_ctx** out, int device, void* cuda_stream, mm_precision pr
     ctx->p64 = prec == MM_FP32_MIXED ? 2 : 1;
     cudaEventCreate(&ctx->ev0);
     cudaEventCreate(&ctx->ev1);
+    if (cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_fault), sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_fault), ctx->h_fault, 0) != cudaSuccess) {
+        mm_destroy(ctx);
+        return MM_ERR_CUDA;
+    }
+    *ctx->h_fault = 0;
     *out = ctx;
     return MM_OK;
 }
@@ -1623,6 +1718,7 @@ mm_status mm_destroy(mm_ctx* ctx) {
         cudaEventDestroy(pr.first);
         cudaEventDestroy(pr.second);
     }
+    if (ctx->h_fault) cudaFreeHost(ctx->h_fault);
     if (ctx->h_st_pinned) cudaFreeHost(ctx->h_st_pinned);
     if (ctx->reduce_host) cudaFreeHost(ctx->reduce_host);
     if (ctx->ev_state) cudaEventDestroy(ctx->ev_state);
@@ -1659,30 +1755,37 @@ mm_status mm_setup_pointing(mm_ctx* ctx, int64_t n_samples, int32_t n_det, int32
     if (n_pix > (1 << 26)) return fail(ctx, MM_ERR_ARG, "n_pix too large");
     for (size_t i = 0; i < (size_t)n_bands * (half_bw + 1); ++i)
         if (!std::isfinite(band[i])) return fail(ctx, MM_ERR_ARG, "band holds a non-finite value");
-    {
-        // the kernels index the map by pix: its range is checked for host and device arrays (a device
-        // array through a bounded host buffer, once per pointing set-up)
-        auto in_range = [n_pix](const int32_t* p, int64_t c) {
-            int32_t lo = 0, hi = -1;
-            for (int64_t i = 0; i < c; ++i) {
-                lo = std::min(lo, p[i]);
-                hi = std::max(hi, p[i]);
-            }
-            return lo >= -1 && hi < n_pix;
-        };
-        if (mem == MM_HOST) {
-            if (!in_range(pix, n_samples)) return fail(ctx, MM_ERR_ARG, "pix out of range [-1, n_pix)");
-        } else {
-            const int64_t chunk = (int64_t)1 << 22;
-            std::vector<int32_t> hb((size_t)std::min<int64_t>(chunk, n_samples));
-            for (int64_t t0 = 0; t0 < n_samples; t0 += chunk) {
-                const int64_t c = std::min<int64_t>(chunk, n_samples - t0);
-                CK(cudaMemcpyAsync(hb.data(), pix + t0, (size_t)c * 4, cudaMemcpyDeviceToHost, ctx->stream));
-                CK(cudaStreamSynchronize(ctx->stream));
-                if (!in_range(hb.data(), c)) return fail(ctx, MM_ERR_ARG, "pix out of range [-1, n_pix)");
-            }
+    // the kernels index the map by pix: its range is checked before anything of the context changes; a device
+    // array by the pass over it that also finds each block's pixel window
+    int64_t longest = 0;
+    for (int b = 0; b < n_blocks; ++b) longest = std::max(longest, block_off[b + 1] - block_off[b]);
+    std::vector<int2> win(n_blocks);
+    DevBuf &d_off = ctx->w_off, &d_win = ctx->w_win;
+    CK(d_off.ensure((size_t)(n_blocks + 1) * 8));
+    CK(d_win.ensure((size_t)n_blocks * sizeof(int2) + 16));
+    auto windows = [&](const int32_t* p, int* bad) -> mm_status {
+        int* d_bad = reinterpret_cast<int*>(d_win.as<int2>() + n_blocks);
+        CK(cudaMemsetAsync(d_bad, 0, 4, ctx->stream));
+        CK(cudaMemcpyAsync(d_off.p, block_off, (size_t)(n_blocks + 1) * 8, cudaMemcpyHostToDevice, ctx->stream));
+        launch_block_windows(p, d_off.as<int64_t>(), n_blocks, longest, n_pix, d_win.as<int2>(), d_bad, ctx->stream);
+        CKL();
+        CK(cudaMemcpyAsync(win.data(), d_win.p, (size_t)n_blocks * sizeof(int2), cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaMemcpyAsync(bad, d_bad, 4, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        return MM_OK;
+    };
+    int bad = 0;
+    if (mem == MM_HOST) {
+        int32_t lo = 0, hi = -1;
+        for (int64_t i = 0; i < n_samples; ++i) {
+            lo = std::min(lo, pix[i]);
+            hi = std::max(hi, pix[i]);
         }
+        bad = lo < -1 || hi >= n_pix;
+    } else {
+        TRY(windows(pix, &bad));
     }
+    if (bad) return fail(ctx, MM_ERR_ARG, "pix out of range [-1, n_pix)");
     destroy_graph(ctx);
     ctx->have_pointing = ctx->have_bd = false;
     ctx->k = 0;
@@ -1702,8 +1805,8 @@ mm_status mm_setup_pointing(mm_ctx* ctx, int64_t n_samples, int32_t n_det, int32
     ctx->band.assign(band, band + (size_t)n_bands * (half_bw + 1));
     const int64_t gb = (n_pix + 255) / 256;
     ctx->grid_x = (int)std::min<int64_t>(gb, 304);
-    CK(ctx->d_pix.ensure(n_samples * 4));
-    CK(ctx->d_psi.ensure(n_samples * 4));
+    CK(ctx->d_pix.ensure(n_samples * 4 + POINTING_SPARE));
+    CK(ctx->d_psi.ensure(n_samples * 4 + POINTING_SPARE));
     CK(ctx->d_cs64.ensure(n_samples * 16));
     CK(copy_in(ctx->d_pix.p, pix, n_samples * 4, mem, ctx->stream));
     CK(copy_in(ctx->d_psi.p, psi, n_samples * 4, mem, ctx->stream));
@@ -1729,6 +1832,8 @@ mm_status mm_setup_pointing(mm_ctx* ctx, int64_t n_samples, int32_t n_det, int32
     ctx->have_csdf = false;
     ctx->tmpl_on = false;
     ctx->tmpl_qu = 0;
+    if (mem == MM_HOST) TRY(windows(ctx->d_pix.as<int32_t>(), &bad));
+    ctx->win.swap(win);
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->have_pointing = true;
     return MM_OK;
@@ -1926,7 +2031,7 @@ mm_status mm_apply_A(mm_ctx* ctx, const double* x, double* y, int32_t nrhs, int 
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     ctx->last_apply_ms = ms;
-    return MM_OK;
+    return filter_fault_check(ctx);
 }
 
 mm_status mm_apply_precond(mm_ctx* ctx, mm_precond which, const double* x, double* y, int32_t nrhs, int mem) {

@@ -76,6 +76,8 @@ struct Seg {
     int32_t n_out;
     int32_t band;
     int32_t shift;   // left halo in the transform buffer: lambda, or 0 for a whole block
+    int32_t win0;    // the block's pixels lie in [win0, win0 + nwin); nwin 0: it sees none
+    int32_t nwin;
 };
 
 // Mixed-radix FFT plan: L = product of radix[p]; pass p works on spans of
@@ -120,6 +122,10 @@ struct FilterArgs {
     const void* Hi;        // half, fused last pass: [n_bands][items][R] coefficients (alpha_k, alpha_{L-k}, beta_k)
     const void* twp;       // half: per-pass twiddles W_S^(j q), pass by pass, [q - 1][j] within a pass; may be null
     int half;              // 1: one whole block per CTA as L = N/2 complex points
+    int three;             // half, float32: three passes of radix r0, r1, 9 (half3_shape)
+    int even;              // every segment starts at an even sample
+    int* fault;            // set to 1 by a bounded wait that gave up
+    int ahead;             // CTAs on the device at a time: the pointing of the CTA so many later goes to L2
     const void* band;      // direct: [n_bands][lambda+1]
     int L, logL, lam, V;
     FftPasses fp;
@@ -153,6 +159,12 @@ void launch_filter_fft_f32(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_fft_f64(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_f32(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_f64(const FilterArgs& a, bool from_tod, cudaStream_t s);
+// Spare bytes behind pix and psi: the chunked copies of the three-pass filter read past the last sample.
+constexpr size_t POINTING_SPARE = 16384;
+// float32 whole blocks in three passes, for M of half3_shape: twp rows W_M^(j q) for q = 1 .. r0/4 - 1 and
+// r0/4, 2 r0/4, 3 r0/4 (9 r1 entries each), tw [9][r1] twiddles W_(9 r1)^(j q), Hi [n_bands][9][r0 r1 / 2 + 1]
+bool half3_shape(int M, int* r0, int* r1);
+void launch_filter_half3(const FilterArgs& a, bool from_tod, cudaStream_t s);
 // Double-float (float32 pairs) variants: maps V4<df> in, float64 accumulators out.
 void launch_filter_fft_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
@@ -163,6 +175,10 @@ size_t direct_smem_bytes(int V, int lam, bool f64);
 // H = DIF(h) for each band in float64 through global scratch; h [n_bands][L].
 void launch_fft_spectrum(const double* h, double* H_out, double2* work, const double2* tw,
                          int n_bands, const FftPasses& fp, cudaStream_t s);
+// Pixel window of every block: win[b] = (smallest pixel, largest pixel) over its unflagged samples (0, -1 if
+// there are none); *bad = 1 if a pixel lies outside [-1, n_pix).
+void launch_block_windows(const int32_t* pix, const int64_t* block_off, int n_blocks, int64_t max_block, int n_pix,
+                          int2* win, int* bad, cudaStream_t s);
 void launch_weights64(const float* psi, double2* cs, int64_t n, cudaStream_t s);
 
 // ---------------- vectors, preconditioners, reductions ----------------

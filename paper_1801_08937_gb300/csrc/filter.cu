@@ -47,7 +47,54 @@ __global__ void k_map_to_df(const V4<double>* src, V4<df>* dst, int64_t n) {
     }
 }
 
+// Smallest and largest pixel of each block, and the range check of the
+// pointing, in one pass over pix (DRAM-bound; slices of WIN_SLICE samples so a
+// few long blocks still fill the device).
+constexpr int WIN_SLICE = 16384;
+__global__ void k_window_init(int2* win, int n) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < n) win[b] = make_int2(0x7fffffff, -1);
+}
+__global__ void __launch_bounds__(256) k_block_windows(const int32_t* __restrict__ pix, const int64_t* __restrict__ off,
+                                                       int n_pix, int2* win, int* bad) {
+    const int b = blockIdx.x;
+    const int64_t o1 = off[b + 1];
+    const int64_t t0 = off[b] + (int64_t)blockIdx.y * WIN_SLICE, t1 = t0 + WIN_SLICE < o1 ? t0 + WIN_SLICE : o1;
+    if (t0 >= t1) return;
+    int lo = 0x7fffffff, hi = -1;
+    bool ok = true;
+    auto take = [&](int p) {
+        ok = ok && p >= -1 && p < n_pix;
+        if (p >= 0) lo = min(lo, p);
+        hi = max(hi, p);
+    };
+    int64_t t = t0 + threadIdx.x;
+    for (; t + 3 * 256 < t1; t += 4 * 256) {
+        int p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = __ldg(pix + t + j * 256);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) take(p[j]);
+    }
+    for (; t < t1; t += 256) take(__ldg(pix + t));
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0 && hi >= 0) {
+        atomicMin(&win[b].x, lo);
+        atomicMax(&win[b].y, hi);
+    }
+    if (!ok) *bad = 1;
+}
+
 // ---------------- launchers ----------------
+void launch_block_windows(const int32_t* pix, const int64_t* block_off, int n_blocks, int64_t max_block, int n_pix,
+                          int2* win, int* bad, cudaStream_t s) {
+    k_window_init<<<(n_blocks + 255) / 256, 256, 0, s>>>(win, n_blocks);
+    k_block_windows<<<dim3(n_blocks, (unsigned)((max_block + WIN_SLICE - 1) / WIN_SLICE)), 256, 0, s>>>(
+        pix, block_off, n_pix, win, bad);
+    count_launches(2);
+}
+
 size_t fft_smem_bytes(int L, bool f64) { return (size_t)(L + (L >> 4)) * (f64 ? 16 : 8); }
 size_t direct_smem_bytes(int V, int lam, bool f64) {
     return (size_t)(((lam + 2) & ~1) + V + 2 * lam) * (f64 ? 8 : 4);

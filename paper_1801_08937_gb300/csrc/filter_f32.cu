@@ -4,7 +4,9 @@
 namespace mm {
 
 void launch_filter_fft_f32(const FilterArgs& a, bool from_tod, cudaStream_t s) {
-    if (a.half) {
+    if (a.three) {
+        launch_filter_half3(a, from_tod, s);
+    } else if (a.half) {
         if (from_tod) launch_half_t<float, true>(a, s);
         else launch_half_t<float, false>(a, s);
     } else {

@@ -207,6 +207,52 @@ template <typename T> struct Dft<T, 16> {
     }
 };
 
+template <typename T> struct Dft<T, 32> {
+    static __device__ __forceinline__ void run(C2<T>* a) {
+        // cos, sin of 2 pi m / 32, m = 1, 2, 3 (the rest by symmetry)
+        constexpr T c1 = T(0.98078528040323044913), s1 = T(0.19509032201612826785);
+        constexpr T c2 = T(0.92387953251128675613), s2 = T(0.38268343236508977173);
+        constexpr T c3 = T(0.83146961230254523708), s3 = T(0.55557023301960222474);
+        constexpr T r2 = T(0.70710678118654752440);
+        // n = 4 n1 + n2, k = k1 + 8 k2
+        C2<T> b[4][8];
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < 8; ++n1) b[n2][n1] = a[4 * n1 + n2];
+            Dft<T, 8>::run(b[n2]);
+        }
+        // b[n2][k1] *= W32^(n2 k1)
+        b[1][1] = cmul(b[1][1], C2<T>{c1, -s1});
+        b[1][2] = cmul(b[1][2], C2<T>{c2, -s2});
+        b[1][3] = cmul(b[1][3], C2<T>{c3, -s3});
+        b[1][4] = cmul(b[1][4], C2<T>{r2, -r2});
+        b[1][5] = cmul(b[1][5], C2<T>{s3, -c3});
+        b[1][6] = cmul(b[1][6], C2<T>{s2, -c2});
+        b[1][7] = cmul(b[1][7], C2<T>{s1, -c1});
+        b[2][1] = cmul(b[2][1], C2<T>{c2, -s2});
+        b[2][2] = cmul(b[2][2], C2<T>{r2, -r2});
+        b[2][3] = cmul(b[2][3], C2<T>{s2, -c2});
+        b[2][4] = C2<T>{b[2][4].y, -b[2][4].x};
+        b[2][5] = cmul(b[2][5], C2<T>{-s2, -c2});
+        b[2][6] = cmul(b[2][6], C2<T>{-r2, -r2});
+        b[2][7] = cmul(b[2][7], C2<T>{-c2, -s2});
+        b[3][1] = cmul(b[3][1], C2<T>{c3, -s3});
+        b[3][2] = cmul(b[3][2], C2<T>{s2, -c2});
+        b[3][3] = cmul(b[3][3], C2<T>{-s1, -c1});
+        b[3][4] = cmul(b[3][4], C2<T>{-r2, -r2});
+        b[3][5] = cmul(b[3][5], C2<T>{-c1, -s1});
+        b[3][6] = cmul(b[3][6], C2<T>{-c2, s2});
+        b[3][7] = cmul(b[3][7], C2<T>{-s3, c3});
+#pragma unroll
+        for (int k1 = 0; k1 < 8; ++k1) {
+            dft4(b[0][k1], b[1][k1], b[2][k1], b[3][k1]);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) a[k1 + 8 * k2] = b[k2][k1];
+        }
+    }
+};
+
 // Powers w^q, q < R, of one twiddle, each a product of two earlier powers
 // (depth <= 4), from a single table load per butterfly.
 template <typename T, int R>
@@ -1189,11 +1235,87 @@ __device__ __forceinline__ void half_gather_t(const FilterArgs& a, const Seg& S,
     }
 }
 
+// pix and psi of eight consecutive samples as one 256-bit load each (32-byte aligned)
+__device__ __forceinline__ void ld8_pointing(const int32_t* pp, const float* pf, int (&p)[8], float (&f)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]), "=r"(p[4]), "=r"(p[5]), "=r"(p[6]), "=r"(p[7])
+                 : "l"(pp));
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7])
+                 : "l"(pf));
+}
+
+// P^T of a warp's 256 consecutive outputs, eight per lane in order (real
+// samples z).  A raster that stays on a pixel for several samples gives a lane
+// at most two pixels, that of its first and that of its last sample: two sums
+// per lane, the first handed to the lane before it when that lane ends on the
+// same pixel (a lane on one pixel keeps its sum), then one atomic per pixel
+// left.  A warp with a lane that sees a third pixel (short runs, single flagged
+// samples) flushes every run of a lane from registers instead.  Every sample is
+// counted once.
+__device__ __forceinline__ void warp_run8_scatter(const int (&p)[8], const float (&f)[8], const float (&z)[8],
+                                                  V4<float>* q) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;   // the last sample's pixel
+    float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f;   // the first sample's, if it is another one
+    bool third = false;
+#pragma unroll
+    for (int j = 1; j < 7; ++j) third = third || (p[j] != p[0] && p[j] != p[7]);
+    bool two = p[0] != p[7];
+    if (!__any_sync(FULL, third)) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float nc, ns;
+            neg_cs(f[j], nc, ns);
+            if (j == 7 || p[j] == p[7]) {
+                a0 += z[j];
+                a1 = fmaf(z[j], nc, a1);
+                a2 = fmaf(z[j], ns, a2);
+            } else {
+                b0 += z[j];
+                b1 = fmaf(z[j], nc, b1);
+                b2 = fmaf(z[j], ns, b2);
+            }
+        }
+    } else {
+        two = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j > 0 && p[j] != p[j - 1]) {
+                if (two && p[j - 1] >= 0) atomic_add3(q + p[j - 1], a0, -a1, -a2);
+                if (!two) {
+                    b0 = a0;
+                    b1 = a1;
+                    b2 = a2;
+                }
+                two = true;
+                a0 = a1 = a2 = 0.0f;
+            }
+            float nc, ns;
+            neg_cs(f[j], nc, ns);
+            a0 += z[j];
+            a1 = fmaf(z[j], nc, a1);
+            a2 = fmaf(z[j], ns, a2);
+        }
+    }
+    const int plast = __shfl_up_sync(FULL, p[7], 1);
+    const bool give = two && lane > 0 && p[0] == plast;
+    const float r0 = __shfl_down_sync(FULL, b0, 1);
+    const float r1 = __shfl_down_sync(FULL, b1, 1);
+    const float r2 = __shfl_down_sync(FULL, b2, 1);
+    if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
+        a0 += r0;
+        a1 += r1;
+        a2 += r2;
+    }
+    if (two && !give && p[0] >= 0) atomic_add3(q + p[0], b0, -b1, -b2);
+    if (p[7] >= 0) atomic_add3(q + p[7], a0, -a1, -a2);
+}
+
 // After the conjugate-domain inverse, point m holds conj(z'_m):
-// y'_{2m} = Re, y'_{2m+1} = -Im.  Each warp takes 128 consecutive samples per
-// step (four per lane); z_t (1, cos 2psi, sin 2psi) is summed over runs of
-// equal pixels (warp_run_scatter).  The next step's pointing is requested
-// before this step's run sums.
+// y'_{2m} = Re, y'_{2m+1} = -Im.  Each warp takes 256 consecutive samples per
+// step, eight per lane.
 template <int NT>
 __device__ __forceinline__ void half_scatter_f32(const FilterArgs& a, const Seg& S, const C2<float>* s, int M) {
     constexpr int NW = NT / 32;
@@ -1201,57 +1323,50 @@ __device__ __forceinline__ void half_scatter_f32(const FilterArgs& a, const Seg&
     V4<float>* q = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)S.rhs * a.n_pix;
     const int32_t* pix = a.pix + S.out0;
     const float* psi = a.psi + S.out0;
-    // steps whose 128 samples all lie inside an aligned block take unchecked vector loads
-    const int nfull = (S.out0 & 3) == 0 ? (S.n_out >> 7) : 0;
+    const int nfull = (S.out0 & 7) == 0 ? (S.n_out >> 8) : 0;
+    if (warp >= NW) return;   // whole warps only
     int st = warp;
     if (st < nfull) {
-        int4 pv;
-        float4 fv;
-        ld4_pointing(pix + 128 * st + 4 * lane, psi + 128 * st + 4 * lane, pv, fv);
+        int p[8];
+        float f[8];
+        ld8_pointing(pix + 8 * (32 * st + lane), psi + 8 * (32 * st + lane), p, f);
+#pragma unroll 1
         for (; st < nfull; st += NW) {
-            const int sn = min(st + NW, nfull - 1);
-            int4 pn;
-            float4 fn;
-            ld4_pointing(pix + 128 * sn + 4 * lane, psi + 128 * sn + 4 * lane, pn, fn);
-            const int m0 = 64 * st + 2 * lane;   // even: points m0, m0 + 1 share a padding group
-            const C2<float> e0 = s[sidx(m0)], e1 = s[sidx(m0) + 1];
-            const int p[4] = {pv.x, pv.y, pv.z, pv.w};
-            const float f[4] = {fv.x, fv.y, fv.z, fv.w};
-            const float z[4] = {e0.x, -e0.y, e1.x, -e1.y};
-            float v0[4], v1[4], v2[4];
+            // the next step's pointing is requested before this step's sums
+            int pn[8];
+            float fn[8];
+            const int un = 32 * min(st + NW, nfull - 1) + lane;
+            ld8_pointing(pix + 8 * un, psi + 8 * un, pn, fn);
+            const int b = sidx(4 * (32 * st + lane));   // points 4u .. 4u + 3 share a padding group
+            float z[8];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                float nc, ns;
-                neg_cs(f[j], nc, ns);
-                const float zz = p[j] >= 0 ? z[j] : 0.0f;
-                v0[j] = zz;
-                v1[j] = -zz * nc;
-                v2[j] = -zz * ns;
+                const C2<float> e = s[b + j];
+                z[2 * j] = e.x;
+                z[2 * j + 1] = -e.y;
             }
-            warp_run_scatter(p, v0, v1, v2, q);
-            pv = pn;
-            fv = fn;
+            warp_run8_scatter(p, f, z, q);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                p[j] = pn[j];
+                f[j] = fn[j];
+            }
         }
     }
-    for (; 128 * st < S.n_out; st += NW) {
-        const int i0 = 128 * st + 4 * lane;
-        const int m0 = min(i0 >> 1, M - 2);
-        const C2<float> e0 = s[sidx(m0)], e1 = s[sidx(m0) + 1];
-        const float z[4] = {e0.x, -e0.y, e1.x, -e1.y};
-        int p[4];
-        float v0[4], v1[4], v2[4];
+#pragma unroll 1
+    for (; 256 * st < S.n_out; st += NW) {
+        const int u = 32 * st + lane;
+        int p[8];
+        float f[8], z[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool ok = i0 + j < S.n_out;
-            p[j] = ok ? __ldg(pix + i0 + j) : -1;
-            float nc, ns;
-            neg_cs(ok ? __ldg(psi + i0 + j) : 0.0f, nc, ns);
-            const float zz = p[j] >= 0 ? z[j] : 0.0f;
-            v0[j] = zz;
-            v1[j] = -zz * nc;
-            v2[j] = -zz * ns;
+        for (int j = 0; j < 8; ++j) {
+            const bool ok = 8 * u + j < S.n_out;
+            p[j] = ok ? __ldg(pix + 8 * u + j) : -1;
+            f[j] = ok ? __ldg(psi + 8 * u + j) : 0.0f;
+            const C2<float> e = s[sidx(min(4 * u + j / 2, M - 1))];
+            z[j] = (j & 1) ? -e.y : e.x;
         }
-        warp_run_scatter(p, v0, v1, v2, q);
+        warp_run8_scatter(p, f, z, q);
     }
 }
 
@@ -1650,26 +1765,17 @@ inline void launch_half_nt(const FilterArgs& a, size_t sm, cudaStream_t s) {
     count_launches(1);
 }
 
-// Half-length real transforms (a.L = M complex points): float32 with two
-// CTAs per SM (512 threads for the large transforms, 256 otherwise);
-// double-float with 512 threads; float64 with 256.  Compile-time transforms
-// for the common block shapes.
+// Half-length real transforms (a.L = M complex points): float32 lengths that
+// filter_half3.cuh does not take, two CTAs per SM (512 threads for M = 8192,
+// 256 otherwise); double-float with 512 threads; float64 with 256.
+// Compile-time transforms for the common block shapes.
 template <typename T, bool FROM_TOD>
 inline void launch_half_t(const FilterArgs& a, cudaStream_t s) {
     if (a.n_work <= 0) return;
     const size_t sm = fft_smem_bytes(a.L, sizeof(T) == 8);
     if constexpr (std::is_same<T, float>::value) {
-        if constexpr (!FROM_TOD) {
-            switch (a.L) {
-                case 9216: return launch_half_nt<T, FROM_TOD, 512, 9216>(a, sm, s);
-                case 8192: return launch_half_nt<T, FROM_TOD, 512, 8192>(a, sm, s);
-                case 4608: return launch_half_nt<T, FROM_TOD, 256, 4608>(a, sm, s);
-                case 2304: return launch_half_nt<T, FROM_TOD, 256, 2304>(a, sm, s);
-                default: break;
-            }
-        } else {
-            if (a.L == 9216) return launch_half_nt<T, FROM_TOD, 512, 9216>(a, sm, s);
-        }
+        if constexpr (!FROM_TOD)
+            if (a.L == 8192) return launch_half_nt<T, FROM_TOD, 512, 8192>(a, sm, s);
         return launch_half_nt<T, FROM_TOD, 256, 0>(a, sm, s);
     } else if constexpr (std::is_same<T, df>::value) {
         if (a.L == 9216) return launch_half_nt<T, FROM_TOD, 512, 9216>(a, sm, s);

@@ -1,0 +1,75 @@
+"""The three-pass whole-block float32 filter at the edges of its tiles.
+
+Tolerance 1e-5 (relative 2-norm, per Stokes column too): the float32 operator's.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import synth
+from helpers import assert_close
+
+pytestmark = pytest.mark.gpu
+
+P = pytest.importorskip("paper_1801_08937_gb300")
+MM = P.mapmaker
+
+TOL32 = 1e-5
+LAM = 37
+
+
+def scan_with(lengths, pixels, nx, seed):
+    """A one-detector scan of blocks of the given lengths; pixels: "raster", "random" (a new pixel
+    every sample, anywhere on the map), "steps" (runs of 1 to 12 samples) or "still" (one pixel)."""
+    rng = np.random.default_rng(seed)
+    n = int(np.sum(lengths))
+    s = synth.make_scan(nx=nx, ny=nx, n_det=1, n_t=n, n_int=1, half_bw=LAM, f_knee=1.0, seed=seed, flag_frac=0.002)
+    if pixels == "random":
+        s.pix[:] = rng.integers(0, nx * nx, n)
+    elif pixels == "steps":
+        s.pix[:] = np.repeat(rng.integers(0, nx * nx, n), rng.integers(1, 13, n))[:n]
+    elif pixels == "still":
+        s.pix[:] = 5
+    s.pix[rng.random(n) < 0.002] = -1
+    s.block_off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    s.block_band = np.zeros(len(lengths), dtype=np.int32)
+    return s
+
+
+@pytest.mark.parametrize("L", [4608, 9216, 18432])
+@pytest.mark.parametrize("pixels,nx", [("raster", 16), ("random", 8), ("random", 80), ("steps", 16), ("still", 8)])
+def test_blocks_of_every_fill(L, pixels, nx):
+    """Blocks that fill the transform exactly, end inside a chunk, a row or a pair of samples, hold a
+    single sample, start at every offset from a 16-byte boundary; pixel windows that are staged and
+    that are not; lanes with one, two and more pixels."""
+    full = L - LAM
+    scan = scan_with([full, 1, 2, 3, full - 1, 255, 257, full // 2, L // 8, L // 8 + 1, 7], pixels, nx, L + nx)
+    c = MM.Context(0, None, MM.MM_FP32_MIXED)
+    c.set_option("filter", 2)
+    c.set_option("fft_len", L)
+    c.setup_scan(scan)
+    x = np.random.default_rng(L).standard_normal((2, scan.n_pix, 3))
+    y = c.apply_A(x)
+    assert c.get_option("plan_whole") == 2 and c.get_option("plan_fft_len") == L
+    prob = O.Problem.from_scan(scan)
+    for r in range(2):
+        assert_close(y[r], O.apply_A(prob, x[r]), TOL32)
+    c.close()
+
+
+def test_device_pixels_out_of_range_are_refused_and_leave_the_scan():
+    """A device array with a pixel outside [-1, n_pix) is refused before the context changes."""
+    import torch
+    scan = scan_with([1000, 3000], "raster", 8, 3)
+    c = MM.Context(0, None, MM.MM_FP64)
+    c.setup_scan(scan)
+    x = np.random.default_rng(3).standard_normal((1, scan.n_pix, 3))
+    y = c.apply_A(x)
+    for bad in (-2, scan.n_pix):
+        pix = torch.from_numpy(scan.pix).cuda()
+        pix[2345] = bad
+        with pytest.raises(MM.MapMakerError) as e:
+            c.setup_pointing(pix, torch.from_numpy(scan.psi).cuda(), scan.block_off, scan.block_band, scan.band, scan.n_pix)
+        assert e.value.status == MM.MM_ERR_ARG
+        assert_close(c.apply_A(x)[0], y[0], 1e-13)
+    c.close()
