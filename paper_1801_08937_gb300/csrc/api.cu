@@ -18,6 +18,7 @@
 
 #include "../../include/mapmaker.h"
 #include "common.cuh"
+#include "sincos2.cuh"
 
 namespace mm {
 
@@ -109,7 +110,10 @@ struct mm_ctx {
     std::vector<int32_t> block_band;
     std::vector<double> band;
     DevBuf d_pix, d_psi, d_cs64, d_block_off, d_block_band, d_band64, d_band32, d_banddf, d_csdf;
-    bool have_csdf = false;
+    bool have_csdf = false, have_cs64 = false;
+    DevBuf d_trig;           // nodes of sincos2.cuh
+    DevBuf w_tw64, w_spec;   // scratch of the plans' spectra
+    std::unique_ptr<Plan> spare;   // a plan of the previous pointing, kept for its buffers
     DevBuf w_off, w_win;     // scratch of the pointing check
     std::vector<int2> win;   // pixel window (smallest, largest) of each block
     int p64 = 1;   // precision of the float64-accurate products: 1 native, 2 double-float
@@ -479,44 +483,34 @@ std::vector<int> dif_frequency(const FftPasses& fp) {
     return k;
 }
 
-// Spectra of the bands for circular products of N points, in natural order of
-// the frequency and scaled by 1/N: [n_bands][N].
-mm_status band_spectra(mm_ctx* ctx, int N, std::vector<double>& H) {
+// Spectra of the bands for circular products of N points, scaled by 1/N, on the
+// device: H [n_bands][N], frequencies 0 .. N/2 in natural order.  Few or narrow
+// bands go by the cosine sum (1.6e-12 s a term on the device's float64 units),
+// which beats the one-SM transform (about 350 us per 152 bands at N = 18432)
+// below 1e8 terms.
+mm_status band_spectra_dev(mm_ctx* ctx, int N, DevBuf& H) {
     FftPasses fpN;
     if (!fft_passes(N, &fpN, 16)) return fail(ctx, MM_ERR_ARG, "no transform plan for the block spectrum");
-    std::vector<double> twN(2 * (size_t)N), h((size_t)ctx->n_bands * N, 0.0);
-    for (int e = 0; e < N; ++e) {
-        const double ang = -2.0 * M_PI * (double)e / (double)N;
-        twN[2 * e] = std::cos(ang);
-        twN[2 * e + 1] = std::sin(ang);
+    const size_t all = (size_t)ctx->n_bands * N;
+    CK(H.ensure(all * 8));
+    CK(ctx->w_tw64.ensure((size_t)N * 16));
+    launch_twiddles64(ctx->w_tw64.as<double2>(), N, ctx->stream);
+    if ((double)ctx->n_bands * ctx->lam * (N / 2) < 1e8) {
+        launch_band_cosines(ctx->d_band64.as<double>(), ctx->lam, ctx->n_bands, N, ctx->w_tw64.as<double2>(),
+                            H.as<double>(), ctx->stream);
+        CKL();
+        return MM_OK;
     }
-    for (int b = 0; b < ctx->n_bands; ++b) {
-        const double* c = &ctx->band[(size_t)b * (ctx->lam + 1)];
-        double* hb = &h[(size_t)b * N];
-        hb[0] = c[0];
-        for (int i = 1; i <= ctx->lam; ++i) {
-            hb[i] = c[i];
-            hb[N - i] = c[i];
-        }
-    }
-    std::vector<double> Hp(h.size());
-    DevBuf d_tw, d_h, d_H, d_work;
-    CK(d_tw.ensure(twN.size() * 8));
-    CK(d_h.ensure(h.size() * 8));
-    CK(d_H.ensure(h.size() * 8));
-    CK(d_work.ensure((size_t)ctx->n_bands * (N + (N >> 4)) * 16));
-    CK(cudaMemcpyAsync(d_tw.p, twN.data(), twN.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(d_h.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    launch_fft_spectrum(d_h.as<double>(), d_H.as<double>(), d_work.as<double2>(), d_tw.as<double2>(), ctx->n_bands, fpN,
+    DevBuf h, Hp, work;
+    CK(h.ensure(all * 8));
+    CK(Hp.ensure(all * 8));
+    CK(work.ensure((size_t)ctx->n_bands * (N + (N >> 4)) * 16));
+    launch_band_circle(ctx->d_band64.as<double>(), ctx->lam, ctx->n_bands, N, h.as<double>(), ctx->stream);
+    launch_fft_spectrum(h.as<double>(), Hp.as<double>(), work.as<double2>(), ctx->w_tw64.as<double2>(), ctx->n_bands, fpN,
                         ctx->stream);
+    launch_spectrum_order(Hp.as<double>(), H.as<double>(), ctx->n_bands, fpN, ctx->stream);
     CKL();
-    CK(cudaMemcpyAsync(Hp.data(), d_H.p, Hp.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    const std::vector<int> kN = dif_frequency(fpN);
-    H.resize(h.size());
-    for (int b = 0; b < ctx->n_bands; ++b)
-        for (int p = 0; p < N; ++p) H[(size_t)b * N + kN[p]] = Hp[(size_t)b * N + p];
-    return MM_OK;
+    return MM_OK;   // the buffers' release waits for the kernels
 }
 
 // Tables of the three-pass whole-block transform (filter_half3.cuh): twiddles
@@ -527,48 +521,13 @@ mm_status build_half3_tables(mm_ctx* ctx, FftTables& ft, int N) {
     int r0 = 0, r1 = 0;
     if (!half3_shape(M, &r0, &r1)) return fail(ctx, MM_ERR_STATE, "not a three-pass length");
     if (ft.L == M) return MM_OK;
-    std::vector<double> H;
-    TRY(band_spectra(ctx, N, H));
-    const int sr = 9 * r1, nb = r0 * r1, ni = nb / 2 + 1, ra = r0 / 4;
-    std::vector<float> t1, t2;
-    auto put = [](std::vector<float>& t, int64_t e, int64_t n) {
-        const double ang = -2.0 * M_PI * (double)(e % n) / (double)n;
-        t.push_back((float)std::cos(ang));
-        t.push_back((float)std::sin(ang));
-    };
-    for (int q = 1; q < ra + 3; ++q)
-        for (int j = 0; j < sr; ++j) put(t1, (int64_t)j * (q < ra ? q : (q - ra + 1) * ra), M);
-    for (int j = 0; j < 9; ++j)
-        for (int q = 0; q < r1; ++q) put(t2, (int64_t)j * q, sr);
-    std::vector<float> C((size_t)ctx->n_bands * 9 * ni * 4, 0.0f);
-    for (int t = 0; t < ni; ++t) {
-        int g = t / r1, r = t % r1;
-        if (t == nb / 2) {
-            g = 0;
-            r = r1 / 2;
-        } else if (g == 0) {
-            if (r < r1 / 2) g = r0 / 2;
-            else r -= r1 / 2;
-        }
-        for (int q = 0; q < 9; ++q) {
-            const int k = g + r0 * r + nb * q;
-            const double th = 2.0 * M_PI * (double)k / (double)N, sn = std::sin(th), cs = std::cos(th);
-            for (int b = 0; b < ctx->n_bands; ++b) {
-                const double h1 = 2.0 * H[(size_t)b * N + k], h2 = 2.0 * H[(size_t)b * N + M - k];
-                float* o = &C[(((size_t)b * 9 + q) * ni + t) * 4];
-                o[0] = (float)(0.5 * ((h1 + h2) + (h2 - h1) * sn));
-                o[1] = (float)(0.5 * ((h1 + h2) - (h2 - h1) * sn));
-                o[2] = (float)(-0.5 * (h2 - h1) * cs);
-            }
-        }
-    }
-    CK(ft.twp.ensure(t1.size() * 4));
-    CK(ft.tw.ensure(t2.size() * 4));
-    CK(ft.Hi.ensure(C.size() * 4));
-    CK(cudaMemcpyAsync(ft.twp.p, t1.data(), t1.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ft.tw.p, t2.data(), t2.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ft.Hi.p, C.data(), C.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    TRY(band_spectra_dev(ctx, N, ctx->w_spec));
+    CK(ft.twp.ensure((size_t)(r0 / 4 + 2) * 9 * r1 * sizeof(float2)));
+    CK(ft.tw.ensure((size_t)9 * r1 * sizeof(float2)));
+    CK(ft.Hi.ensure((size_t)ctx->n_bands * 9 * (r0 * r1 / 2 + 1) * sizeof(float4)));
+    launch_half3_tables(ctx->w_spec.as<double>(), ctx->n_bands, r0, r1, ft.twp.as<float2>(), ft.tw.as<float2>(),
+                        ft.Hi.as<float4>(), ctx->stream);
+    CKL();
     ft.L = M;
     return MM_OK;
 }
@@ -580,8 +539,10 @@ mm_status build_half3_tables(mm_ctx* ctx, FftTables& ft, int N) {
 mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, int N, int f64) {
     const int M = fpM.L;
     if (ft.L == M && ft.pairs.p) return MM_OK;
-    std::vector<double> Hp;
-    TRY(band_spectra(ctx, N, Hp));
+    TRY(band_spectra_dev(ctx, N, ctx->w_spec));
+    std::vector<double> Hp((size_t)ctx->n_bands * N);
+    CK(cudaMemcpyAsync(Hp.data(), ctx->w_spec.p, Hp.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     const std::vector<int> kM = dif_frequency(fpM);
     std::vector<int> posM(M);
     for (int p = 0; p < M; ++p) posM[kM[p]] = p;
@@ -749,6 +710,21 @@ mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, in
     return MM_OK;
 }
 
+TrigTable trig_of(const mm_ctx* ctx) {
+    return {ctx->d_trig.as<double2>(), reinterpret_cast<const float2*>(ctx->d_trig.as<double2>() + TRIG_N)};
+}
+
+// The stored float64 weights: part of the set-up of an MM_FP64 context; a mixed
+// one needs them for native float64 products only and stores none until then.
+mm_status ensure_weights64(mm_ctx* ctx) {
+    if (ctx->have_cs64) return MM_OK;
+    CK(ctx->d_cs64.ensure((size_t)ctx->n_samples * 16));
+    launch_weights64(ctx->d_psi.as<float>(), trig_of(ctx), ctx->d_cs64.as<double2>(), ctx->n_samples, ctx->stream);
+    CKL();
+    ctx->have_cs64 = true;
+    return MM_OK;
+}
+
 // Segment list: for every block, chunk and right-hand side, pairs of segments
 // that share a band (and halo).
 // starts (optional, per right-hand side): the first starts[r] samples of every
@@ -810,7 +786,11 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
         e.shift = segs.back().shift;
         segs.push_back(e);
     }
-    auto p = std::make_unique<Plan>();
+    auto p = std::move(ctx->spare);
+    if (!p) p = std::make_unique<Plan>();
+    p->ft.L = 0;   // its tables are another scan's
+    p->three = false;
+    p->even = true;
     p->variant = variant;
     p->L = L;
     p->logL = logL;
@@ -834,10 +814,11 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     else if (variant == 2) TRY(build_fft_tables(ctx, p->ft, fp, f64));
     if (f64 == 2 && !ctx->have_csdf) {
         CK(ctx->d_csdf.ensure((size_t)ctx->n_samples * 16));
-        launch_weights_df(ctx->d_cs64.as<double2>(), ctx->d_csdf.as<float4>(), ctx->n_samples, ctx->stream);
+        launch_weights_df(ctx->d_psi.as<float>(), trig_of(ctx), ctx->d_csdf.as<float4>(), ctx->n_samples, ctx->stream);
         CKL();
         ctx->have_csdf = true;
     }
+    if (f64 == 1) TRY(ensure_weights64(ctx));
     ctx->plans.push_back(std::move(p));
     *out = ctx->plans.back().get();
     return MM_OK;
@@ -1333,9 +1314,10 @@ mm_status bd_for_lens(mm_ctx* ctx) {
     CK(cudaMemcpyAsync(d_sorted.p, sorted.data(), R * sizeof(int64_t), cudaMemcpyHostToDevice, ctx->stream));
     CK(sums.ensure((size_t)R * ctx->n_pix * 7 * sizeof(double)));
     CK(cudaMemsetAsync(sums.p, 0, sums.bytes, ctx->stream));
-    launch_bd_accumulate(ctx->d_pix.as<int32_t>(), ctx->d_psi.as<float>(), ctx->d_block_off.as<int64_t>(),
-                         ctx->d_block_band.as<int32_t>(), ctx->d_band64.as<double>(), ctx->lam + 1, ctx->n_blocks, 0,
-                         ctx->n_t, d_sorted.as<int64_t>(), R, sums.as<double>(), ctx->n_pix, ctx->stream);
+    launch_bd_accumulate(ctx->d_pix.as<int32_t>(), ctx->d_psi.as<float>(),
+                         ctx->have_cs64 ? ctx->d_cs64.as<double2>() : nullptr, trig_of(ctx), ctx->d_block_off.as<int64_t>(),
+                         ctx->d_block_band.as<int32_t>(), ctx->d_band64.as<double>(), ctx->lam + 1, ctx->n_blocks,
+                         max_block_len(ctx), ctx->n_t, d_sorted.as<int64_t>(), R, sums.as<double>(), ctx->n_pix, ctx->stream);
     CK(bdsorted.ensure((size_t)R * ctx->n_pix * 6 * sizeof(double)));
     launch_bd_invert(sums.as<double>(), bdsorted.as<double>(), ctx->d_good.as<uint8_t>(), nullptr, ctx->n_pix, R, 0.0, 0,
                      ctx->stream, ctx->tmpl_on ? ctx->tmpl_qu : 0);
@@ -1792,6 +1774,7 @@ mm_status mm_setup_pointing(mm_ctx* ctx, int64_t n_samples, int32_t n_det, int32
     ctx->tpref_valid = false;
     ctx->z32_valid = false;
     ctx->have_lastb = false;
+    if (!ctx->plans.empty()) ctx->spare = std::move(ctx->plans.back());
     ctx->plans.clear();
     ctx->n_samples = n_samples;
     ctx->n_det = n_det;
@@ -1807,11 +1790,15 @@ mm_status mm_setup_pointing(mm_ctx* ctx, int64_t n_samples, int32_t n_det, int32
     ctx->grid_x = (int)std::min<int64_t>(gb, 304);
     CK(ctx->d_pix.ensure(n_samples * 4 + POINTING_SPARE));
     CK(ctx->d_psi.ensure(n_samples * 4 + POINTING_SPARE));
-    CK(ctx->d_cs64.ensure(n_samples * 16));
     CK(copy_in(ctx->d_pix.p, pix, n_samples * 4, mem, ctx->stream));
     CK(copy_in(ctx->d_psi.p, psi, n_samples * 4, mem, ctx->stream));
-    launch_weights64(ctx->d_psi.as<float>(), ctx->d_cs64.as<double2>(), n_samples, ctx->stream);
-    CKL();
+    if (!ctx->d_trig.p) {
+        static const std::vector<double> table = trig_table();
+        CK(ctx->d_trig.ensure(table.size() * 8));
+        CK(cudaMemcpyAsync(ctx->d_trig.p, table.data(), table.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    }
+    ctx->have_cs64 = false;
+    if (!is_f32(ctx)) TRY(ensure_weights64(ctx));
     CK(ctx->d_block_off.ensure((n_blocks + 1) * 8));
     CK(ctx->d_block_band.ensure(n_blocks * 4));
     CK(cudaMemcpyAsync(ctx->d_block_off.p, block_off, (n_blocks + 1) * 8, cudaMemcpyHostToDevice, ctx->stream));
@@ -1925,18 +1912,16 @@ mm_status mm_build_bd(mm_ctx* ctx, double rcond_min, int32_t* n_dropped_out) {
     CK(ctx->d_dropped.ensure(16));
     CK(cudaMemsetAsync(ctx->d_sums.p, 0, ctx->d_sums.bytes, ctx->stream));
     CK(cudaMemsetAsync(ctx->d_dropped.p, 0, 16, ctx->stream));
-    DevBuf d_len;
-    CK(d_len.ensure(8));
-    const int64_t full = ctx->n_t;
-    CK(cudaMemcpyAsync(d_len.p, &full, 8, cudaMemcpyHostToDevice, ctx->stream));
-    launch_bd_accumulate(ctx->d_pix.as<int32_t>(), ctx->d_psi.as<float>(), ctx->d_block_off.as<int64_t>(),
-                         ctx->d_block_band.as<int32_t>(), ctx->d_band64.as<double>(), ctx->lam + 1, ctx->n_blocks, 0,
-                         ctx->n_t, d_len.as<int64_t>(), 1, ctx->d_sums.as<double>(), n_pix, ctx->stream);
+    launch_bd_accumulate(ctx->d_pix.as<int32_t>(), ctx->d_psi.as<float>(),
+                         ctx->have_cs64 ? ctx->d_cs64.as<double2>() : nullptr, trig_of(ctx), ctx->d_block_off.as<int64_t>(),
+                         ctx->d_block_band.as<int32_t>(), ctx->d_band64.as<double>(), ctx->lam + 1, ctx->n_blocks,
+                         max_block_len(ctx), ctx->n_t, nullptr, 1, ctx->d_sums.as<double>(), n_pix, ctx->stream);
     CKL();
     TRY(reduce_sum(ctx, ctx->d_sums.p, (int64_t)n_pix * 7, 8));
     launch_bd_invert(ctx->d_sums.as<double>(), ctx->d_bd.as<double>(), ctx->d_good.as<uint8_t>(),
                      ctx->d_dropped.as<int>(), n_pix, 1, rcond_min, 1, ctx->stream, ctx->tmpl_on ? ctx->tmpl_qu : 0);
-    launch_flag_samples(ctx->d_pix.as<int32_t>(), ctx->d_good.as<uint8_t>(), ctx->n_samples, ctx->stream);
+    launch_flag_samples(ctx->d_pix.as<int32_t>(), ctx->d_good.as<uint8_t>(), ctx->d_dropped.as<int>(), ctx->n_samples,
+                        ctx->stream);
     CKL();
     int dropped = 0;
     CK(cudaMemcpyAsync(&dropped, ctx->d_dropped.p, 4, cudaMemcpyDeviceToHost, ctx->stream));

@@ -20,6 +20,8 @@
 
 namespace mm {
 
+struct TrigTable;   // sincos2.cuh
+
 // Largest coarse space (number of deflation vectors k) the M_2l kernels hold.
 constexpr int MM_K_MAX = 512;
 
@@ -161,6 +163,14 @@ void launch_filter_direct_f32(const FilterArgs& a, bool from_tod, cudaStream_t s
 void launch_filter_direct_f64(const FilterArgs& a, bool from_tod, cudaStream_t s);
 // Spare bytes behind pix and psi: the chunked copies of the three-pass filter read past the last sample.
 constexpr size_t POINTING_SPARE = 16384;
+// Spectra of the bands for circular products of N points by the cosine sum, on the device: H[b][k] / N for
+// k = 0 .. N/2 (the rest by symmetry).  tw: exp(-2 pi i e / N).
+void launch_band_cosines(const double* band, int lam, int n_bands, int N, const double2* tw, double* H, cudaStream_t s);
+void launch_twiddles64(double2* tw, int N, cudaStream_t s);
+// Digit-reversed spectra [n_bands][N] of launch_fft_spectrum to the layout of launch_band_cosines.
+void launch_spectrum_order(const double* Hp, double* H, int n_bands, const FftPasses& fp, cudaStream_t s);
+// Tables of the three-pass transform of M = r0 r1 9 points (see half3_shape) from those spectra, N = 2 M.
+void launch_half3_tables(const double* H, int n_bands, int r0, int r1, float2* t1, float2* t2, float4* Hi, cudaStream_t s);
 // float32 whole blocks in three passes, for M of half3_shape: twp rows W_M^(j q) for q = 1 .. r0/4 - 1 and
 // r0/4, 2 r0/4, 3 r0/4 (9 r1 entries each), tw [9][r1] twiddles W_(9 r1)^(j q), Hi [n_bands][9][r0 r1 / 2 + 1]
 bool half3_shape(int M, int* r0, int* r1);
@@ -168,18 +178,22 @@ void launch_filter_half3(const FilterArgs& a, bool from_tod, cudaStream_t s);
 // Double-float (float32 pairs) variants: maps V4<df> in, float64 accumulators out.
 void launch_filter_fft_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
-void launch_weights_df(const double2* cs, float4* out, int64_t n, cudaStream_t s);
+void launch_weights_df(const float* psi, const TrigTable& trig, float4* out, int64_t n, cudaStream_t s);
 void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t s);
 size_t fft_smem_bytes(int L, bool f64);
 size_t direct_smem_bytes(int V, int lam, bool f64);
 // H = DIF(h) for each band in float64 through global scratch; h [n_bands][L].
 void launch_fft_spectrum(const double* h, double* H_out, double2* work, const double2* tw,
                          int n_bands, const FftPasses& fp, cudaStream_t s);
+// h[b][i] of the bands (c_i at i and N - i) for launch_fft_spectrum
+void launch_band_circle(const double* band, int lam, int n_bands, int N, double* h, cudaStream_t s);
 // Pixel window of every block: win[b] = (smallest pixel, largest pixel) over its unflagged samples (0, -1 if
 // there are none); *bad = 1 if a pixel lies outside [-1, n_pix).
 void launch_block_windows(const int32_t* pix, const int64_t* block_off, int n_blocks, int64_t max_block, int n_pix,
                           int2* win, int* bad, cudaStream_t s);
-void launch_weights64(const float* psi, double2* cs, int64_t n, cudaStream_t s);
+void launch_weights64(const float* psi, const TrigTable& trig, double2* cs, int64_t n, cudaStream_t s);
+// Table of sincos2.cuh on the host: TRIG_N nodes (cos, sin), then TRIG_N float tails (as many doubles).
+std::vector<double> trig_table();
 
 // ---------------- vectors, preconditioners, reductions ----------------
 void launch_map_in(const double* src3, V4<double>* dst4, int64_t n_vec, cudaStream_t s);
@@ -189,14 +203,16 @@ void launch_from_f32(const V4<float>* src, V4<double>* dst, int64_t n, cudaStrea
 void launch_zero(void* p, size_t bytes, cudaStream_t s);
 
 // M_BD build: 6 sums + hits per pixel; then flagging and inversion.
-void launch_bd_accumulate(const int32_t* pix, const float* psi, const int64_t* block_off,
-                          const int32_t* block_band, const double* band, int lam1, int n_blocks,
-                          int64_t t_cap_per_det, int64_t n_t, const int64_t* rhs_len, int nrhs,
+// cs64: stored float64 weights, or null (the weights then come from the table).  sorted_len null: one
+// right-hand side over whole timelines.
+void launch_bd_accumulate(const int32_t* pix, const float* psi, const double2* cs64, const TrigTable& trig,
+                          const int64_t* block_off, const int32_t* block_band, const double* band, int lam1, int n_blocks,
+                          int64_t max_block, int64_t n_t, const int64_t* sorted_len, int nrhs,
                           double* sums /*[nrhs][n_pix][7]*/, int n_pix, cudaStream_t s);
 void launch_bd_invert(const double* sums, double* bd /*[nrhs][n_pix][6]*/, uint8_t* good,
                       int* n_dropped, int n_pix, int nrhs, double rcond_min, int set_good,
                       cudaStream_t s, int stokes = 0);
-void launch_flag_samples(int32_t* pix, const uint8_t* good, int64_t n, cudaStream_t s);
+void launch_flag_samples(int32_t* pix, const uint8_t* good, const int* dropped, int64_t n, cudaStream_t s);
 void launch_bd_apply(const double* bd, int bd_per_rhs, const V4<double>* x, V4<double>* y,
                      int n_pix, int nrhs, cudaStream_t s);
 

@@ -25,6 +25,16 @@ __device__ __forceinline__ float d2f_trunc(double x) {
     if (e <= 0 || e >= 255) return d2f_hw(x);
     return __uint_as_float((hi & 0x80000000u) | ((uint32_t)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
 }
+// The same rounded to nearest even.
+__device__ __forceinline__ float d2f_rn(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    const int e = (int)((hi >> 20) & 0x7FF) - 1023 + 127;
+    if (e <= 0 || e >= 254) return d2f_hw(x);
+    const uint32_t t = ((uint32_t)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1FFFFFFFu;   // a carry out of the significand moves to the exponent
+    return __uint_as_float((hi & 0x80000000u) | (t + (rest + (t & 1u) > 0x10000000u ? 1u : 0u)));
+}
 __device__ __forceinline__ double f2d_exact(float f) {
     const uint32_t u = __float_as_uint(f);
     if ((u & 0x7FFFFFFFu) == 0u) return __hiloint2double((int)u, 0);

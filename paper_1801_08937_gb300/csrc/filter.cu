@@ -1,5 +1,6 @@
 // Set-up kernels of the filter (spectra, pointing weights) and the launch counter.
 #include "filter_impl.cuh"
+#include "sincos2.cuh"
 
 namespace mm {
 
@@ -9,6 +10,73 @@ void count_launches(int n) { __atomic_fetch_add(&g_launches, (long long)n, __ATO
 std::mutex& smem_config_mutex() {
     static std::mutex m;
     return m;
+}
+
+// ---------------- trigonometric nodes ----------------
+// cos and sin of 2 pi k / TRIG_N to about 100 bits by Taylor series in
+// double-double arithmetic (Dekker; products through fma), for the first
+// octant; the rest by symmetry.
+namespace {
+struct dd {
+    double hi, lo;
+};
+dd dd_sum(double a, double b) {
+    const double s = a + b, bb = s - a;
+    return {s, (a - (s - bb)) + (b - bb)};
+}
+dd dd_add(dd a, dd b) {
+    const dd s = dd_sum(a.hi, b.hi);
+    return dd_sum(s.hi, s.lo + a.lo + b.lo);
+}
+dd dd_mul(dd a, dd b) {
+    const double p = a.hi * b.hi, e = std::fma(a.hi, b.hi, -p);
+    return dd_sum(p, e + (a.hi * b.lo + a.lo * b.hi));
+}
+dd dd_div(dd a, double d) {
+    const double q = a.hi / d;
+    const double r = std::fma(-q, d, a.hi) + a.lo;
+    return dd_sum(q, r / d);
+}
+}  // namespace
+
+std::vector<double> trig_table() {
+    const dd two_pi{6.283185307179586477, 2.4492935982947064e-16};
+    constexpr int N = TRIG_N, O = N / 8;
+    std::vector<dd> c(O + 1), s(O + 1);
+    for (int k = 0; k <= O; ++k) {
+        const dd x = dd_div(dd_mul(two_pi, dd{(double)k, 0.0}), (double)N), x2 = dd_mul(x, x);
+        dd tc{1.0, 0.0}, ts = x;
+        c[k] = tc;
+        s[k] = ts;
+        for (int i = 1; i <= 14; ++i) {
+            tc = dd_div(dd_mul(tc, x2), -(2.0 * i - 1.0) * (2.0 * i));
+            ts = dd_div(dd_mul(ts, x2), -(2.0 * i) * (2.0 * i + 1.0));
+            c[k] = dd_add(c[k], tc);
+            s[k] = dd_add(s[k], ts);
+        }
+    }
+    std::vector<double> t(3 * (size_t)N);
+    float* tail = reinterpret_cast<float*>(&t[2 * (size_t)N]);
+    for (int k = 0; k < N; ++k) {
+        const int quad = k / (N / 4), q = k % (N / 4);
+        const dd cq = q <= O ? c[q] : s[N / 4 - q], sq = q <= O ? s[q] : c[N / 4 - q];
+        dd cv = cq, sv = sq;
+        if (quad == 1) {
+            cv = {-sq.hi, -sq.lo};
+            sv = cq;
+        } else if (quad == 2) {
+            cv = {-cq.hi, -cq.lo};
+            sv = {-sq.hi, -sq.lo};
+        } else if (quad == 3) {
+            cv = sq;
+            sv = {-cq.hi, -cq.lo};
+        }
+        t[2 * k] = cv.hi;
+        t[2 * k + 1] = sv.hi;
+        tail[2 * k] = (float)cv.lo;
+        tail[2 * k + 1] = (float)sv.lo;
+    }
+    return t;
 }
 
 // ---------------- setup kernels ----------------
@@ -24,26 +92,117 @@ __global__ void k_fft_spectrum(const double* h, double* H, C2<double>* work, con
     for (int i = threadIdx.x; i < L; i += blockDim.x) H[(int64_t)blockIdx.x * L + i] = s[sidx(i)].x * inv;
 }
 
-__global__ void k_weights64(const float* psi, double2* cs, int64_t n) {
+__global__ void k_weights64(const float* psi, const TrigTable trig, double2* cs, int64_t n) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         double sn, c;
-        sincos(2.0 * (double)psi[t], &sn, &c);
+        sincos_2psi(psi[t], trig, c, sn);
         cs[t] = make_double2(c, sn);
     }
 }
 
-// Double-float weights (cos 2psi, sin 2psi) from the float64 table.
-__global__ void k_weights_df(const double2* cs, float4* out, int64_t n) {
+// Double-float weights (cos 2psi, sin 2psi).
+__global__ void k_weights_df(const float* psi, const TrigTable trig, float4* out, int64_t n) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = cs[t];
-        const df c(v.x), s(v.y);
-        out[t] = make_float4(c.hi, c.lo, s.hi, s.lo);
+        double sn, cs;
+        sincos_2psi(psi[t], trig, cs, sn);
+        const float c = d2f_rn(cs), s = d2f_rn(sn);
+        out[t] = make_float4(c, d2f_rn(cs - f2d_exact(c)), s, d2f_rn(sn - f2d_exact(s)));
     }
 }
 __global__ void k_map_to_df(const V4<double>* src, V4<df>* dst, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const V4<double> v = src[i];
         dst[i] = V4<df>{df(v.x), df(v.y), df(v.z), df(0.0)};
+    }
+}
+
+__global__ void k_twiddles64(double2* tw, int N) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < N) {
+        double sn, cs;
+        sincospi(-2.0 * (double)e / (double)N, &sn, &cs);
+        tw[e] = make_double2(cs, sn);
+    }
+}
+__global__ void k_band_circle(const double* __restrict__ band, int lam, int N, double* h) {
+    const int b = blockIdx.y;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const int d = min(i, N - i);
+        h[(int64_t)b * N + i] = d <= lam ? band[(int64_t)b * (lam + 1) + d] : 0.0;
+    }
+}
+// H_k = (c_0 + 2 sum_i c_i cos(2 pi k i / N)) / N, a warp per frequency: the
+// band's transform in global memory takes 364 us on one SM for N = 18432
+// however few bands there are, the sums spread over the device.
+__global__ void __launch_bounds__(256) k_band_cosines(const double* __restrict__ band, int lam, int N,
+                                                      const double2* __restrict__ tw, double* H) {
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k > N / 2) return;
+    const double* c = band + (int64_t)blockIdx.y * (lam + 1);
+    double s0 = 0.0, s1 = 0.0;
+    const int step = (int)((int64_t)k * 64 % N);
+    int e0 = (int)((int64_t)k * (lane + 1) % N), e1 = (int)((int64_t)k * (lane + 33) % N);
+    for (int i = lane + 1; i <= lam; i += 64) {
+        s0 = fma(c[i], tw[e0].x, s0);
+        if (i + 32 <= lam) s1 = fma(c[i + 32], tw[e1].x, s1);
+        e0 += step;
+        e1 += step;
+        e0 -= e0 >= N ? N : 0;
+        e1 -= e1 >= N ? N : 0;
+    }
+    s0 += s1;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s0 += __shfl_down_sync(0xffffffffu, s0, d);
+    if (lane == 0) H[(int64_t)blockIdx.y * N + k] = (c[0] + 2.0 * s0) / (double)N;
+}
+__global__ void k_spectrum_order(const double* __restrict__ Hp, double* H, const FftPasses fp) {
+    const int64_t b = (int64_t)blockIdx.y * fp.L;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < fp.L; p += gridDim.x * blockDim.x) {
+        int rem = p, mult = 1, f = 0;   // the frequency at position p (mixed-radix digit reversal)
+        for (int i = 0; i < fp.npass; ++i) {
+            const int sr = fp.span[i] / fp.radix[i], d = rem / sr;
+            rem -= d * sr;
+            f += d * mult;
+            mult *= fp.radix[i];
+        }
+        H[b + f] = Hp[b + p];
+    }
+}
+// Twiddles (rows of filter_half3.cuh's Pass1Twiddle; [9][r1]) and, per band,
+// the coefficients of the paired spectrum step: item t pairs k = kc + r0 r1 q
+// with M - k, kc in the order of h3_spectrum's items.
+__global__ void k_half3_twiddles(int r0, int r1, float2* t1, float2* t2) {
+    const int sr = 9 * r1, M = r0 * sr, ra = r0 / 4, n1 = (ra + 2) * sr, i = blockIdx.x * blockDim.x + threadIdx.x;
+    double sn, cs;
+    if (i < n1) {
+        const int q = i / sr + 1, j = i % sr;
+        sincospi(-2.0 * (double)(j * (q < ra ? q : (q - ra + 1) * ra) % M) / (double)M, &sn, &cs);
+        t1[i] = make_float2((float)cs, (float)sn);
+    } else if (i < n1 + sr) {
+        const int j = (i - n1) / r1, q = (i - n1) % r1;
+        sincospi(-2.0 * (double)(j * q % sr) / (double)sr, &sn, &cs);
+        t2[i - n1] = make_float2((float)cs, (float)sn);
+    }
+}
+__global__ void k_half3_coef(const double* __restrict__ H, int n_bands, int r0, int r1, float4* Hi) {
+    const int nb = r0 * r1, ni = nb / 2 + 1, M = 9 * nb, N = 2 * M, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 9 * ni) return;
+    const int q = i / ni, t = i % ni;
+    int g = t / r1, r = t % r1;
+    if (t == nb / 2) {
+        g = 0;
+        r = r1 / 2;
+    } else if (g == 0) {
+        if (r < r1 / 2) g = r0 / 2;
+        else r -= r1 / 2;
+    }
+    const int k = g + r0 * r + nb * q;
+    double sn, cs;
+    sincospi(2.0 * (double)k / (double)N, &sn, &cs);
+    for (int b = blockIdx.y; b < n_bands; b += gridDim.y) {
+        const double h1 = 2.0 * H[(int64_t)b * N + k], h2 = 2.0 * H[(int64_t)b * N + M - k];   // H / M
+        Hi[(int64_t)b * 9 * ni + i] = make_float4((float)(0.5 * ((h1 + h2) + (h2 - h1) * sn)),
+                                                  (float)(0.5 * ((h1 + h2) - (h2 - h1) * sn)), (float)(-0.5 * (h2 - h1) * cs), 0.0f);
     }
 }
 
@@ -109,10 +268,33 @@ void launch_fft_spectrum(const double* h, double* H_out, double2* work, const do
     count_launches(1);
 }
 
-void launch_weights_df(const double2* cs, float4* out, int64_t n, cudaStream_t s) {
+void launch_twiddles64(double2* tw, int N, cudaStream_t s) {
+    k_twiddles64<<<(N + 255) / 256, 256, 0, s>>>(tw, N);
+    count_launches(1);
+}
+void launch_band_circle(const double* band, int lam, int n_bands, int N, double* h, cudaStream_t s) {
+    k_band_circle<<<dim3((N + 1023) / 1024, n_bands), 256, 0, s>>>(band, lam, N, h);
+    count_launches(1);
+}
+void launch_band_cosines(const double* band, int lam, int n_bands, int N, const double2* tw, double* H, cudaStream_t s) {
+    k_band_cosines<<<dim3((N / 2 + 8) / 8, n_bands), 256, 0, s>>>(band, lam, N, tw, H);
+    count_launches(1);
+}
+void launch_spectrum_order(const double* Hp, double* H, int n_bands, const FftPasses& fp, cudaStream_t s) {
+    k_spectrum_order<<<dim3((fp.L + 1023) / 1024, n_bands), 256, 0, s>>>(Hp, H, fp);
+    count_launches(1);
+}
+void launch_half3_tables(const double* H, int n_bands, int r0, int r1, float2* t1, float2* t2, float4* Hi, cudaStream_t s) {
+    const int n = (r0 / 4 + 3) * 9 * r1, ni = r0 * r1 / 2 + 1;
+    k_half3_twiddles<<<(n + 255) / 256, 256, 0, s>>>(r0, r1, t1, t2);
+    k_half3_coef<<<dim3((9 * ni + 255) / 256, n_bands < 64 ? n_bands : 64), 256, 0, s>>>(H, n_bands, r0, r1, Hi);
+    count_launches(2);
+}
+
+void launch_weights_df(const float* psi, const TrigTable& trig, float4* out, int64_t n, cudaStream_t s) {
     if (n <= 0) return;
     const int64_t blocks = (n + 255) / 256;
-    k_weights_df<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(cs, out, n);
+    k_weights_df<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(psi, trig, out, n);
     count_launches(1);
 }
 void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t s) {
@@ -121,10 +303,10 @@ void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t 
     k_map_to_df<<<(int)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(src, reinterpret_cast<V4<df>*>(dst), n);
     count_launches(1);
 }
-void launch_weights64(const float* psi, double2* cs, int64_t n, cudaStream_t s) {
+void launch_weights64(const float* psi, const TrigTable& trig, double2* cs, int64_t n, cudaStream_t s) {
     if (n <= 0) return;
     const int64_t blocks = (n + 255) / 256;
-    k_weights64<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(psi, cs, n);
+    k_weights64<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(psi, trig, cs, n);
     count_launches(1);
 }
 
