@@ -814,7 +814,8 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     else if (variant == 2) TRY(build_fft_tables(ctx, p->ft, fp, f64));
     if (f64 == 2 && !ctx->have_csdf) {
         CK(ctx->d_csdf.ensure((size_t)ctx->n_samples * 16));
-        launch_weights_df(ctx->d_psi.as<float>(), trig_of(ctx), ctx->d_csdf.as<float4>(), ctx->n_samples, ctx->stream);
+        launch_weights_df(ctx->d_psi.as<float>(), ctx->have_cs64 ? ctx->d_cs64.as<double2>() : nullptr, trig_of(ctx),
+                          ctx->d_csdf.as<float4>(), ctx->n_samples, ctx->stream);
         CKL();
         ctx->have_csdf = true;
     }
@@ -912,16 +913,26 @@ void tune_record(const TuneKey& k, const TuneVal& v) {
 
 // Time each candidate plan once (after one warm-up launch) on the current
 // pointing and keep the fastest.  Candidates: the six cheapest FFT plans of
-// the cost model, every three-pass whole-block plan that fits and, for narrow bands, the direct band at two tile sizes.
+// the cost model, the two shortest half-length and every three-pass plan of
+// whole blocks and, for narrow bands, the direct band at two tile sizes.
 mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& lens, TuneVal* best) {
     struct Opt { int variant, L, whole, V; };
     std::vector<Opt> opts;
     auto cands = fft_candidates(ctx, f64, 0, 0);
-    int r0 = 0, r1 = 0;
-    for (size_t i = 0; i < cands.size(); ++i)   // the three-pass whole blocks are cheaper than the model says
-        if (i < 6 || (f64 == 0 && cands[i].whole == 2 && half3_shape(cands[i].L / 2, &r0, &r1)))
+    // the cost model underrates whole blocks as half-length transforms (no halo, half the points): the two
+    // shortest of them are always timed
+    std::vector<int> half;
+    for (const FftCand& c : cands)
+        if (c.whole == 2) half.push_back(c.L);
+    std::sort(half.begin(), half.end());
+    for (size_t i = 0; i < cands.size(); ++i) {
+        const bool short_half = cands[i].whole == 2 && !half.empty() && cands[i].L <= half[std::min<size_t>(1, half.size() - 1)];
+        int r0 = 0, r1 = 0;
+        const bool three = f64 == 0 && cands[i].whole == 2 && half3_shape(cands[i].L / 2, &r0, &r1);
+        if (i < 6 || short_half || three)
             opts.push_back(
                 {2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
+    }
     if (ctx->lam <= 256)
         for (int tile : {1024, 2048})
             if (direct_smem_bytes(tile, ctx->lam, f64 != 0) <= 200 * 1024) opts.push_back({1, 0, 0, tile});

@@ -178,7 +178,8 @@ void launch_filter_half3(const FilterArgs& a, bool from_tod, cudaStream_t s);
 // Double-float (float32 pairs) variants: maps V4<df> in, float64 accumulators out.
 void launch_filter_fft_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_df(const FilterArgs& a, bool from_tod, cudaStream_t s);
-void launch_weights_df(const float* psi, const TrigTable& trig, float4* out, int64_t n, cudaStream_t s);
+void launch_weights_df(const float* psi, const double2* cs64, const TrigTable& trig, float4* out, int64_t n,
+                       cudaStream_t s);   // from the stored float64 weights where there are any
 void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t s);
 size_t fft_smem_bytes(int L, bool f64);
 size_t direct_smem_bytes(int V, int lam, bool f64);

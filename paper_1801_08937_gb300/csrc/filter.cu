@@ -101,10 +101,16 @@ __global__ void k_weights64(const float* psi, const TrigTable trig, double2* cs,
 }
 
 // Double-float weights (cos 2psi, sin 2psi).
-__global__ void k_weights_df(const float* psi, const TrigTable trig, float4* out, int64_t n) {
+__global__ void k_weights_df(const float* psi, const double2* cs64, const TrigTable trig, float4* out, int64_t n) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         double sn, cs;
-        sincos_2psi(psi[t], trig, cs, sn);
+        if (cs64) {
+            const double2 w = cs64[t];
+            cs = w.x;
+            sn = w.y;
+        } else {
+            sincos_2psi(psi[t], trig, cs, sn);
+        }
         const float c = d2f_rn(cs), s = d2f_rn(sn);
         out[t] = make_float4(c, d2f_rn(cs - f2d_exact(c)), s, d2f_rn(sn - f2d_exact(s)));
     }
@@ -291,10 +297,11 @@ void launch_half3_tables(const double* H, int n_bands, int r0, int r1, float2* t
     count_launches(2);
 }
 
-void launch_weights_df(const float* psi, const TrigTable& trig, float4* out, int64_t n, cudaStream_t s) {
+void launch_weights_df(const float* psi, const double2* cs64, const TrigTable& trig, float4* out, int64_t n,
+                       cudaStream_t s) {
     if (n <= 0) return;
     const int64_t blocks = (n + 255) / 256;
-    k_weights_df<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(psi, trig, out, n);
+    k_weights_df<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(psi, cs64, trig, out, n);
     count_launches(1);
 }
 void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t s) {

@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "df64.cuh"
+#include "fconv.cuh"
 
 namespace mm {
 
@@ -556,13 +557,22 @@ __device__ __forceinline__ T xmap_value(const FilterArgs& a, int64_t t, int rhs)
     return m.x + c * m.y + s * m.z;
 }
 
+// A timeline value in the arithmetic type.  The double-float one is split by
+// integer operations and one subtraction: the hardware conversions run on the
+// float64 pipe and are issued, predicated off, for float32 timelines too.
+template <typename T> __device__ __forceinline__ T from64(double d) { return T(d); }
+template <> __device__ __forceinline__ df from64<df>(double d) {
+    const float hi = d2f_rn(d);
+    return df(hi, d2f_rn(d - f2d_exact(hi)));
+}
+
 // y_t of right-hand side `rhs`: (P x)_t, or d_t when FROM_TOD (d_t - (P x)_t
 // when a residual map is given).
 template <typename T, bool FROM_TOD>
 __device__ __forceinline__ T sample_value(const FilterArgs& a, int64_t t, int rhs) {
     if (FROM_TOD) {
         T v = a.tod_is_float ? T(__ldg(reinterpret_cast<const float*>(a.src) + rhs * a.n_samples + t))
-                             : T(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + t));
+                             : from64<T>(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + t));
         if (sizeof(T) > 4 && a.xmap) v = v - xmap_value<T>(a, t, rhs);
         return v;
     } else {
@@ -657,10 +667,13 @@ __device__ __forceinline__ void atomic_add3(V4<double>* q, double a, double b, d
     atomicAdd(&q->y, b);
     atomicAdd(&q->z, c);
 }
+// float64 of a double-float sum with one operation on the float64 pipe (the
+// conversions go by integer operations)
+__device__ __forceinline__ double df_sum64(df v) { return f2d_exact(v.hi) + f2d_exact(v.lo); }
 __device__ __forceinline__ void atomic_add3(V4<double>* q, df a, df b, df c) {
-    atomicAdd(&q->x, (double)a);
-    atomicAdd(&q->y, (double)b);
-    atomicAdd(&q->z, (double)c);
+    atomicAdd(&q->x, df_sum64(a));
+    atomicAdd(&q->y, df_sum64(b));
+    atomicAdd(&q->z, df_sum64(c));
 }
 
 // Warp-cooperative P^T: every lane holds one sample (p < 0: nothing).
@@ -831,6 +844,86 @@ __device__ __forceinline__ bool seg_active(const FilterArgs& a, const Seg& S) {
     return S.n_out > 0 && (a.state == nullptr || a.state[S.rhs].active);
 }
 
+// a + b c with one rounding where the type has a fused operation
+__device__ __forceinline__ double madd(double b, double c, double a) { return fma(b, c, a); }
+__device__ __forceinline__ df madd(df b, df c, df a) { return a + b * c; }
+
+// Weights of samples t and t + 1 (t even) as one 256-bit load.
+__device__ __forceinline__ void weights2(const FilterArgs& a, int64_t t, double (&c)[2], double (&s)[2]) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(c[0]), "=d"(s[0]), "=d"(c[1]), "=d"(s[1]) : "l"(a.cs64 + t));
+}
+__device__ __forceinline__ void weights2(const FilterArgs& a, int64_t t, df (&c)[2], df (&s)[2]) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(c[0].hi), "=f"(c[0].lo), "=f"(s[0].hi), "=f"(s[0].lo), "=f"(c[1].hi), "=f"(c[1].lo), "=f"(s[1].hi),
+          "=f"(s[1].lo)
+        : "l"(a.csdf + t));
+}
+
+// P^T of a segment for float64 and double-float: eight consecutive outputs per
+// lane, z(i) the filtered sample i.  A lane sums its runs of equal pixels one
+// after the other (three operations per sample; a warp instruction of the
+// float64 pipe costs 64 cycles whatever lanes take part, so sums shuffled over
+// lanes and conversions at every run's end cost more than the transform
+// passes); its first run joins the lane before it when that lane ends on the
+// same pixel, then one set of atomics per run.  Measured: b of 3.4e7 samples in
+// double-float 1.03 -> 0.96 ms (with the timeline's conversion above; float64
+// pipe 35 -> 4 % busy), A x in float64 on ragged blocks 0.833 -> 0.736 ms.
+template <typename T, int NW, typename Z>
+__device__ __forceinline__ void scatter8_t(const FilterArgs& a, const Seg& S, bool act, Z z) {
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    V4<typename AccT<T>::type>* q = reinterpret_cast<V4<typename AccT<T>::type>*>(a.dst) + (int64_t)(act ? S.rhs : 0) * a.n_pix;
+    const int n = act ? S.n_out : 0;
+#pragma unroll 1
+    for (int base = warp * 256; base < n; base += NW * 256) {
+        const int i0 = base + 8 * lane;
+        const int64_t t0 = S.out0 + i0;
+        int p[8];
+        int (&pl)[4] = *reinterpret_cast<int (*)[4]>(p), (&ph)[4] = *reinterpret_cast<int (*)[4]>(p + 4);
+        load4_pix(a, t0, true, n - i0, pl);
+        load4_pix(a, t0 + 4, true, n - i0 - 4, ph);
+        T a0 = T(0), a1 = T(0), a2 = T(0), b0 = T(0), b1 = T(0), b2 = T(0);
+        bool multi = false;
+        const bool pairs = (t0 & 1) == 0 && i0 + 8 <= n;
+        T c[2], sn[2];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (pairs) {
+                if (j % 2 == 0) weights2(a, t0 + j, c, sn);
+            } else if (p[j] >= 0) {
+                weights(a, t0 + j, c[j & 1], sn[j & 1]);
+            }
+            if (j > 0 && p[j] != p[j - 1]) {
+                if (multi) {
+                    if (p[j - 1] >= 0) atomic_add3(q + p[j - 1], a0, a1, a2);
+                } else {
+                    b0 = a0;
+                    b1 = a1;
+                    b2 = a2;
+                    multi = true;
+                }
+                a0 = a1 = a2 = T(0);
+            }
+            if (p[j] >= 0) {
+                const T v = z(i0 + j);
+                a0 += v;
+                a1 = madd(v, c[j & 1], a1);
+                a2 = madd(v, sn[j & 1], a2);
+            }
+        }
+        const int plast = __shfl_up_sync(FULL, p[7], 1);
+        const bool give = multi && lane > 0 && p[0] == plast;
+        const T r0 = shfl_down_t(b0, 1), r1 = shfl_down_t(b1, 1), r2 = shfl_down_t(b2, 1);
+        if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
+            a0 += r0;
+            a1 += r1;
+            a2 += r2;
+        }
+        if (multi && !give && p[0] >= 0) atomic_add3(q + p[0], b0, b1, b2);
+        if (p[7] >= 0) atomic_add3(q + p[7], a0, a1, a2);
+    }
+}
+
 // ---------------- FFT overlap-save variant ----------------
 // Largest power-of-two radix of the compile-time transforms: 8 for
 // double-float (register pressure at 512 threads), 16 otherwise.  The host
@@ -867,55 +960,19 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT == 256) ? 3 : 1) k_f
         ct_dit<T, LCT, NT, MaxRadix<T>::value, make_ct_plan(LCT > 0 ? LCT : 64, MaxRadix<T>::value).np - 1>(s, tw);
     else fft_dit_conj<T>(s, tw, a.fp);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int vmax = max(actA ? A.n_out : 0, actB ? B.n_out : 0);
-    constexpr int SB = 2;
-    using Acc = typename AccT<T>::type;
-    V4<Acc>* qA = reinterpret_cast<V4<Acc>*>(a.dst) + (int64_t)(actA ? A.rhs : 0) * a.n_pix;
-    V4<Acc>* qB = reinterpret_cast<V4<Acc>*>(a.dst) + (int64_t)(actB ? B.rhs : 0) * a.n_pix;
     if constexpr (std::is_same<T, float>::value) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+        const int vmax = max(actA ? A.n_out : 0, actB ? B.n_out : 0);
+        V4<float>* qA = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)(actA ? A.rhs : 0) * a.n_pix;
+        V4<float>* qB = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)(actB ? B.rhs : 0) * a.n_pix;
         for (int base = warp * 128; base < vmax; base += nwarp * 128) {
             const int i0 = base + 4 * lane;
             scatter4_f32(a, A, actA, i0, s, lam, L, false, qA);
             scatter4_f32(a, B, actB, i0, s, lam, L, true, qB);
         }
-        return;
-    }
-    for (int base = warp * 32; base < vmax; base += nwarp * 32 * SB) {
-        int pa[SB], pb[SB];
-        float fa[SB], fb[SB];
-#pragma unroll
-        for (int g = 0; g < SB; ++g) {
-            const int i = base + g * nwarp * 32 + lane;
-            pa[g] = -1;
-            pb[g] = -1;
-            if (actA && i < A.n_out) {
-                pa[g] = __ldg(a.pix + A.out0 + i);
-                if (sizeof(T) == 4) fa[g] = __ldg(a.psi + A.out0 + i);
-            }
-            if (actB && i < B.n_out) {
-                pb[g] = __ldg(a.pix + B.out0 + i);
-                if (sizeof(T) == 4) fb[g] = __ldg(a.psi + B.out0 + i);
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < SB; ++g) {
-            const int i = base + g * nwarp * 32 + lane;
-            const C2<T> v = s[sidx(min(lam + i, L - 1))];
-            T c = T(0), sn = T(0), za = T(0), zb = T(0);
-            if (pa[g] >= 0) {
-                weights_from(a, A.out0 + i, fa[g], c, sn);
-                za = v.x;
-            }
-            scatter_warp<T>(pa[g], c, sn, za, qA);
-            c = T(0);
-            sn = T(0);
-            if (pb[g] >= 0) {
-                weights_from(a, B.out0 + i, fb[g], c, sn);
-                zb = -v.y;
-            }
-            scatter_warp<T>(pb[g], c, sn, zb, qB);
-        }
+    } else {
+        scatter8_t<T, NT / 32>(a, A, actA, [&](int i) { return s[sidx(lam + i)].x; });
+        scatter8_t<T, NT / 32>(a, B, actB, [&](int i) { return -s[sidx(lam + i)].y; });
     }
 }
 
@@ -1210,7 +1267,7 @@ __device__ __forceinline__ void half_gather_t(const FilterArgs& a, const Seg& S,
                 if (act && j < S.n_out - i0)
                     y[j] = a.tod_is_float
                                ? T(__ldg(reinterpret_cast<const float*>(a.src) + S.rhs * a.n_samples + t0 + j))
-                               : T(__ldg(reinterpret_cast<const double*>(a.src) + S.rhs * a.n_samples + t0 + j));
+                               : from64<T>(__ldg(reinterpret_cast<const double*>(a.src) + S.rhs * a.n_samples + t0 + j));
         }
         if (with_map) {
             int p[4];
@@ -1370,36 +1427,12 @@ __device__ __forceinline__ void half_scatter_f32(const FilterArgs& a, const Seg&
     }
 }
 
-// float64 / double-float scatter, four consecutive samples per lane as in
-// the float32 one (in-lane run sums, then the warp-segmented reduction).
 template <typename T, int NT>
-__device__ __forceinline__ void half_scatter_t(const FilterArgs& a, const Seg& S, const C2<T>* s, int M) {
-    constexpr int NW = NT / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    using Acc = typename AccT<T>::type;
-    V4<Acc>* q = reinterpret_cast<V4<Acc>*>(a.dst) + (int64_t)S.rhs * a.n_pix;
-    for (int base = warp * 128; base < S.n_out; base += NW * 128) {
-        const int i0 = base + 4 * lane;
-        const int64_t t0 = S.out0 + i0;
-        int p[4];
-        load4_pix(a, t0, i0 < S.n_out, S.n_out - i0, p);
-        const int m0 = min(i0 >> 1, M - 2);
-        const C2<T> e0 = s[sidx(m0)], e1 = s[sidx(m0 + 1)];
-        const T z[4] = {e0.x, -e0.y, e1.x, -e1.y};
-        T v0[4], v1[4], v2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            T zz = T(0), c = T(0), sn = T(0);
-            if (p[j] >= 0) {
-                zz = z[j];
-                weights(a, t0 + j, c, sn);
-            }
-            v0[j] = zz;
-            v1[j] = zz * c;
-            v2[j] = zz * sn;
-        }
-        scatter4_vals<T>(p, v0, v1, v2, q);
-    }
+__device__ __forceinline__ void half_scatter_t(const FilterArgs& a, const Seg& S, const C2<T>* s) {
+    scatter8_t<T, NT / 32>(a, S, true, [&](int i) {
+        const C2<T> e = s[sidx(i >> 1)];
+        return (i & 1) ? -e.y : e.x;
+    });
 }
 
 // Last forward pass, paired real-spectrum step and first inverse pass in
@@ -1469,7 +1502,7 @@ template <typename T> struct HalfMinBlocks { static constexpr int value = 1; };
 template <> struct HalfMinBlocks<float> { static constexpr int value = 2; };
 
 template <typename T, bool FROM_TOD, int NT, int MCT>
-__global__ void __launch_bounds__(NT, HalfMinBlocks<T>::value) k_filter_half(const FilterArgs a) {
+__global__ void __launch_bounds__(NT, HalfMinBlocks<T>::value * (sizeof(T) == 8 && std::is_same<T, df>::value ? 512 / NT : 1)) k_filter_half(const FilterArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     C2<T>* s = reinterpret_cast<C2<T>*>(smraw);
     const Seg S = a.segs[blockIdx.x];
@@ -1490,7 +1523,7 @@ __global__ void __launch_bounds__(NT, HalfMinBlocks<T>::value) k_filter_half(con
             __syncthreads();
             if constexpr (pl.np >= 2) ct_dit<T, MCT, NT, MaxRadix<T>::value, pl.np - 2>(s, tw, tt);
             if constexpr (std::is_same<T, float>::value) half_scatter_f32<NT>(a, S, s, M);
-            else half_scatter_t<T, NT>(a, S, s, M);
+            else half_scatter_t<T, NT>(a, S, s);
             return;
         }
     }
@@ -1527,7 +1560,7 @@ __global__ void __launch_bounds__(NT, HalfMinBlocks<T>::value) k_filter_half(con
         ct_dit<T, MCT, NT, MaxRadix<T>::value, make_ct_plan(MCT > 0 ? MCT : 64, MaxRadix<T>::value).np - 1>(s, tw);
     else fft_dit_conj<T>(s, tw, a.fp);
     if constexpr (std::is_same<T, float>::value) half_scatter_f32<NT>(a, S, s, M);
-    else half_scatter_t<T, NT>(a, S, s, M);
+    else half_scatter_t<T, NT>(a, S, s);
 }
 
 // ---------------- direct band variant, float32, four samples per thread ----------------
@@ -1778,11 +1811,20 @@ inline void launch_half_t(const FilterArgs& a, cudaStream_t s) {
             if (a.L == 8192) return launch_half_nt<T, FROM_TOD, 512, 8192>(a, sm, s);
         return launch_half_nt<T, FROM_TOD, 256, 0>(a, sm, s);
     } else if constexpr (std::is_same<T, df>::value) {
-        if (a.L == 9216) return launch_half_nt<T, FROM_TOD, 512, 9216>(a, sm, s);
-        if (a.L == 12288) return launch_half_nt<T, FROM_TOD, 512, 12288>(a, sm, s);
+        switch (a.L) {
+            case 12288: return launch_half_nt<T, FROM_TOD, 512, 12288>(a, sm, s);
+            case 9216: return launch_half_nt<T, FROM_TOD, 512, 9216>(a, sm, s);
+            case 4608: return launch_half_nt<T, FROM_TOD, 256, 4608>(a, sm, s);
+            case 2304: return launch_half_nt<T, FROM_TOD, 256, 2304>(a, sm, s);
+            default: break;
+        }
         return launch_half_nt<T, FROM_TOD, 512, 0>(a, sm, s);
     } else {
-        if (a.L == 9216) return launch_half_nt<T, FROM_TOD, 256, 9216>(a, sm, s);
+        switch (a.L) {
+            case 9216: return launch_half_nt<T, FROM_TOD, 256, 9216>(a, sm, s);
+            case 2304: return launch_half_nt<T, FROM_TOD, 256, 2304>(a, sm, s);
+            default: break;
+        }
         return launch_half_nt<T, FROM_TOD, 256, 0>(a, sm, s);
     }
 }

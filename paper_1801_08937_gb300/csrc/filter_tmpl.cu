@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(TMPL_NT) k_filter_tmpl(const FilterArgs a, con
                 for (int j = 0; j < 4; ++j)
                     if (i0 + j < nb)
                         v[j] = a.tod_is_float ? T(__ldg(reinterpret_cast<const float*>(a.src) + rhs * a.n_samples + t0 + j))
-                                              : T(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + t0 + j));
+                                              : from64<T>(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + t0 + j));
             }
             if (xm) {
                 V4<T> m[4];
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(TMPL_NT) k_filter_tmpl(const FilterArgs a, con
         T v = T(0);
         if (FROM_TOD)
             v = a.tod_is_float ? T(__ldg(reinterpret_cast<const float*>(a.src) + rhs * a.n_samples + ts))
-                               : T(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + ts));
+                               : from64<T>(__ldg(reinterpret_cast<const double*>(a.src) + rhs * a.n_samples + ts));
         if (xm) {
             const int p = __ldg(a.pix + ts);
             if (p >= 0) {

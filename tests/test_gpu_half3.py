@@ -73,3 +73,27 @@ def test_device_pixels_out_of_range_are_refused_and_leave_the_scan():
         assert e.value.status == MM.MM_ERR_ARG
         assert_close(c.apply_A(x)[0], y[0], 1e-13)
     c.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "df"])
+@pytest.mark.parametrize("L", [512, 4608, 9216])
+@pytest.mark.parametrize("pixels,nx", [("raster", 16), ("random", 8), ("steps", 16), ("still", 8)])
+def test_float64_scatter_of_every_fill(prec, L, pixels, nx):
+    """The eight-samples-a-lane scatter of the float64 and double-float filters, as overlap-save segments
+    (512) and whole blocks: 1e-11, those operators' tolerance."""
+    full = 4608 - LAM
+    scan = scan_with([full, 1, 2, 3, full - 1, 255, 257, 1151, 7, 9], pixels, nx, L + nx)
+    c = MM.Context(0, None, MM.MM_FP64 if prec == "f64" else MM.MM_FP32_MIXED)
+    c.set_option("filter", 2)
+    c.set_option("fft_len", L)
+    if prec == "df":
+        c.set_option("apply_precision", 2)
+    c.setup_scan(scan)
+    x = np.random.default_rng(L).standard_normal((2, scan.n_pix, 3))
+    y = c.apply_A(x)
+    prob = O.Problem.from_scan(scan)
+    for r in range(2):
+        assert_close(y[r], O.apply_A(prob, x[r]), 1e-11)
+    d = np.random.default_rng(1).standard_normal((1, scan.n_samples)).astype(c.tod_dtype)
+    assert_close(c.rhs(d)[0], O.rhs(prob, d[0].astype(np.float64)), 1e-11)
+    c.close()
