@@ -130,6 +130,7 @@ struct mm_ctx {
     std::vector<double> ritz;
 
     // workspace
+    DevBuf w_gram;                    // slices of Gram matrices
     DevBuf w_a, w_b, w_src, w_q, w_partial, w_counter, w_norms, d_lastb;
     bool have_lastb = false;
     int grid_x = 1;
@@ -290,7 +291,7 @@ int64_t max_block_len(const mm_ctx* c) {
 // first, then radix 16 while it divides, then one radix 2, 4 or 8 pass
 // (radix 8 plans end in 4, 4 instead of 8, 2, so the last pass -- fused with
 // the spectrum step -- is never a radix-2 one).  maxr: largest power-of-two
-// radix (8 for double-float plans, 16 otherwise), the same rule as the
+// radix (16 for float32 plans, 8 otherwise), the same rule as the
 // kernels' compile-time plans.
 bool fft_passes(int L, FftPasses* fp, int maxr = 16) {
     int rest = L, np = 0, span = L;
@@ -342,7 +343,7 @@ std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, i
             // a whole block as an L/2-point complex transform, one block per CTA
             FftPasses fh;
             if (L >= nb + lam && c->opt_half && L % 4 == 0 && L / 2 <= 65535 &&
-                fft_smem_bytes(L / 2, f64 != 0) <= smem_limit_bytes() && fft_passes(L / 2, &fh, f64 == 2 ? 8 : 16)) {
+                fft_smem_bytes(L / 2, f64 != 0) <= smem_limit_bytes() && fft_passes(L / 2, &fh, f64 ? 8 : 16)) {
                 const size_t smh = fft_smem_bytes(L / 2, f64 != 0);
                 const double fit = std::floor(228.0 * 1024 / (double)(smh + 1024));
                 const double per_smh = std::max(1.0, std::min(fit, f64 ? 1.0 : 2.0));
@@ -354,7 +355,7 @@ std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, i
             const size_t sm = fft_smem_bytes(L, f64 != 0);
             if (sm > smem_limit_bytes()) continue;
             FftPasses fp;
-            if (!fft_passes(L, &fp, f64 == 2 ? 8 : 16)) continue;
+            if (!fft_passes(L, &fp, f64 ? 8 : 16)) continue;
             double points = 0, gathered = 0, ctas = 0;
             int whole = 0;
             if (L >= nb + lam) {
@@ -735,7 +736,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     FftPasses fp{};
     int logL = 0;
     if (variant == 2) {
-        fft_passes(whole == 2 ? L / 2 : L, &fp, f64 == 2 ? 8 : 16);
+        fft_passes(whole == 2 ? L / 2 : L, &fp, f64 ? 8 : 16);
         logL = ilog2(whole == 2 ? L / 2 : L);
     }
     for (auto& p : ctx->plans)
@@ -980,14 +981,20 @@ mm_status get_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& l
     int variant = ctx->opt_filter;
     int L = 0, V = 0, whole = 0;
     if (variant == 0 && ctx->opt_fft_len == 0 && ctx->opt_fft_log2 == 0 && ctx->opt_autotune && !ctx->capturing) {
-        // tuned once per precision and geometry on a single right-hand side: the
-        // per-CTA work of a plan does not depend on how many right-hand sides share it
-        TuneKey key{f64, ctx->lam, ctx->n_blocks, 1, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix};
+        // tuned once per precision and geometry, on a single right-hand side where that fills the device (the
+        // per-CTA work of a plan does not depend on how many right-hand sides share it).  With fewer blocks than
+        // two per SM one right-hand side wants short segments on many SMs and a batch the least work per sample
+        // (64 blocks of 4096 samples, float64: 67 us alone in 2048-point segments, but 32 together 1.59 ms
+        // against 1.15 ms in whole blocks), so batches there are tuned on up to 16.
+        int tn = 1;
+        if (ctx->n_blocks < 304)
+            while (tn < 16 && 2 * tn <= nrhs) tn *= 2;
+        TuneKey key{f64, ctx->lam, ctx->n_blocks, tn, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix};
         TuneVal hit{};
         if (tune_lookup(key, ctx->opt_half != 0, &hit))
             return make_plan(ctx, f64, nrhs, lens, hit.variant, hit.L, hit.whole, hit.V, out, starts);
         TuneVal best{};
-        TRY(autotune_plan(ctx, f64, 1, {}, &best));
+        TRY(autotune_plan(ctx, f64, tn, {}, &best));
         tune_record(key, best);
         return make_plan(ctx, f64, nrhs, lens, best.variant, best.L, best.whole, best.V, out, starts);
     }
@@ -1098,7 +1105,7 @@ mm_status ensure_work(mm_ctx* ctx, int nrhs, int kmax) {
     CK(ctx->w_src.ensure(nv * sizeof(V4<double>)));
     CK(ctx->w_q.ensure(nv * sizeof(V4<double>)));
     const size_t per = (size_t)std::max({2, kmax, 1}) * std::max(1, nrhs);
-    CK(ctx->w_partial.ensure((size_t)ctx->grid_x * std::max<size_t>(per, 512) * sizeof(double)));
+    CK(ctx->w_partial.ensure((size_t)m2l_ztr_grid(ctx->n_pix) * std::max<size_t>(per, 512) * sizeof(double)));
     if (ctx->w_counter.bytes < (size_t)std::max(1, nrhs) * sizeof(unsigned)) {
         CK(ctx->w_counter.ensure((size_t)std::max(1, nrhs) * sizeof(unsigned) + 64));
         CK(cudaMemsetAsync(ctx->w_counter.p, 0, ctx->w_counter.bytes, ctx->stream));
@@ -1349,10 +1356,9 @@ mm_status orthonormalise(mm_ctx* ctx, DevBuf& X, int kin, int* kout) {
     for (int pass = 0; pass < 2; ++pass) {
         DevBuf dG;
         CK(dG.ensure((size_t)kcur * kcur * sizeof(double)));
-        TRY(ensure_work(ctx, 1, std::max(kcur, ctx->k)));
-        CK(ctx->w_partial.ensure((size_t)ctx->grid_x * std::max(kcur, 2) * sizeof(double) + 64));
-        launch_gram(X.as<double>(), kcur, X.as<double>(), kcur, n, n, dG.as<double>(), ctx->w_partial.as<double>(),
-                    ctx->w_counter.as<unsigned>(), ctx->grid_x, ctx->stream);
+        CK(ctx->w_gram.ensure(gram_scratch_doubles(kcur, kcur, ctx->n_pix) * 8));
+        launch_gram(X.as<V4<double>>(), kcur, X.as<V4<double>>(), kcur, ctx->n_pix, dG.as<double>(),
+                    ctx->w_gram.as<double>(), ctx->stream);
         CKL();
         std::vector<double> G((size_t)kcur * kcur);
         CK(cudaMemcpyAsync(G.data(), dG.p, G.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1410,9 +1416,9 @@ mm_status finish_coarse(mm_ctx* ctx) {
     TRY(apply_A_dev(ctx, op_prec(ctx), ctx->d_Z.as<V4<double>>(), ctx->d_AZ.as<V4<double>>(), k));
     DevBuf dG;
     CK(dG.ensure((size_t)k * k * 8));
-    CK(ctx->w_partial.ensure((size_t)ctx->grid_x * std::max(k, 2) * sizeof(double) + 64));
-    launch_gram(ctx->d_Z.as<double>(), k, ctx->d_AZ.as<double>(), k, n, n, dG.as<double>(), ctx->w_partial.as<double>(),
-                ctx->w_counter.as<unsigned>(), ctx->grid_x, ctx->stream);
+    CK(ctx->w_gram.ensure(gram_scratch_doubles(k, k, ctx->n_pix) * 8));
+    launch_gram(ctx->d_Z.as<V4<double>>(), k, ctx->d_AZ.as<V4<double>>(), k, ctx->n_pix, dG.as<double>(),
+                ctx->w_gram.as<double>(), ctx->stream);
     CKL();
     std::vector<double> G((size_t)k * k), E((size_t)k * k);
     CK(cudaMemcpyAsync(G.data(), dG.p, G.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1609,11 +1615,10 @@ mm_status coarse_for_lens(mm_ctx* ctx, const std::vector<uint8_t>& deflate) {
     TRY(coarse_products_for_lens(ctx, op_prec(ctx)));
     DevBuf dG;
     CK(dG.ensure((size_t)R * k * k * 8));
-    CK(ctx->w_partial.ensure((size_t)ctx->grid_x * std::max(k, 2) * sizeof(double) + 64));
+    CK(ctx->w_gram.ensure(gram_scratch_doubles(k, k, ctx->n_pix) * 8));
     for (int r = 0; r < R; ++r)
-        launch_gram(ctx->d_Z.as<double>(), k, ctx->d_AZr.as<double>() + (size_t)r * k * n, k, n, n,
-                    dG.as<double>() + (size_t)r * k * k, ctx->w_partial.as<double>(), ctx->w_counter.as<unsigned>(),
-                    ctx->grid_x, ctx->stream);
+        launch_gram(ctx->d_Z.as<V4<double>>(), k, reinterpret_cast<V4<double>*>(ctx->d_AZr.as<double>() + (size_t)r * k * n),
+                    k, ctx->n_pix, dG.as<double>() + (size_t)r * k * k, ctx->w_gram.as<double>(), ctx->stream);
     CKL();
     std::vector<double> G((size_t)R * k * k), Einv_all((size_t)R * k * k);
     CK(cudaMemcpyAsync(G.data(), dG.p, G.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
@@ -2004,26 +2009,25 @@ mm_status mm_apply_A(mm_ctx* ctx, const double* x, double* y, int32_t nrhs, int 
         CK(cudaMemcpyAsync(in3.p, x, nv * 24, cudaMemcpyHostToDevice, ctx->stream));
         xsrc = in3.as<double>();
     }
-    launch_map_in(xsrc, in4.as<V4<double>>(), nv, ctx->stream);
-    CKL();
     Plan* plan = nullptr;
     const int aprec = ctx->opt_apply_prec ? ctx->opt_apply_prec : op_prec(ctx);
     TRY(get_plan(ctx, aprec, nrhs, {}, &plan));
     CK(cudaEventRecord(ctx->ev0, ctx->stream));
-    TRY(apply_A_dev(ctx, aprec, in4.as<V4<double>>(), out4.as<V4<double>>(), nrhs, plan));
-    CK(cudaEventRecord(ctx->ev1, ctx->stream));
+    launch_apply_in(xsrc, aprec, in4.p, out4.p, nv, ctx->stream);
+    CKL();
+    TRY(run_filter(ctx, plan, false, in4.p, out4.p, nullptr, 0));
+    DevBuf o;
+    double* yd = y;
     if (mem == MM_HOST) {
-        DevBuf o;
         CK(o.ensure(nv * 24));
-        launch_map_out(out4.as<V4<double>>(), o.as<double>(), nv, ctx->stream);
-        CKL();
-        CK(cudaMemcpyAsync(y, o.p, nv * 24, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-    } else {
-        launch_map_out(out4.as<V4<double>>(), y, nv, ctx->stream);
-        CKL();
-        CK(cudaStreamSynchronize(ctx->stream));
+        yd = o.as<double>();
     }
+    if (aprec == 0) launch_map_out_f32(out4.as<V4<float>>(), yd, nv, ctx->stream);
+    else launch_map_out(out4.as<V4<double>>(), yd, nv, ctx->stream);
+    CKL();
+    CK(cudaEventRecord(ctx->ev1, ctx->stream));
+    if (mem == MM_HOST) CK(cudaMemcpyAsync(y, o.p, nv * 24, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     ctx->last_apply_ms = ms;
@@ -2059,7 +2063,7 @@ mm_status mm_apply_precond(mm_ctx* ctx, mm_precond which, const double* x, doubl
                         ctx->stream);
     } else {
         CK(u.ensure((size_t)nrhs * ctx->k * 8));
-        CK(ctx->w_partial.ensure((size_t)ctx->grid_x * nrhs * ctx->k * 8 + 64));
+        CK(ctx->w_partial.ensure((size_t)m2l_ztr_grid(ctx->n_pix) * nrhs * ctx->k * 8 + 64));
         PcgArgs a{};
         a.n_pix = ctx->n_pix;
         a.nrhs = nrhs;
@@ -2413,7 +2417,7 @@ mm_status mm_solve_begin(mm_ctx* ctx, const void* tod, int32_t nrhs, const int64
     const size_t v4 = nv * sizeof(V4<double>);
     const bool f32 = is_f32(ctx);
     TRY(ensure_work(ctx, nrhs, ctx->k));
-    CK(ctx->w_partial.ensure((size_t)ctx->grid_x * nrhs * std::max(2, ctx->k) * 8 + 64));
+    CK(ctx->w_partial.ensure((size_t)m2l_ztr_grid(ctx->n_pix) * nrhs * std::max(2, ctx->k) * 8 + 64));
     CK(ctx->s_b.ensure(v4));
     CK(ctx->s_x.ensure(v4));
     CK(ctx->s_r.ensure(v4));

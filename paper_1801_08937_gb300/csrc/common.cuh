@@ -199,6 +199,9 @@ std::vector<double> trig_table();
 // ---------------- vectors, preconditioners, reductions ----------------
 void launch_map_in(const double* src3, V4<double>* dst4, int64_t n_vec, cudaStream_t s);
 void launch_map_out(const V4<double>* src4, double* dst3, int64_t n_vec, cudaStream_t s);
+// mm_apply_A's input (and cleared accumulators) and float32 output; prec 0 float32, 1 float64, 2 double-float
+void launch_apply_in(const double* src3, int prec, void* dst, void* acc, int64_t n_vec, cudaStream_t s);
+void launch_map_out_f32(const V4<float>* src4, double* dst3, int64_t n_vec, cudaStream_t s);
 void launch_to_f32(const V4<double>* src, V4<float>* dst, int64_t n, cudaStream_t s);
 void launch_from_f32(const V4<float>* src, V4<double>* dst, int64_t n, cudaStream_t s);
 void launch_zero(void* p, size_t bytes, cudaStream_t s);
@@ -254,6 +257,7 @@ void launch_pcg_src(const PcgArgs& a, int first, cudaStream_t s);
 void launch_pcg_pq(const PcgArgs& a, cudaStream_t s);
 void launch_pcg_update(const PcgArgs& a, int two_level, cudaStream_t s);
 void launch_precond_bd_dot(const PcgArgs& a, int finalize_beta, cudaStream_t s);
+int m2l_ztr_grid(int n_pix);   // CTAs per right-hand side of the two M_2l kernels (partials per value)
 void launch_m2l_ztr(const PcgArgs& a, const V4<double>* v, cudaStream_t s);
 void launch_m2l_apply(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta,
                       cudaStream_t s);
@@ -276,9 +280,10 @@ void launch_sub_combo(const double* X, int64_t ldx, int m, const double* h, doub
 // Y[c][n] = sum_i X[i][n] C[i*kc + c] for c < kc
 void launch_combo(const double* X, int64_t ldx, int m, const double* C, int kc, double* Y,
                   int64_t ldy, int64_t n, cudaStream_t s);
-// G[j*mx + i] = sum_n X[i][n] Y[j][n]
-void launch_gram(const double* X, int mx, const double* Y, int my, int64_t ld, int64_t n, double* G,
-                 double* partial, unsigned* counter, int grid_x, cudaStream_t s);
+// G[j*mx + i] = sum over pixels of X_i . Y_j (three entries per pixel); scratch: gram_scratch_doubles
+size_t gram_scratch_doubles(int mx, int my, int64_t n_pix);
+void launch_gram(const V4<double>* X, int mx, const V4<double>* Y, int my, int64_t n_pix, double* G, double* scratch,
+                 cudaStream_t s);
 void launch_scale_host(double* v, int64_t n, double factor, cudaStream_t s);
 void launch_residual(const V4<double>* b, const V4<double>* q, V4<double>* r_out, double* norms, int n_pix,
                      int nrhs, double* partial, unsigned* counter, int grid_x, cudaStream_t s);

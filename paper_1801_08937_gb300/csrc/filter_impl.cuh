@@ -925,14 +925,15 @@ __device__ __forceinline__ void scatter8_t(const FilterArgs& a, const Seg& S, bo
 }
 
 // ---------------- FFT overlap-save variant ----------------
-// Largest power-of-two radix of the compile-time transforms: 8 for
-// double-float (register pressure at 512 threads), 16 otherwise.  The host
-// planner uses the same rule, so the spectra share the digit order.
-template <typename T> struct MaxRadix { static constexpr int value = 16; };
-template <> struct MaxRadix<df> { static constexpr int value = 8; };
+// Largest power-of-two radix of the compile-time transforms: 16 for float32, 8
+// for double-float and float64 (registers: a radix-16 butterfly pair of the
+// fused spectrum pass alone takes 128 of them; the float64 operations per point
+// are the same).  The host planner uses the same rule, so the spectra share
+// the digit order.
+template <typename T> struct MaxRadix { static constexpr int value = sizeof(T) == 4 ? 16 : 8; };
 
 template <typename T, bool FROM_TOD, int NT, int LCT>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT == 256) ? 3 : 1) k_filter_fft(const FilterArgs a) {
+__global__ void __launch_bounds__(NT, NT == 256 ? (sizeof(T) == 4 ? 3 : 2) : 1) k_filter_fft(const FilterArgs a) {
     static_assert(sizeof(C2<T>) == 2 * sizeof(T), "complex layout");
     extern __shared__ __align__(16) unsigned char smraw[];
     C2<T>* s = reinterpret_cast<C2<T>*>(smraw);
@@ -1498,11 +1499,8 @@ __device__ __forceinline__ void ct_fused_spectrum(C2<T>* s, const uint32_t* __re
     }
 }
 
-template <typename T> struct HalfMinBlocks { static constexpr int value = 1; };
-template <> struct HalfMinBlocks<float> { static constexpr int value = 2; };
-
 template <typename T, bool FROM_TOD, int NT, int MCT>
-__global__ void __launch_bounds__(NT, HalfMinBlocks<T>::value * (sizeof(T) == 8 && std::is_same<T, df>::value ? 512 / NT : 1)) k_filter_half(const FilterArgs a) {
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 512 / NT) k_filter_half(const FilterArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     C2<T>* s = reinterpret_cast<C2<T>*>(smraw);
     const Seg S = a.segs[blockIdx.x];
@@ -1782,6 +1780,8 @@ inline void launch_fft_t(const FilterArgs& a, cudaStream_t s) {
             case 9216: return launch_fft_nt<T, FROM_TOD, 256, 9216>(a, sm, s);
             case 8192: return launch_fft_nt<T, FROM_TOD, 256, 8192>(a, sm, s);
             case 4608: return launch_fft_nt<T, FROM_TOD, 256, 4608>(a, sm, s);
+            case 3072: return launch_fft_nt<T, FROM_TOD, 256, 3072>(a, sm, s);
+            case 2048: return launch_fft_nt<T, FROM_TOD, 256, 2048>(a, sm, s);
             default: break;
         }
     }

@@ -8,6 +8,7 @@
 // adds them in CTA order and applies the scalar update.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -128,9 +129,48 @@ __global__ void k_from_f32(const V4<float>* src, V4<double>* dst, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)VT + threadIdx.x; i < n; i += (int64_t)gridDim.x * VT)
         dst[i] = ld4(src + i);
 }
+// mm_apply_A's input in one pass: the caller's (I, Q, U) to the operator's
+// vectors (prec 0 float32, 1 float64, 2 double-float) and the accumulators to
+// zero; and its output.  Four launches of conversions and clears around the
+// filter became two (12 us -> 6 us of a product on a small map).
+template <int PREC>
+__global__ void k_apply_in(const double* __restrict__ src, void* dst, void* acc, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)VT + threadIdx.x; i < n; i += (int64_t)gridDim.x * VT) {
+        const double x = src[3 * i], y = src[3 * i + 1], z = src[3 * i + 2];
+        if constexpr (PREC == 0) {
+            reinterpret_cast<V4<float>*>(dst)[i] = V4<float>{(float)x, (float)y, (float)z, 0.0f};
+            reinterpret_cast<V4<float>*>(acc)[i] = V4<float>{0.0f, 0.0f, 0.0f, 0.0f};
+        } else {
+            if constexpr (PREC == 1) reinterpret_cast<V4<double>*>(dst)[i] = V4<double>{x, y, z, 0.0};
+            else reinterpret_cast<V4<df>*>(dst)[i] = V4<df>{df(x), df(y), df(z), df(0.0)};
+            reinterpret_cast<V4<double>*>(acc)[i] = V4<double>{0.0, 0.0, 0.0, 0.0};
+        }
+    }
+}
+__global__ void k_map_out_f32(const V4<float>* __restrict__ src, double* dst, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)VT + threadIdx.x; i < n; i += (int64_t)gridDim.x * VT) {
+        const V4<float> v = src[i];
+        dst[3 * i] = v.x;
+        dst[3 * i + 1] = v.y;
+        dst[3 * i + 2] = v.z;
+    }
+}
 static int grid_for(int64_t n) {
     const int64_t b = (n + VT - 1) / VT;
     return (int)(b < 152 * 8 ? (b > 0 ? b : 1) : 152 * 8);
+}
+void launch_apply_in(const double* src3, int prec, void* dst, void* acc, int64_t n, cudaStream_t s) {
+    if (n <= 0) return;
+    if (prec == 0) k_apply_in<0><<<grid_for(n), VT, 0, s>>>(src3, dst, acc, n);
+    else if (prec == 1) k_apply_in<1><<<grid_for(n), VT, 0, s>>>(src3, dst, acc, n);
+    else k_apply_in<2><<<grid_for(n), VT, 0, s>>>(src3, dst, acc, n);
+    count_launches(1);
+}
+void launch_map_out_f32(const V4<float>* src4, double* dst3, int64_t n, cudaStream_t s) {
+    if (n > 0) {
+        k_map_out_f32<<<grid_for(n), VT, 0, s>>>(src4, dst3, n);
+        count_launches(1);
+    }
 }
 void launch_map_in(const double* src3, V4<double>* dst4, int64_t n, cudaStream_t s) {
     if (n > 0) {
@@ -649,9 +689,32 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
     // this CTA's pixel range
     const int chunk = (a.n_pix + gridDim.x - 1) / gridDim.x;
     const int i0 = blockIdx.x * chunk, i1 = min(a.n_pix, i0 + chunk);
+    // float32: the residual of the chunk is converted once and shared by the warps (each coarse vector's warp
+    // converted it anew: 32 -> 14 us at 65536 pixels, k = 32)
+    constexpr int STAGE = 1024;
+    __shared__ float vx[3][STAGE];
+    const bool staged = a.Z32 && chunk <= STAGE;
+    if (staged) {
+        for (int i = i0 + threadIdx.x; i < i1; i += VT) {
+            const V4<double> x = v[off + i];
+            vx[0][i - i0] = d2f_trunc(x.x);
+            vx[1][i - i0] = d2f_trunc(x.y);
+            vx[2][i - i0] = d2f_trunc(x.z);
+        }
+        __syncthreads();
+    }
     for (int c = warp; c < k; c += nw) {
         double s = 0.0;
-        if (a.Z32) {
+        if (staged) {
+            const V4<float>* zc = a.Z32 + (int64_t)c * a.n_pix;
+            float sf = 0.0f;
+#pragma unroll 8
+            for (int i = i0 + lane; i < i1; i += 32) {
+                const V4<float> z = zc[i];
+                sf = fmaf(z.x, vx[0][i - i0], fmaf(z.y, vx[1][i - i0], fmaf(z.z, vx[2][i - i0], sf)));
+            }
+            s = f2d_exact(sf);
+        } else if (a.Z32) {
             // float32 products summed per lane in float32 (a few dozen terms), the lanes in float64
             const V4<float>* zc = a.Z32 + (int64_t)c * a.n_pix;
             float sf = 0.0f;
@@ -701,46 +764,68 @@ __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* ou
     __syncthreads();
     double acc[1] = {0.0};
     const V4<double>* AZ = a.AZ + (int64_t)rhs * a.az_stride;
-    PIX_LOOP(i) {
-        V4<double> y = v[off + i];
-        V4<double> zu{0, 0, 0, 0};
-        if (a.Z32) {
-            // the coarse sums AZ u and Z u in float32 (mixed precision), the rest in float64
-            float ax = 0.0f, ay = 0.0f, az = 0.0f, zx = 0.0f, zy = 0.0f, zz = 0.0f;
-#pragma unroll 8
-            for (int c = 0; c < a.k; ++c) {
-                const V4<float> azc = a.AZ32[(int64_t)c * a.n_pix + i];
-                const V4<float> zc = a.Z32[(int64_t)c * a.n_pix + i];
-                const float uc = uf[c];
-                ax = fmaf(azc.x, uc, ax);
-                ay = fmaf(azc.y, uc, ay);
-                az = fmaf(azc.z, uc, az);
-                zx = fmaf(zc.x, uc, zx);
-                zy = fmaf(zc.y, uc, zy);
-                zz = fmaf(zc.z, uc, zz);
+    // four lanes per pixel, each a quarter of the coarse vectors: a small map still fills the SMs' float64 pipes
+    // and the loads of a pixel's vectors are in flight together
+    const int g = threadIdx.x & 3;
+    for (int base = blockIdx.x * (VT / 4); base < a.n_pix; base += gridDim.x * (VT / 4)) {
+        const int i = base + (threadIdx.x >> 2);
+        const bool in = i < a.n_pix;
+        double yx = 0.0, yy = 0.0, yz = 0.0, zx = 0.0, zy = 0.0, zz = 0.0;
+        if (in) {
+            if (a.Z32) {
+                // the coarse sums AZ u and Z u in float32 (mixed precision), the rest in float64
+                float fx = 0.0f, fy = 0.0f, fz = 0.0f, hx = 0.0f, hy = 0.0f, hz = 0.0f;
+#pragma unroll 4
+                for (int c = g; c < a.k; c += 4) {
+                    const V4<float> azc = a.AZ32[(int64_t)c * a.n_pix + i];
+                    const V4<float> zc = a.Z32[(int64_t)c * a.n_pix + i];
+                    const float uc = uf[c];
+                    fx = fmaf(azc.x, uc, fx);
+                    fy = fmaf(azc.y, uc, fy);
+                    fz = fmaf(azc.z, uc, fz);
+                    hx = fmaf(zc.x, uc, hx);
+                    hy = fmaf(zc.y, uc, hy);
+                    hz = fmaf(zc.z, uc, hz);
+                }
+                yx = f2d_exact(fx);
+                yy = f2d_exact(fy);
+                yz = f2d_exact(fz);
+                zx = f2d_exact(hx);
+                zy = f2d_exact(hy);
+                zz = f2d_exact(hz);
+            } else {
+#pragma unroll 4
+                for (int c = g; c < a.k; c += 4) {
+                    const V4<double> azc = AZ[(int64_t)c * a.n_pix + i];
+                    const V4<double> zc = a.Z[(int64_t)c * a.n_pix + i];
+                    const double uc = u[c];
+                    yx = fma(azc.x, uc, yx);
+                    yy = fma(azc.y, uc, yy);
+                    yz = fma(azc.z, uc, yz);
+                    zx = fma(zc.x, uc, zx);
+                    zy = fma(zc.y, uc, zy);
+                    zz = fma(zc.z, uc, zz);
+                }
             }
-            y.x -= f2d_exact(ax);
-            y.y -= f2d_exact(ay);
-            y.z -= f2d_exact(az);
-            zu = V4<double>{f2d_exact(zx), f2d_exact(zy), f2d_exact(zz), 0.0};
-        } else
-        for (int c = 0; c < a.k; ++c) {
-            const V4<double> azc = AZ[(int64_t)c * a.n_pix + i];
-            const V4<double> zc = a.Z[(int64_t)c * a.n_pix + i];
-            const double uc = u[c];
-            y.x -= azc.x * uc;
-            y.y -= azc.y * uc;
-            y.z -= azc.z * uc;
-            zu.x += zc.x * uc;
-            zu.y += zc.y * uc;
-            zu.z += zc.z * uc;
         }
-        V4<double> o = bd_mul(bd_of(a, rhs, i), y);
-        o.x += zu.x;
-        o.y += zu.y;
-        o.z += zu.z;
-        out[off + i] = o;
-        acc[0] += dot3(v[off + i], o);
+#pragma unroll
+        for (int d = 1; d < 4; d <<= 1) {
+            yx += __shfl_xor_sync(0xffffffffu, yx, d);
+            yy += __shfl_xor_sync(0xffffffffu, yy, d);
+            yz += __shfl_xor_sync(0xffffffffu, yz, d);
+            zx += __shfl_xor_sync(0xffffffffu, zx, d);
+            zy += __shfl_xor_sync(0xffffffffu, zy, d);
+            zz += __shfl_xor_sync(0xffffffffu, zz, d);
+        }
+        if (in && g == 0) {
+            const V4<double> r = v[off + i];
+            V4<double> o = bd_mul(bd_of(a, rhs, i), V4<double>{r.x - yx, r.y - yy, r.z - yz, 0.0});
+            o.x += zx;
+            o.y += zy;
+            o.z += zz;
+            out[off + i] = o;
+            acc[0] += dot3(r, o);
+        }
     }
     if (finalize_beta < 0) return;
     block_partials<1>(acc, a.partial + ((int64_t)blockIdx.x * a.nrhs + rhs));
@@ -798,12 +883,15 @@ void launch_precond_bd_dot(const PcgArgs& a, int finalize_beta, cudaStream_t s) 
     k_bd_dot<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, finalize_beta);
     count_launches(1);
 }
+// CTAs of k_m2l_ztr: a small map is cut into 64-pixel chunks so that its k vectors spread over more SMs (the
+// partials then hold this many entries per value).
+int m2l_ztr_grid(int n_pix) { return std::min(304, (n_pix + 63) / 64); }
 void launch_m2l_ztr(const PcgArgs& a, const V4<double>* v, cudaStream_t s) {
-    k_m2l_ztr<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, v);
+    k_m2l_ztr<<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v);
     count_launches(1);
 }
 void launch_m2l_apply(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, cudaStream_t s) {
-    k_m2l_apply<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+    k_m2l_apply<<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
     count_launches(1);
 }
 
@@ -851,38 +939,114 @@ void launch_sub_combo(const double* X, int64_t ldx, int m, const double* h, doub
     count_launches(1);
 }
 
-// Y[c][i] = sum_r X[r][i] C[r*kc + c], eight outputs per pass.
+// Y[c][i] = sum_r X[r][i] C[r*kc + c]: eight outputs per thread, a group of
+// eight columns per grid row, so a small map still fills the device (85 -> 25 us
+// for 32 columns of a 1024-pixel map).
 __global__ void k_combo(const double* X, int64_t ldx, int m, const double* C, int kc, double* Y, int64_t ldy,
                         int64_t n) {
+    const int c0 = 8 * blockIdx.y;
     for (int64_t i = blockIdx.x * (int64_t)VT + threadIdx.x; i < n; i += (int64_t)gridDim.x * VT) {
-        for (int c0 = 0; c0 < kc; c0 += 8) {
-            double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            for (int r = 0; r < m; ++r) {
-                const double xv = X[(int64_t)r * ldx + i];
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c0 + c < kc) acc[c] += xv * C[(int64_t)r * kc + c0 + c];
-            }
+        double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 4
+        for (int r = 0; r < m; ++r) {
+            const double xv = X[(int64_t)r * ldx + i];
 #pragma unroll
             for (int c = 0; c < 8; ++c)
-                if (c0 + c < kc) Y[(int64_t)(c0 + c) * ldy + i] = acc[c];
+                if (c0 + c < kc) acc[c] += xv * C[(int64_t)r * kc + c0 + c];
         }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c0 + c < kc) Y[(int64_t)(c0 + c) * ldy + i] = acc[c];
     }
 }
 void launch_combo(const double* X, int64_t ldx, int m, const double* C, int kc, double* Y, int64_t ldy, int64_t n,
                   cudaStream_t s) {
     if (kc <= 0) return;
-    k_combo<<<grid_for(n), VT, 0, s>>>(X, ldx, m, C, kc, Y, ldy, n);
+    k_combo<<<dim3(grid_for(n), (kc + 7) / 8), VT, 0, s>>>(X, ldx, m, C, kc, Y, ldy, n);
     count_launches(1);
 }
 
-void launch_gram(const double* X, int mx, const double* Y, int my, int64_t ld, int64_t n, double* G, double* partial,
-                 unsigned* counter, int grid_x, cudaStream_t s) {
-    // column j of G^T: G[i][j] = X_i . Y_j, as multidots against each Y_j
-    for (int j = 0; j < my; ++j) {
-        k_multidot<<<grid_x, VT, 0, s>>>(X, ld, mx, Y + (int64_t)j * ld, n, G + (int64_t)j * mx, partial, counter);
-        count_launches(1);
+// Gram matrices.  A CTA takes a 32 x 32 tile of products over a slice of
+// pixels: both operands' slices pass through shared memory (the unused fourth
+// entry of a pixel is left out), a thread keeps 2 x 2 sums.  Slices are chosen
+// so that about two CTAs per SM run whatever the number of tiles, and the
+// slices' sums are added in order by a second kernel, so the result does not
+// depend on the schedule.  Bound by the float64 pipe (one product of 32 x 32 at
+// 1024 pixels: 7 us at its measured rate); one multidot per column took 38 us
+// each on four CTAs there, 1.2 ms a matrix.
+constexpr int GT = 32;        // tile edge
+constexpr int GP = 8;         // pixels staged at a time
+__global__ void __launch_bounds__(256) k_gram(const V4<double>* __restrict__ X, int mx, const V4<double>* __restrict__ Y,
+                                              int my, int64_t ld, int64_t n_pix, int64_t per, double* part) {
+    __shared__ double xs[3 * GP][GT + 2], ys[3 * GP][GT + 2];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    const int64_t p0 = blockIdx.z * per, p1 = p0 + per < n_pix ? p0 + per : n_pix;
+    double acc[2][2] = {{0, 0}, {0, 0}};
+    const int row = threadIdx.x >> 3, pp = threadIdx.x & 7;   // a thread stages pixel pp of row `row` of both tiles
+    for (int64_t p = p0; p < p1; p += GP) {
+        V4<double> x{0, 0, 0, 0}, y{0, 0, 0, 0};
+        if (p + pp < p1) {
+            if (i0 + row < mx) x = X[(int64_t)(i0 + row) * ld + p + pp];
+            if (j0 + row < my) y = Y[(int64_t)(j0 + row) * ld + p + pp];
+        }
+        __syncthreads();
+        xs[3 * pp][row] = x.x;
+        xs[3 * pp + 1][row] = x.y;
+        xs[3 * pp + 2][row] = x.z;
+        ys[3 * pp][row] = y.x;
+        ys[3 * pp + 1][row] = y.y;
+        ys[3 * pp + 2][row] = y.z;
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 3 * GP; ++e) {
+            const double a0 = xs[e][tx], a1 = xs[e][tx + 16], b0 = ys[e][ty], b1 = ys[e][ty + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
+        }
     }
+    double* o = part + (int64_t)blockIdx.z * mx * my;
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
+            if (i < mx && j < my) o[(int64_t)j * mx + i] = acc[u][v];
+        }
+}
+// Slices added in a fixed order: eight interleaved partial sums, then their sum.
+__global__ void __launch_bounds__(VT) k_gram_sum(const double* part, int slices, int64_t n, double* G) {
+    __shared__ double red[8][VT / 8];
+    const int o = threadIdx.x % (VT / 8), g = threadIdx.x / (VT / 8);
+    const int64_t i = (int64_t)blockIdx.x * (VT / 8) + o;
+    double s = 0.0;
+    if (i < n) {
+#pragma unroll 4
+        for (int z = g; z < slices; z += 8) s += part[z * n + i];
+    }
+    red[g][o] = s;
+    __syncthreads();
+    if (g == 0 && i < n) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) s += red[q][o];
+        G[i] = s;
+    }
+}
+static int gram_slices(int mx, int my, int64_t n_pix) {
+    const int64_t tiles = (int64_t)((mx + GT - 1) / GT) * ((my + GT - 1) / GT);
+    const int64_t want = (304 + tiles - 1) / tiles, most = (n_pix + GP - 1) / GP;
+    return (int)std::max<int64_t>(1, std::min(want, most));
+}
+size_t gram_scratch_doubles(int mx, int my, int64_t n_pix) { return (size_t)gram_slices(mx, my, n_pix) * mx * my; }
+void launch_gram(const V4<double>* X, int mx, const V4<double>* Y, int my, int64_t n_pix, double* G, double* scratch,
+                 cudaStream_t s) {
+    const int slices = gram_slices(mx, my, n_pix);
+    const int64_t per = ((n_pix + slices - 1) / slices + GP - 1) / GP * GP;
+    k_gram<<<dim3((mx + GT - 1) / GT, (my + GT - 1) / GT, slices), 256, 0, s>>>(X, mx, Y, my, n_pix, n_pix, per, scratch);
+    k_gram_sum<<<(unsigned)(((int64_t)mx * my + VT / 8 - 1) / (VT / 8)), VT, 0, s>>>(scratch, slices, (int64_t)mx * my, G);
+    count_launches(2);
 }
 
 __global__ void k_scale(double* v, int64_t n, double f) {
