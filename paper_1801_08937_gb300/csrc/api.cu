@@ -112,7 +112,7 @@ struct mm_ctx {
     DevBuf d_pix, d_psi, d_cs64, d_block_off, d_block_band, d_band64, d_band32, d_banddf, d_csdf;
     bool have_csdf = false, have_cs64 = false;
     DevBuf d_trig;           // nodes of sincos2.cuh
-    DevBuf w_tw64, w_spec;   // scratch of the plans' spectra
+    DevBuf w_tw64, w_spec, w_index;   // scratch of the plans' tables
     std::unique_ptr<Plan> spare;   // a plan of the previous pointing, kept for its buffers
     DevBuf w_off, w_win;     // scratch of the pointing check
     std::vector<int2> win;   // pixel window (smallest, largest) of each block
@@ -396,99 +396,10 @@ bool choose_fft(const mm_ctx* c, int f64, int forced_log2, int forced_len, int* 
     return true;
 }
 
-mm_status build_fft_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fp, int f64) {
-    const int L = fp.L;
-    if (ft.L == L) return MM_OK;
-    // twiddles exp(-2 pi i e / L) in float64 on the host
-    std::vector<double> tw64(2 * (size_t)L);
-    for (int e = 0; e < L; ++e) {
-        const double ang = -2.0 * M_PI * (double)e / (double)L;
-        tw64[2 * e] = std::cos(ang);
-        tw64[2 * e + 1] = std::sin(ang);
-    }
-    // circular placement of each band: h[i] = c_i, h[L - i] = c_i
-    std::vector<double> h((size_t)ctx->n_bands * L, 0.0);
-    for (int b = 0; b < ctx->n_bands; ++b) {
-        const double* c = &ctx->band[(size_t)b * (ctx->lam + 1)];
-        double* hb = &h[(size_t)b * L];
-        hb[0] = c[0];
-        for (int i = 1; i <= ctx->lam; ++i) {
-            hb[i] = c[i];
-            hb[L - i] = c[i];
-        }
-    }
-    DevBuf d_tw64, d_h, d_H64, d_work;
-    CK(d_tw64.ensure(tw64.size() * 8));
-    CK(d_h.ensure(h.size() * 8));
-    CK(d_H64.ensure(h.size() * 8));
-    CK(d_work.ensure((size_t)ctx->n_bands * (L + (L >> 4)) * 16));
-    CK(cudaMemcpyAsync(d_tw64.p, tw64.data(), tw64.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(d_h.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    launch_fft_spectrum(d_h.as<double>(), d_H64.as<double>(), d_work.as<double2>(), d_tw64.as<double2>(),
-                        ctx->n_bands, fp, ctx->stream);
-    CKL();
-    if (f64 == 1) {
-        CK(ft.tw.ensure(tw64.size() * 8));
-        CK(ft.H.ensure(h.size() * 8));
-        CK(cudaMemcpyAsync(ft.tw.p, d_tw64.p, tw64.size() * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        CK(cudaMemcpyAsync(ft.H.p, d_H64.p, h.size() * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-    } else if (f64 == 2) {
-        // double-float: each value as (hi, lo) float32 pair
-        std::vector<double> H64(h.size());
-        CK(cudaMemcpyAsync(H64.data(), d_H64.p, h.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-        std::vector<float> Hdf(2 * h.size()), twdf(2 * tw64.size());
-        auto split = [](double d, float* o) {
-            o[0] = (float)d;
-            o[1] = (float)(d - (double)o[0]);
-        };
-        for (size_t i = 0; i < h.size(); ++i) split(H64[i], &Hdf[2 * i]);
-        for (size_t i = 0; i < tw64.size(); ++i) split(tw64[i], &twdf[2 * i]);
-        CK(ft.tw.ensure(twdf.size() * 4));
-        CK(ft.H.ensure(Hdf.size() * 4));
-        CK(cudaMemcpyAsync(ft.tw.p, twdf.data(), twdf.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-        CK(cudaMemcpyAsync(ft.H.p, Hdf.data(), Hdf.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    } else {
-        std::vector<double> H64(h.size());
-        CK(cudaMemcpyAsync(H64.data(), d_H64.p, h.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-        std::vector<float> H32(h.size()), tw32(tw64.size());
-        for (size_t i = 0; i < h.size(); ++i) H32[i] = (float)H64[i];
-        for (size_t i = 0; i < tw64.size(); ++i) tw32[i] = (float)tw64[i];
-        CK(ft.tw.ensure(tw32.size() * 4));
-        CK(ft.H.ensure(H32.size() * 4));
-        CK(cudaMemcpyAsync(ft.tw.p, tw32.data(), tw32.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-        CK(cudaMemcpyAsync(ft.H.p, H32.data(), H32.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    }
-    CK(cudaStreamSynchronize(ctx->stream));
-    ft.L = L;
-    return MM_OK;
-}
-
-// Frequency index held at each position after the DIF passes of fp: with
-// position p = sum_i d_i (span_i / radix_i), the frequency is
-// d_0 + radix_0 (d_1 + radix_1 (d_2 + ...)) (mixed-radix digit reversal).
-std::vector<int> dif_frequency(const FftPasses& fp) {
-    std::vector<int> k(fp.L);
-    for (int p = 0; p < fp.L; ++p) {
-        int rem = p, mult = 1, f = 0;
-        for (int i = 0; i < fp.npass; ++i) {
-            const int sr = fp.span[i] / fp.radix[i];
-            const int d = rem / sr;
-            rem -= d * sr;
-            f += d * mult;
-            mult *= fp.radix[i];
-        }
-        k[p] = f;
-    }
-    return k;
-}
-
 // Spectra of the bands for circular products of N points, scaled by 1/N, on the
 // device: H [n_bands][N], frequencies 0 .. N/2 in natural order.  Few or narrow
-// bands go by the cosine sum (1.6e-12 s a term on the device's float64 units),
-// which beats the one-SM transform (about 350 us per 152 bands at N = 18432)
-// below 1e8 terms.
+// bands go by the cosine sum (about 2e-12 s a term), which beats the one-SM
+// transform (350 us per 152 bands at N = 18432) below 1.5e8 terms.
 mm_status band_spectra_dev(mm_ctx* ctx, int N, DevBuf& H) {
     FftPasses fpN;
     if (!fft_passes(N, &fpN, 16)) return fail(ctx, MM_ERR_ARG, "no transform plan for the block spectrum");
@@ -496,7 +407,7 @@ mm_status band_spectra_dev(mm_ctx* ctx, int N, DevBuf& H) {
     CK(H.ensure(all * 8));
     CK(ctx->w_tw64.ensure((size_t)N * 16));
     launch_twiddles64(ctx->w_tw64.as<double2>(), N, ctx->stream);
-    if ((double)ctx->n_bands * ctx->lam * (N / 2) < 1e8) {
+    if ((double)ctx->n_bands * ctx->lam * (N / 2) < 1.5e8) {
         launch_band_cosines(ctx->d_band64.as<double>(), ctx->lam, ctx->n_bands, N, ctx->w_tw64.as<double2>(),
                             H.as<double>(), ctx->stream);
         CKL();
@@ -533,180 +444,43 @@ mm_status build_half3_tables(mm_ctx* ctx, FftTables& ft, int N) {
     return MM_OK;
 }
 
+// Twiddles and spectra of a two-segment plan of fp.L points.
+mm_status build_fft_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fp, int f64) {
+    const int L = fp.L;
+    if (ft.L == L) return MM_OK;
+    TRY(band_spectra_dev(ctx, L, ctx->w_spec));
+    const size_t esz = f64 ? 8 : 4;
+    CK(ft.tw.ensure(2 * (size_t)L * esz));
+    CK(ft.H.ensure((size_t)ctx->n_bands * L * esz));
+    launch_plan_tables(ctx->w_spec.as<double>(), ctx->n_bands, fp, f64, ft.tw.p, ft.H.p, ctx->stream);
+    CKL();
+    ft.L = L;
+    return MM_OK;
+}
+
 // Tables of a whole-block plan run as an M = N/2 point complex transform:
 // twiddles of length M, the pair positions (k, M - k) and, per band, the
 // coefficients (alpha_k, alpha_{M-k}, beta_k) of the paired real-spectrum
 // filter, from the band's length-N spectrum, with 1/M folded in.
 mm_status build_half_tables(mm_ctx* ctx, FftTables& ft, const FftPasses& fpM, int N, int f64) {
-    const int M = fpM.L;
+    const int M = fpM.L, R = fpM.radix[fpM.npass - 1], np = M / 2 + 1, ni = M / R / 2 + 1;
     if (ft.L == M && ft.pairs.p) return MM_OK;
     TRY(band_spectra_dev(ctx, N, ctx->w_spec));
-    std::vector<double> Hp((size_t)ctx->n_bands * N);
-    CK(cudaMemcpyAsync(Hp.data(), ctx->w_spec.p, Hp.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    const std::vector<int> kM = dif_frequency(fpM);
-    std::vector<int> posM(M);
-    for (int p = 0; p < M; ++p) posM[kM[p]] = p;
-    const int np = M / 2 + 1;
-    // pairs in the order of their first position: neighbouring threads then
-    // touch neighbouring points (the frequency order would stride by M/r_0
-    // and put a warp's accesses on one bank)
-    std::vector<int> order(np);
-    for (int k = 0; k < np; ++k) order[k] = k;
-    std::sort(order.begin(), order.end(), [&](int x, int y) { return posM[x] < posM[y]; });
-    std::vector<uint32_t> pairs(np);
-    for (int e = 0; e < np; ++e) {
-        const int k = order[e];
-        pairs[e] = (uint32_t)posM[k] | ((uint32_t)posM[(M - k) % M] << 16);
-    }
-    // The last pass of radix R works on butterflies c of R consecutive
-    // positions; butterfly c holds the frequencies kc + (M/R) q and its partner
-    // c' (frequency digits M/R - kc) holds their mirror images M - k, at output
-    // R - 1 - q (kc = 0 and kc = M/(2R) pair with themselves).  One item per
-    // pair {c, c'}, kc = 0 .. M/(2R).
-    const int R = fpM.radix[fpM.npass - 1];
-    const int NB = M / R;
-    const bool fused = fpM.span[fpM.npass - 1] == R && NB % 2 == 0 && 16 % R == 0;
-    const int ni = fused ? NB / 2 + 1 : 0;
-    std::vector<uint32_t> items(std::max(ni, 1), 0u);
-    std::vector<int> item_kc;
+    const size_t esz = f64 ? 8 : 4;
+    const bool fused = half_fused(fpM);
+    CK(ft.tw.ensure(2 * (size_t)M * esz));
+    CK(ft.twp.ensure(2 * (size_t)plan_powers(fpM) * esz));
+    CK(ft.H.ensure((size_t)ctx->n_bands * np * 4 * esz));
+    CK(ft.pairs.ensure((size_t)np * 4));
     if (fused) {
-        std::vector<int> bfly(NB, -1);
-        for (int c = 0; c < NB; ++c) {
-            const int kc = kM[c * R];
-            for (int q = 0; q < R; ++q)
-                if (kM[c * R + q] != kc + NB * q) return fail(ctx, MM_ERR_STATE, "unexpected digit order of the last pass");
-            bfly[kc] = c;
-        }
-        // items in the order of their first butterfly's position: neighbouring
-        // threads then touch neighbouring points (2-way bank conflicts at most),
-        // where the frequency order would put a warp on one bank; bit 31 marks
-        // the kc = 0 item
-        std::vector<int> kcs(ni);
-        for (int i = 0; i < ni; ++i) kcs[i] = i;
-        std::sort(kcs.begin(), kcs.end(), [&](int x, int y) { return bfly[x] < bfly[y]; });
-        for (int i = 0; i < ni; ++i) {
-            const int kc = kcs[i];
-            items[i] = (uint32_t)bfly[kc] | ((uint32_t)bfly[(NB - kc) % NB] << 16) | (kc == 0 ? 0x80000000u : 0u);
-        }
-        item_kc.swap(kcs);
+        CK(ft.Hi.ensure((size_t)ctx->n_bands * ni * R * 4 * esz));
+        CK(ft.items.ensure((size_t)ni * 4));
     }
-    // coefficients in float64: H_k / M = 2 (H_k / N)
-    std::vector<double> coef((size_t)ctx->n_bands * np * 3), coefi((size_t)ctx->n_bands * std::max(ni, 1) * R * 3);
-    const double* Hn = nullptr;
-    auto pair_coef = [&](int k, double* o) {
-        const double h1 = 2.0 * Hn[k], h2 = 2.0 * Hn[M - k];
-        const double th = 2.0 * M_PI * (double)k / (double)N;
-        const double sn = std::sin(th), cs = std::cos(th);
-        o[0] = 0.5 * ((h1 + h2) + (h2 - h1) * sn);
-        o[1] = 0.5 * ((h1 + h2) - (h2 - h1) * sn);
-        o[2] = -0.5 * (h2 - h1) * cs;
-    };
-    for (int b = 0; b < ctx->n_bands; ++b) {
-        Hn = &Hp[(size_t)b * N];
-        for (int e = 0; e < np; ++e) pair_coef(order[e], &coef[((size_t)b * np + e) * 3]);
-        for (int i = 0; i < ni; ++i)
-            for (int q = 0; q < R; ++q) pair_coef(item_kc[i] + NB * q, &coefi[(((size_t)b * ni + i) * R + q) * 3]);
-    }
-    std::vector<double> twM(2 * (size_t)M);
-    for (int e = 0; e < M; ++e) {
-        const double ang = -2.0 * M_PI * (double)e / (double)M;
-        twM[2 * e] = std::cos(ang);
-        twM[2 * e + 1] = std::sin(ang);
-    }
-    // device layouts per element type: float64 (a, b, c, 0) as two double2;
-    // double-float (hi, lo) pairs as two float4; float32 (a, b, c, 0) as float4
-    auto upload = [&](DevBuf& dst, const std::vector<double>& src) -> cudaError_t {
-        const size_t n = src.size() / 3;
-        if (f64 == 1) {
-            std::vector<double> C(n * 4, 0.0);
-            for (size_t i = 0; i < n; ++i)
-                for (int j = 0; j < 3; ++j) C[4 * i + j] = src[3 * i + j];
-            cudaError_t e = dst.ensure(C.size() * 8);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(dst.p, C.data(), C.size() * 8, cudaMemcpyHostToDevice, ctx->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-            return e;
-        } else if (f64 == 2) {
-            std::vector<float> C(n * 8, 0.0f);
-            for (size_t i = 0; i < n; ++i)
-                for (int j = 0; j < 3; ++j) {
-                    const double d = src[3 * i + j];
-                    C[8 * i + 2 * j] = (float)d;
-                    C[8 * i + 2 * j + 1] = (float)(d - (double)(float)d);
-                }
-            cudaError_t e = dst.ensure(C.size() * 4);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(dst.p, C.data(), C.size() * 4, cudaMemcpyHostToDevice, ctx->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-            return e;
-        }
-        std::vector<float> C(n * 4, 0.0f);
-        for (size_t i = 0; i < n; ++i)
-            for (int j = 0; j < 3; ++j) C[4 * i + j] = (float)src[3 * i + j];
-        cudaError_t e = dst.ensure(C.size() * 4);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dst.p, C.data(), C.size() * 4, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        return e;
-    };
-    CK(upload(ft.H, coef));
-    if (fused) CK(upload(ft.Hi, coefi));
-    if (f64 == 1) {
-        CK(ft.tw.ensure(twM.size() * 8));
-        CK(cudaMemcpyAsync(ft.tw.p, twM.data(), twM.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    } else if (f64 == 2) {
-        std::vector<float> tw(2 * twM.size());
-        for (size_t i = 0; i < twM.size(); ++i) {
-            tw[2 * i] = (float)twM[i];
-            tw[2 * i + 1] = (float)(twM[i] - (double)(float)twM[i]);
-        }
-        CK(ft.tw.ensure(tw.size() * 4));
-        CK(cudaMemcpyAsync(ft.tw.p, tw.data(), tw.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    } else {
-        std::vector<float> tw(twM.size());
-        for (size_t i = 0; i < twM.size(); ++i) tw[i] = (float)twM[i];
-        CK(ft.tw.ensure(tw.size() * 4));
-        CK(cudaMemcpyAsync(ft.tw.p, tw.data(), tw.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    }
-    CK(cudaStreamSynchronize(ctx->stream));
-    // per-pass twiddle powers: pass p (radix R, span S, Sr = S/R > 1) holds
-    // W_S^(j q) at [(q - 1) Sr + j], passes concatenated in order
-    {
-        std::vector<double> t;
-        for (int i = 0; i < fpM.npass; ++i) {
-            const int Rp = fpM.radix[i], S = fpM.span[i], Sr = S / Rp;
-            for (int q = 1; q < Rp; ++q)
-                for (int j = 0; j < Sr; ++j) {
-                    const double ang = -2.0 * M_PI * (double)((int64_t)j * q % S) / (double)S;
-                    t.push_back(std::cos(ang));
-                    t.push_back(std::sin(ang));
-                }
-        }
-        if (t.empty()) t.assign(2, 0.0);
-        if (f64 == 1) {
-            CK(ft.twp.ensure(t.size() * 8));
-            CK(cudaMemcpyAsync(ft.twp.p, t.data(), t.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-        } else {
-            const bool dfp = f64 == 2;
-            std::vector<float> tf(t.size() * (dfp ? 2 : 1));
-            for (size_t i = 0; i < t.size(); ++i) {
-                if (dfp) {
-                    tf[2 * i] = (float)t[i];
-                    tf[2 * i + 1] = (float)(t[i] - (double)(float)t[i]);
-                } else {
-                    tf[i] = (float)t[i];
-                }
-            }
-            CK(ft.twp.ensure(tf.size() * 4));
-            CK(cudaMemcpyAsync(ft.twp.p, tf.data(), tf.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-        }
-        CK(cudaStreamSynchronize(ctx->stream));
-    }
-    if (fused) {
-        CK(ft.items.ensure(items.size() * 4));
-        CK(cudaMemcpyAsync(ft.items.p, items.data(), items.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    }
-    CK(ft.pairs.ensure(pairs.size() * 4));
-    CK(cudaMemcpyAsync(ft.pairs.p, pairs.data(), pairs.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    CK(ctx->w_index.ensure((size_t)(np + ni) * 4));
+    const HalfTables t{ft.tw.p, ft.twp.p, ft.H.p, ft.Hi.p, ft.pairs.as<uint32_t>(), ft.items.as<uint32_t>(),
+                       ctx->w_index.as<int>()};
+    launch_half_tables(ctx->w_spec.as<double>(), ctx->n_bands, fpM, f64, t, ctx->stream);
+    CKL();
     ft.L = M;
     return MM_OK;
 }

@@ -169,6 +169,17 @@ void launch_band_cosines(const double* band, int lam, int n_bands, int N, const 
 void launch_twiddles64(double2* tw, int N, cudaStream_t s);
 // Digit-reversed spectra [n_bands][N] of launch_fft_spectrum to the layout of launch_band_cosines.
 void launch_spectrum_order(const double* Hp, double* H, int n_bands, const FftPasses& fp, cudaStream_t s);
+// Tables of a plan from the bands' spectra S [n_bands][N] (kind 0 float32, 1 float64, 2 double-float): a
+// two-segment plan of N = fp.L points, or a half-length one of M = fp.L = N / 2.
+void launch_plan_tables(const double* S, int n_bands, const FftPasses& fp, int kind, void* tw, void* H, cudaStream_t s);
+struct HalfTables {
+    void *tw, *twp, *H, *Hi;
+    uint32_t *pairs, *items;
+    int* scratch;            // [M]: frequencies of the pairs and of the items
+};
+bool half_fused(const FftPasses& fp);          // the last pass takes the spectrum step (needs items and Hi)
+int64_t plan_powers(const FftPasses& fp);      // complex entries of twp
+void launch_half_tables(const double* S, int n_bands, const FftPasses& fp, int kind, const HalfTables& t, cudaStream_t s);
 // Tables of the three-pass transform of M = r0 r1 9 points (see half3_shape) from those spectra, N = 2 M.
 void launch_half3_tables(const double* H, int n_bands, int r0, int r1, float2* t1, float2* t2, float4* Hi, cudaStream_t s);
 // float32 whole blocks in three passes, for M of half3_shape: twp rows W_M^(j q) for q = 1 .. r0/4 - 1 and

@@ -137,42 +137,171 @@ __global__ void k_band_circle(const double* __restrict__ band, int lam, int N, d
         h[(int64_t)b * N + i] = d <= lam ? band[(int64_t)b * (lam + 1) + d] : 0.0;
     }
 }
-// H_k = (c_0 + 2 sum_i c_i cos(2 pi k i / N)) / N, a warp per frequency: the
-// band's transform in global memory takes 364 us on one SM for N = 18432
-// however few bands there are, the sums spread over the device.
-__global__ void __launch_bounds__(256) k_band_cosines(const double* __restrict__ band, int lam, int N,
+// H_k = (c_0 + 2 sum_i c_i cos(2 pi k i / N)) / N, a warp per frequency and
+// group of eight bands (they share the cosines): the band's transform in global
+// memory takes 364 us on one SM for N = 18432 however few bands there are, the
+// sums spread over the device.
+constexpr int COS_B = 8;
+__global__ void __launch_bounds__(256) k_band_cosines(const double* __restrict__ band, int lam, int n_bands, int N,
                                                       const double2* __restrict__ tw, double* H) {
-    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, b0 = blockIdx.y * COS_B;
     if (k > N / 2) return;
-    const double* c = band + (int64_t)blockIdx.y * (lam + 1);
-    double s0 = 0.0, s1 = 0.0;
-    const int step = (int)((int64_t)k * 64 % N);
-    int e0 = (int)((int64_t)k * (lane + 1) % N), e1 = (int)((int64_t)k * (lane + 33) % N);
-    for (int i = lane + 1; i <= lam; i += 64) {
-        s0 = fma(c[i], tw[e0].x, s0);
-        if (i + 32 <= lam) s1 = fma(c[i + 32], tw[e1].x, s1);
-        e0 += step;
-        e1 += step;
-        e0 -= e0 >= N ? N : 0;
-        e1 -= e1 >= N ? N : 0;
-    }
-    s0 += s1;
+    const double* c = band + (int64_t)b0 * (lam + 1);
+    const int nb = min(COS_B, n_bands - b0);
+    double s[COS_B] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int step = (int)((int64_t)k * 32 % N);
+    int e = (int)((int64_t)k * (lane + 1) % N);
+#pragma unroll 2
+    for (int i = lane + 1; i <= lam; i += 32) {
+        const double w = tw[e].x;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) s0 += __shfl_down_sync(0xffffffffu, s0, d);
-    if (lane == 0) H[(int64_t)blockIdx.y * N + k] = (c[0] + 2.0 * s0) / (double)N;
+        for (int b = 0; b < COS_B; ++b)
+            if (b < nb) s[b] = fma(__ldg(c + (int64_t)b * (lam + 1) + i), w, s[b]);
+        e += step;
+        e -= e >= N ? N : 0;
+    }
+#pragma unroll
+    for (int b = 0; b < COS_B; ++b) {
+        if (b >= nb) break;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) s[b] += __shfl_down_sync(0xffffffffu, s[b], d);
+        if (lane == 0) H[(int64_t)(b0 + b) * N + k] = (c[(int64_t)b * (lam + 1)] + 2.0 * s[b]) / (double)N;
+    }
+}
+// Frequency at position p after the DIF passes (mixed-radix digit reversal:
+// position sum_i d_i span_i / radix_i holds d_0 + radix_0 (d_1 + radix_1 ...)),
+// and the position of a frequency.
+__device__ __forceinline__ int dif_freq(const FftPasses& fp, int p) {
+    int mult = 1, f = 0;
+    for (int i = 0; i < fp.npass; ++i) {
+        const int sr = fp.span[i] / fp.radix[i], d = p / sr;
+        p -= d * sr;
+        f += d * mult;
+        mult *= fp.radix[i];
+    }
+    return f;
+}
+__device__ __forceinline__ int dif_pos(const FftPasses& fp, int f) {
+    int p = 0;
+    for (int i = 0; i < fp.npass; ++i) {
+        p += f % fp.radix[i] * (fp.span[i] / fp.radix[i]);
+        f /= fp.radix[i];
+    }
+    return p;
+}
+// Table values in the layouts of the kernels: KIND 0 float32, 1 float64, 2
+// double-float (hi, lo).
+template <int KIND> struct Tab;
+template <> struct Tab<0> {
+    static __device__ void put(void* t, int64_t i, double v) { reinterpret_cast<float*>(t)[i] = (float)v; }
+};
+template <> struct Tab<1> {
+    static __device__ void put(void* t, int64_t i, double v) { reinterpret_cast<double*>(t)[i] = v; }
+};
+template <> struct Tab<2> {
+    static __device__ void put(void* t, int64_t i, double v) {
+        const float hi = (float)v;
+        reinterpret_cast<float2*>(t)[i] = make_float2(hi, (float)(v - (double)hi));
+    }
+};
+// tw[e] = exp(-2 pi i e / L); then the passes' own powers W_S^(j q), pass by pass, [q - 1][j], into twp (may be null)
+template <int KIND>
+__global__ void k_plan_twiddles(const FftPasses fp, void* tw, void* twp, int64_t n_twp) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    double sn, cs;
+    if (i < fp.L) {
+        sincospi(-2.0 * (double)i / (double)fp.L, &sn, &cs);
+        Tab<KIND>::put(tw, 2 * i, cs);
+        Tab<KIND>::put(tw, 2 * i + 1, sn);
+    }
+    if (twp && i < n_twp) {
+        int64_t r = i;
+        int p = 0;
+        for (; p < fp.npass - 1; ++p) {
+            const int64_t n = (int64_t)(fp.radix[p] - 1) * (fp.span[p] / fp.radix[p]);
+            if (r < n) break;
+            r -= n;
+        }
+        const int sr = fp.span[p] / fp.radix[p], q = (int)(r / sr) + 1, j = (int)(r % sr);
+        sincospi(-2.0 * (double)((int64_t)j * q % fp.span[p]) / (double)fp.span[p], &sn, &cs);
+        Tab<KIND>::put(twp, 2 * i, cs);
+        Tab<KIND>::put(twp, 2 * i + 1, sn);
+    }
+}
+// Spectrum of a two-segment plan: position p holds H at its frequency.
+template <int KIND>
+__global__ void k_plan_spectrum(const double* __restrict__ S, const FftPasses fp, void* H) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= fp.L) return;
+    const int k = dif_freq(fp, p);
+    Tab<KIND>::put(H, (int64_t)blockIdx.y * fp.L + p, S[(int64_t)blockIdx.y * fp.L + min(k, fp.L - k)]);
+}
+// Index tables of a half-length plan (one CTA).  Pairs (k, M - k), k = 0 ..
+// M/2, in the order of the position of k: neighbouring threads then touch
+// neighbouring points (the frequency order would stride by M / radix_0 and put a
+// warp's accesses on one bank).  Items of the fused spectrum pass: the last
+// pass of radix R works on butterflies c of R consecutive positions; butterfly
+// c holds the frequencies kc + (M/R) q and its partner c' (frequency digits
+// M/R - kc) their mirror images M - k, at output R - 1 - q (kc = 0 and kc =
+// M/(2R) pair with themselves); one item per pair {c, c'}, kc = 0 .. M/(2R), in
+// the order of c, bit 31 marking kc = 0.
+__global__ void __launch_bounds__(1024) k_half_index(const FftPasses fp, uint32_t* pairs, int* pair_k, uint32_t* items,
+                                                     int* item_k) {
+    __shared__ int part[32];
+    const int M = fp.L, R = fp.radix[fp.npass - 1], NB = M / R, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int which = 0; which < (items ? 2 : 1); ++which) {
+        const int n = which ? NB : M;
+        int base = 0;
+        for (int c0 = 0; c0 < n; c0 += 1024) {
+            const int c = c0 + threadIdx.x;
+            const int k = c < n ? dif_freq(fp, which ? c * R : c) : n;
+            const bool in = c < n && k <= n / 2;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (lane == 0) part[warp] = __popc(m);
+            __syncthreads();
+            int at = base + __popc(m & ((1u << lane) - 1u)), all = 0;
+            for (int w = 0; w < 32; ++w) {
+                if (w < warp) at += part[w];
+                all += part[w];
+            }
+            if (in) {
+                if (which) {
+                    items[at] = (uint32_t)c | (uint32_t)(dif_pos(fp, (NB - k) % NB) / R) << 16 | (k == 0 ? 0x80000000u : 0u);
+                    item_k[at] = k;
+                } else {
+                    pairs[at] = (uint32_t)c | (uint32_t)dif_pos(fp, (M - k) % M) << 16;
+                    pair_k[at] = k;
+                }
+            }
+            base += all;
+            __syncthreads();
+        }
+    }
+}
+// Coefficients (alpha_k, alpha_{M-k}, beta_k, 0) of the paired real-spectrum
+// filter with 1/M folded in, from the spectra S [n_bands][2 M]: entry e of R
+// consecutive ones per index takes k = idx[e / R] + (M / R) (e % R).
+template <int KIND>
+__global__ void k_half_coef(const double* __restrict__ S, int M, const int* __restrict__ idx, int n, int R, int n_bands,
+                            void* C) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * R) return;
+    const int k = idx[e / R] + M / R * (e % R), N = 2 * M;
+    double sn, cs;
+    sincospi(2.0 * (double)k / (double)N, &sn, &cs);
+    for (int b = blockIdx.y; b < n_bands; b += gridDim.y) {
+        const double h1 = 2.0 * S[(int64_t)b * N + k], h2 = 2.0 * S[(int64_t)b * N + M - k];
+        const int64_t o = 4 * ((int64_t)b * n * R + e);
+        Tab<KIND>::put(C, o, 0.5 * ((h1 + h2) + (h2 - h1) * sn));
+        Tab<KIND>::put(C, o + 1, 0.5 * ((h1 + h2) - (h2 - h1) * sn));
+        Tab<KIND>::put(C, o + 2, -0.5 * (h2 - h1) * cs);
+        Tab<KIND>::put(C, o + 3, 0.0);
+    }
 }
 __global__ void k_spectrum_order(const double* __restrict__ Hp, double* H, const FftPasses fp) {
     const int64_t b = (int64_t)blockIdx.y * fp.L;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < fp.L; p += gridDim.x * blockDim.x) {
-        int rem = p, mult = 1, f = 0;   // the frequency at position p (mixed-radix digit reversal)
-        for (int i = 0; i < fp.npass; ++i) {
-            const int sr = fp.span[i] / fp.radix[i], d = rem / sr;
-            rem -= d * sr;
-            f += d * mult;
-            mult *= fp.radix[i];
-        }
-        H[b + f] = Hp[b + p];
-    }
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < fp.L; p += gridDim.x * blockDim.x)
+        H[b + dif_freq(fp, p)] = Hp[b + p];
 }
 // Twiddles (rows of filter_half3.cuh's Pass1Twiddle; [9][r1]) and, per band,
 // the coefficients of the paired spectrum step: item t pairs k = kc + r0 r1 q
@@ -283,12 +412,49 @@ void launch_band_circle(const double* band, int lam, int n_bands, int N, double*
     count_launches(1);
 }
 void launch_band_cosines(const double* band, int lam, int n_bands, int N, const double2* tw, double* H, cudaStream_t s) {
-    k_band_cosines<<<dim3((N / 2 + 8) / 8, n_bands), 256, 0, s>>>(band, lam, N, tw, H);
+    k_band_cosines<<<dim3((N / 2 + 8) / 8, (n_bands + COS_B - 1) / COS_B), 256, 0, s>>>(band, lam, n_bands, N, tw, H);
     count_launches(1);
 }
 void launch_spectrum_order(const double* Hp, double* H, int n_bands, const FftPasses& fp, cudaStream_t s) {
     k_spectrum_order<<<dim3((fp.L + 1023) / 1024, n_bands), 256, 0, s>>>(Hp, H, fp);
     count_launches(1);
+}
+template <int KIND>
+static void plan_tables(const double* S, int n_bands, const FftPasses& fp, void* tw, void* H, cudaStream_t s) {
+    k_plan_twiddles<KIND><<<(fp.L + 255) / 256, 256, 0, s>>>(fp, tw, nullptr, 0);
+    k_plan_spectrum<KIND><<<dim3((fp.L + 255) / 256, n_bands), 256, 0, s>>>(S, fp, H);
+    count_launches(2);
+}
+void launch_plan_tables(const double* S, int n_bands, const FftPasses& fp, int kind, void* tw, void* H, cudaStream_t s) {
+    if (kind == 0) plan_tables<0>(S, n_bands, fp, tw, H, s);
+    else if (kind == 1) plan_tables<1>(S, n_bands, fp, tw, H, s);
+    else plan_tables<2>(S, n_bands, fp, tw, H, s);
+}
+bool half_fused(const FftPasses& fp) {
+    const int R = fp.radix[fp.npass - 1];
+    return fp.span[fp.npass - 1] == R && (fp.L / R) % 2 == 0 && 16 % R == 0;
+}
+int64_t plan_powers(const FftPasses& fp) {
+    int64_t n = 0;
+    for (int i = 0; i < fp.npass; ++i) n += (int64_t)(fp.radix[i] - 1) * (fp.span[i] / fp.radix[i]);
+    return n > 0 ? n : 1;
+}
+template <int KIND>
+static void half_tables(const double* S, int n_bands, const FftPasses& fp, const HalfTables& t, cudaStream_t s) {
+    const int M = fp.L, R = fp.radix[fp.npass - 1], np = M / 2 + 1, ni = M / R / 2 + 1;
+    const bool fused = half_fused(fp);
+    const int64_t n = std::max<int64_t>(M, plan_powers(fp));
+    k_plan_twiddles<KIND><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(fp, t.tw, t.twp, plan_powers(fp));
+    k_half_index<<<1, 1024, 0, s>>>(fp, t.pairs, t.scratch, fused ? t.items : nullptr, t.scratch + np);
+    const int gy = std::min(n_bands, 64);
+    k_half_coef<KIND><<<dim3((np + 255) / 256, gy), 256, 0, s>>>(S, M, t.scratch, np, 1, n_bands, t.H);
+    if (fused) k_half_coef<KIND><<<dim3((ni * R + 255) / 256, gy), 256, 0, s>>>(S, M, t.scratch + np, ni, R, n_bands, t.Hi);
+    count_launches(fused ? 4 : 3);
+}
+void launch_half_tables(const double* S, int n_bands, const FftPasses& fp, int kind, const HalfTables& t, cudaStream_t s) {
+    if (kind == 0) half_tables<0>(S, n_bands, fp, t, s);
+    else if (kind == 1) half_tables<1>(S, n_bands, fp, t, s);
+    else half_tables<2>(S, n_bands, fp, t, s);
 }
 void launch_half3_tables(const double* H, int n_bands, int r0, int r1, float2* t1, float2* t2, float4* Hi, cudaStream_t s) {
     const int n = (r0 / 4 + 3) * 9 * r1, ni = r0 * r1 / 2 + 1;
