@@ -1831,8 +1831,15 @@ mm_status mm_apply_precond(mm_ctx* ctx, mm_precond which, const double* x, doubl
         CK(cudaMemcpyAsync(in3.p, x, nv * 24, cudaMemcpyHostToDevice, ctx->stream));
         xsrc = in3.as<double>();
     }
-    launch_map_in(xsrc, in4.as<V4<double>>(), nv, ctx->stream);
+    DevBuf o;
+    double* yd = y;
+    if (mem == MM_HOST) {
+        CK(o.ensure(nv * 24));
+        yd = o.as<double>();
+    }
+    bool direct = false;   // the tensor-core kernels read and write the caller's three-wide maps themselves
     if (which == MM_PRECOND_BD) {
+        launch_map_in(xsrc, in4.as<V4<double>>(), nv, ctx->stream);
         launch_bd_apply(ctx->d_bd.as<double>(), 0, in4.as<V4<double>>(), out4.as<V4<double>>(), ctx->n_pix, nrhs,
                         ctx->stream);
     } else {
@@ -1853,18 +1860,20 @@ mm_status mm_apply_precond(mm_ctx* ctx, mm_precond which, const double* x, doubl
         a.counter = ctx->w_counter.as<unsigned>();
         a.grid_x = ctx->grid_x;
         if (tc_wanted(ctx, a)) TRY(ensure_tc_scratch(ctx, a));
-        m2l_apply(ctx, a, in4.as<V4<double>>(), out4.as<V4<double>>(), -1);
+        // arrays that overlap without being the same one go through the context's copies
+        const uintptr_t x0 = reinterpret_cast<uintptr_t>(xsrc), y0 = reinterpret_cast<uintptr_t>(yd), len = (uintptr_t)nv * 24;
+        direct = use_tc(ctx, a) && (x0 == y0 || x0 + len <= y0 || y0 + len <= x0);
+        if (direct) {
+            launch_m2l_tc3(a, xsrc, yd, ctx->w_zu.as<double>(), ctx->stream);
+        } else {
+            launch_map_in(xsrc, in4.as<V4<double>>(), nv, ctx->stream);
+            m2l_apply(ctx, a, in4.as<V4<double>>(), out4.as<V4<double>>(), -1);
+        }
     }
     CKL();
-    if (mem == MM_HOST) {
-        DevBuf o;
-        CK(o.ensure(nv * 24));
-        launch_map_out(out4.as<V4<double>>(), o.as<double>(), nv, ctx->stream);
-        CK(cudaMemcpyAsync(y, o.p, nv * 24, cudaMemcpyDeviceToHost, ctx->stream));
-    } else {
-        launch_map_out(out4.as<V4<double>>(), y, nv, ctx->stream);
-    }
+    if (!direct) launch_map_out(out4.as<V4<double>>(), yd, nv, ctx->stream);
     CKL();
+    if (mem == MM_HOST) CK(cudaMemcpyAsync(y, yd, nv * 24, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (which == MM_PRECOND_2L) TRY(tc_fault_check(ctx));
     return MM_OK;

@@ -279,6 +279,8 @@ bool m2l_tc_pays(const PcgArgs& a);
 size_t m2l_tc_scratch_doubles(int n_pix, int nrhs, int k);
 void launch_m2l_tc(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, double* scratch,
                    cudaStream_t s);
+// the same on maps of three entries per pixel (one array or two that do not overlap)
+void launch_m2l_tc3(const PcgArgs& a, const double* v3, double* out3, double* scratch, cudaStream_t s);
 cudaError_t m2l_tc_fault_take(cudaStream_t s, int* fault);
 
 // Tall-skinny float64 products over vectors of n doubles (n = 4 n_pix).

@@ -169,6 +169,13 @@ __device__ __forceinline__ void load_seg(const double* row, int64_t kb, int64_t 
         for (int j = 0; j < TC_SEG; ++j) v[j] = kb + j < k1 ? __ldg(row + kb + j) : 0.0;
     }
 }
+// The same from a map of three entries per pixel (kb a multiple of 16 in
+// four-wide entries): the fourth entries are zero.
+__device__ __forceinline__ void load_seg3(const double* map3, int64_t kb, int64_t k1, double (&v)[TC_SEG]) {
+    const double* p = map3 + kb / 4 * 3;
+#pragma unroll
+    for (int j = 0; j < TC_SEG; ++j) v[j] = (j & 3) != 3 && kb + j < k1 ? __ldg(p + j / 4 * 3 + (j & 3)) : 0.0;
+}
 __device__ __forceinline__ void store_seg(const double (&v)[TC_SEG], int r, int kc0, uint32_t hi_tile,
                                           uint32_t lo_tile, uint32_t sbo) {
 #pragma unroll
@@ -186,13 +193,14 @@ __device__ __forceinline__ void store_seg(const double (&v)[TC_SEG], int r, int 
 // Dynamic shared memory: two stages of [A_hi, A_lo (128 x TC_KT), B_hi, B_lo
 // (np x TC_KT)] TF32, then two mbarriers and the TMEM address.  Eight warps:
 // all stage operands, warps 0-3 read the accumulator (TMEM lanes 0-127).
+// W3: the right-hand sides are maps of three entries per pixel (mm_apply_precond's own arrays).
 constexpr int TC_ZT = 256;
-__global__ void __launch_bounds__(TC_ZT, 2) k_m2l_tc_ztr(const PcgArgs a, const V4<double>* r, int kchunk) {
+template <bool W3>
+__global__ void __launch_bounds__(TC_ZT, 2) k_m2l_tc_ztr(const PcgArgs a, const double* R, int kchunk) {
     extern __shared__ __align__(128) unsigned char sm[];
     const int nrhs = a.nrhs, k = a.k;
     const int np = (k + 15) & ~15;
     const int64_t n4 = (int64_t)a.n_pix * 4;
-    const double* R = reinterpret_cast<const double*>(r);
     const double* Z = reinterpret_cast<const double*>(a.Z);
     constexpr uint32_t a_bytes = 128 * TC_KT * 4, sbo = TC_KT / 4 * 128;
     const uint32_t b_bytes = (uint32_t)np * TC_KT * 4;
@@ -223,19 +231,20 @@ __global__ void __launch_bounds__(TC_ZT, 2) k_m2l_tc_ztr(const PcgArgs a, const 
     // TC_ZT items, item t + TC_ZT.  Item t's next stage is loaded into registers while the current
     // one is converted and multiplied.
     const int n_items = 2 * (nrhs + k);
-    auto item_src = [&](int it) {
-        const int r = it >> 1;
-        return (r < nrhs ? R + (int64_t)r * n4 : Z + (int64_t)(r - nrhs) * n4) + (it & 1) * TC_SEG;
+    auto item_load = [&](int it, int64_t kb, double (&v)[TC_SEG]) {
+        const int r = it >> 1, h = (it & 1) * TC_SEG;
+        if (r >= nrhs) load_seg(Z + (int64_t)(r - nrhs) * n4, kb + h, k1, v);
+        else if constexpr (W3) load_seg3(R + (int64_t)r * a.n_pix * 3, kb + h, k1, v);
+        else load_seg(R + (int64_t)r * n4, kb + h, k1, v);
     };
     auto item_store = [&](const double (&v)[TC_SEG], int it, uint32_t sa) {
         const int r = it >> 1, kc0 = (it & 1) * (TC_SEG / 4);
         if (r < nrhs) store_seg(v, r, kc0, sa, sa + a_bytes, sbo);
         else store_seg(v, r - nrhs, kc0, sa + 2 * a_bytes, sa + 2 * a_bytes + b_bytes, sbo);
     };
-    auto item_k1 = [&](int it) { return k1 - (it & 1) * TC_SEG; };   // the row's end, shifted like its start
     const bool has1 = tid < n_items, has2 = tid + TC_ZT < n_items;
     double pre[TC_SEG];
-    if (has1 && nst > 0) load_seg(item_src(tid), k0, item_k1(tid), pre);
+    if (has1 && nst > 0) item_load(tid, k0, pre);
     for (int st = 0; st < nst && ok; ++st) {
         const int b = st & 1;
         if (st >= 2) ok = tc_mbar_wait(bars + b, ((st - 2) >> 1) & 1);   // MMAs of stage st - 2 read this buffer
@@ -248,10 +257,10 @@ __global__ void __launch_bounds__(TC_ZT, 2) k_m2l_tc_ztr(const PcgArgs a, const 
         if (has1) item_store(pre, tid, sa);
         if (has2) {
             double v2[TC_SEG];
-            load_seg(item_src(tid + TC_ZT), kb, item_k1(tid + TC_ZT), v2);
+            item_load(tid + TC_ZT, kb, v2);
             item_store(v2, tid + TC_ZT, sa);
         }
-        if (has1 && st + 1 < nst) load_seg(item_src(tid), kb + TC_KT, item_k1(tid), pre);
+        if (has1 && st + 1 < nst) item_load(tid, kb + TC_KT, pre);
         tc_fence_proxy();
         __syncthreads();
         if (tid == 0) {
@@ -340,10 +349,13 @@ __global__ void __launch_bounds__(TC_UT) k_m2l_tc_u(const PcgArgs a, const doubl
 // and tile in a fixed order, then over CTAs in CTA order by the last CTA.
 // Dynamic shared memory: B_hi, B_lo (nr x kp), A tiles Z_hi, Z_lo, AZ_hi,
 // AZ_lo (128 x kp), r^T z sums [4][nr], one mbarrier, the TMEM address.
+// a right-hand side's entry, read once and never again
+__device__ __forceinline__ double ldg_once(const double* p) { return __ldcs(p); }
 constexpr int TC_AT = 512;              // four groups of four warps
 constexpr int TC_AG = TC_AT / 128;
-__global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, const V4<double>* v, V4<double>* out,
-                                                              int finalize_beta, double* partial, int n_tiles) {
+template <bool W3>
+__global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, const double* V, double* O, int finalize_beta,
+                                                              double* partial, int n_tiles) {
     extern __shared__ __align__(128) unsigned char sm[];
     const int nrhs = a.nrhs, k = a.k;
     const int nr = (nrhs + 15) & ~15, kp = (k + 7) & ~7;
@@ -357,8 +369,6 @@ __global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, c
     const uint32_t ncols = tc_cols(2 * nr);
     const double* Z = reinterpret_cast<const double*>(a.Z);
     const double* AZ = reinterpret_cast<const double*>(a.AZ);
-    const double* V = reinterpret_cast<const double*>(v);
-    double* O = reinterpret_cast<double*>(out);
     if (tid == 0) {
         tc_mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -468,6 +478,9 @@ __global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, c
         const int64_t i = i0 + q * 32 + lane;
         const bool in = i < n4;
         const int64_t pix = i >> 2;
+        // this lane's entry of a right-hand side's map; three-wide maps have none for the fourth lane
+        const bool own = in && (!W3 || comp < 3);
+        const int64_t entry = W3 ? pix * 3 + comp : i, stride = W3 ? (int64_t)a.n_pix * 3 : n4;
         // row comp of the pixel's symmetric block [m0 m1 m2; m1 m3 m4; m2 m4 m5]
         const int r0 = comp == 0 ? 0 : (comp == 1 ? 1 : 2), r1 = comp == 0 ? 1 : (comp == 1 ? 3 : 4),
                   r2 = comp == 0 ? 2 : (comp == 1 ? 4 : 5);
@@ -482,7 +495,7 @@ __global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, c
             // the chunk's eight inputs are requested together, before the TMEM reads
             double xs[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) xs[j] = in && n0 + j < nrhs ? __ldg(V + (int64_t)(n0 + j) * n4 + i) : 0.0;
+            for (int j = 0; j < 8; ++j) xs[j] = own && n0 + j < nrhs ? ldg_once(V + (int64_t)(n0 + j) * stride + entry) : 0.0;
             float dz[8], daz[8];
             tc_ld8(lane_addr + n0, dz);
             tc_ld8(lane_addr + nr + n0, daz);
@@ -504,7 +517,7 @@ __global__ void __launch_bounds__(TC_AT, 1) k_m2l_tc_zu_apply(const PcgArgs a, c
                     m2 = (float)m[r2];
                 }
                 const float o = comp < 3 ? fmaf(m0, y0, fmaf(m1, y1, fmaf(m2, y2, dz[j]))) : 0.0f;
-                if (in && active) O[(int64_t)n * n4 + i] = f2d_exact(o);
+                if (own && active) O[(int64_t)n * stride + entry] = f2d_exact(o);
                 if (finalize_beta >= 0) {
                     // the warp's 32 products summed in float32, the warps' sums in float64
                     float d = x * o;
@@ -585,9 +598,10 @@ size_t m2l_tc_scratch_doubles(int n_pix, int nrhs, int k) {
 }
 
 // M_2l v -> out on the tensor cores (see the top of this file); scratch holds
-// m2l_tc_scratch_doubles(n_pix, nrhs, k) doubles.
-void launch_m2l_tc(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, double* scratch,
-                   cudaStream_t s) {
+// m2l_tc_scratch_doubles(n_pix, nrhs, k) doubles.  W3: v and out are maps of
+// three entries per pixel (they may be one array, not overlap otherwise).
+template <bool W3>
+static void launch_tc(const PcgArgs& a, const double* v, double* out, int finalize_beta, double* scratch, cudaStream_t s) {
     const int k = a.k, nrhs = a.nrhs;
     const int np = (k + 15) & ~15, nr = (nrhs + 15) & ~15, kp = (k + 7) & ~7;
     const int64_t n4 = (int64_t)a.n_pix * 4;
@@ -603,18 +617,25 @@ void launch_m2l_tc(const PcgArgs& a, const V4<double>* v, V4<double>* out, int f
     const size_t sm2 = 2 * (size_t)nr * kp * 4 + 4 * (size_t)128 * kp * 4 + 4 * (size_t)nr * 8 + 32;
     static std::atomic<size_t> conf1{0}, conf2{0};
     raise_smem_once(conf1, sm1, [](size_t v) {
-        cudaFuncSetAttribute(k_m2l_tc_ztr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
+        cudaFuncSetAttribute(k_m2l_tc_ztr<W3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
     });
     raise_smem_once(conf2, sm2, [](size_t v) {
-        cudaFuncSetAttribute(k_m2l_tc_zu_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
+        cudaFuncSetAttribute(k_m2l_tc_zu_apply<W3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
     });
     PcgArgs a1 = a;
     a1.partial = scratch;
-    k_m2l_tc_ztr<<<g_used, TC_ZT, sm1, s>>>(a1, v, kchunk);
+    k_m2l_tc_ztr<W3><<<g_used, TC_ZT, sm1, s>>>(a1, v, kchunk);
     k_m2l_tc_u<<<nrhs, TC_UT, 0, s>>>(a, scratch, g_used);
-    k_m2l_tc_zu_apply<<<g2, TC_AT, sm2, s>>>(a, v, out, finalize_beta, scratch + (size_t)g1 * nrhs * std::max(k, 1),
+    k_m2l_tc_zu_apply<W3><<<g2, TC_AT, sm2, s>>>(a, v, out, finalize_beta, scratch + (size_t)g1 * nrhs * std::max(k, 1),
                                              n_tiles);
     count_launches(3);
+}
+void launch_m2l_tc(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, double* scratch,
+                   cudaStream_t s) {
+    launch_tc<false>(a, reinterpret_cast<const double*>(v), reinterpret_cast<double*>(out), finalize_beta, scratch, s);
+}
+void launch_m2l_tc3(const PcgArgs& a, const double* v3, double* out3, double* scratch, cudaStream_t s) {
+    launch_tc<true>(a, v3, out3, -1, scratch, s);
 }
 
 // Failures recorded by the tensor-core kernels since the last call (0: none);

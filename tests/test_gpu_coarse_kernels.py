@@ -41,3 +41,31 @@ def test_coarse_space_of_every_size(nx, k, nrhs):
         ref = np.einsum("pij,pj->pi", M, x[r] - np.einsum("apc,a->pc", AZ, u)) + np.einsum("apc,a->pc", Z, u)
         assert_close(y[r], ref, 1e-9)
     c.close()
+
+
+@pytest.mark.parametrize("nx", [7, 9, 32])
+@pytest.mark.parametrize("nrhs,k", [(8, 3), (33, 17), (64, 64), (128, 40)])
+def test_tensor_core_path_reads_and_writes_three_wide_maps(nx, nrhs, k):
+    """mm_apply_precond's own arrays as operands: odd pixel counts (rows off 16-byte boundaries), an array
+    that starts at an odd element, in place, and an output that overlaps the input shifted by a map
+    (staged, the same values).  2e-5, the tensor-core path's tolerance, against float64."""
+    import torch
+    scan = synth.make_scan(nx=nx, ny=nx, n_det=2, n_t=max(4096, 40 * nx * nx), n_int=2, half_bw=16, f_knee=1.0, seed=nx)
+    c = MM.Context(0, None, MM.MM_FP64)
+    c.setup_scan(scan)
+    assert c.build_bd(1e-6) == 0
+    rng = np.random.default_rng(nrhs)
+    c.set_coarse(rng.standard_normal((min(k, nx * nx), scan.n_pix, 3)))
+    x = torch.from_numpy(rng.standard_normal((nrhs, scan.n_pix, 3))).cuda()
+    c.set_option("tc_coarse", 0)
+    ref = c.apply_precond(MM.MM_PRECOND_2L, x).cpu().numpy()
+    c.set_option("tc_coarse", 2)
+    n = x.numel()
+    buf = torch.zeros(2 * n + 3 * scan.n_pix + 1, dtype=torch.float64, device="cuda")
+    for shift, out_at in ((0, n), (1, n + 1), (0, 0), (1, 1), (0, 3 * scan.n_pix)):
+        xs = buf[shift:shift + n].view(nrhs, scan.n_pix, 3)
+        xs.copy_(x)
+        ys = buf[out_at:out_at + n].view(nrhs, scan.n_pix, 3)
+        c.apply_precond(MM.MM_PRECOND_2L, xs, out=ys)
+        assert_close(ys.cpu().numpy().reshape(-1, 3), ref.reshape(-1, 3), 2e-5)
+    c.close()
