@@ -532,17 +532,19 @@ __device__ __forceinline__ V4<float> ldmap(const V4<float>* m) {
     return {v.x, v.y, v.z, v.w};
 }
 template <>
-__device__ __forceinline__ V4<double> ldmap(const V4<double>* m) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(m));
-    const double2 b = __ldg(reinterpret_cast<const double2*>(m) + 1);
-    return {a.x, a.y, b.x, b.y};
+__device__ __forceinline__ V4<double> ldmap(const V4<double>* m) {   // one 256-bit load
+    V4<double> v;
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(m));
+    return v;
 }
 
 template <>
 __device__ __forceinline__ V4<df> ldmap(const V4<df>* m) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(m));
-    const float4 b = __ldg(reinterpret_cast<const float4*>(m) + 1);
-    return {df(a.x, a.y), df(a.z, a.w), df(b.x, b.y), df(b.z, b.w)};
+    V4<df> v;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v.x.hi), "=f"(v.x.lo), "=f"(v.y.hi), "=f"(v.y.lo), "=f"(v.z.hi), "=f"(v.z.lo), "=f"(v.w.hi), "=f"(v.w.lo)
+        : "l"(m));
+    return v;
 }
 
 // (P x)_t for the map a.xmap: the timeline residual d_t - (P x)_t, whose
