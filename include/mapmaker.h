@@ -285,7 +285,9 @@ mm_status mm_solve(mm_ctx* ctx, const void* tod, double* map_out, int32_t nrhs,
  * MM_FP32_MIXED, the smallest relative tolerance asked of a float32-operator
  * PCG run between float64-accurate refinements (default 2e-6);
  * "half_transform": 1 (default) lets a whole block of N real samples run as
- * one N/2-point complex transform per CTA (paired real-spectrum step), 0
+ * one N/2-point complex transform per CTA (paired real-spectrum step), 2
+ * prefers such a block split by frequency over two CTAs where native float64
+ * products have that form (with 1 it is used where it times faster), 0
  * keeps two blocks per N-point transform; "coarse_prefix": 1 (default) forms
  * the per-RHS coarse products A_i Z of an uneven-length two-level batch from
  * products over whole blocks computed once per coarse space (block-diagonal
@@ -314,7 +316,7 @@ mm_status mm_set_option(mm_ctx* ctx, const char* name, double value);
  * launched by the library since load), "plan_fft_len", "plan_fft_log2",
  * "plan_whole" (the plan a single-RHS product uses: 0 overlap-save segments,
  * 1 whole blocks two per transform, 2 whole blocks as half-length complex
- * transforms), "harvested" (Lanczos
+ * transforms, 3 those split over two CTAs each), "harvested" (Lanczos
  * vectors kept by the last M_BD solve), "device_bytes" (device memory in use),
  * "coarse_len" (samples per detector of the operator the basis was built from),
  * "coarse_rank_min" (the fewest coarse vectors a right-hand side of the last

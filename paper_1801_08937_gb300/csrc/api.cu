@@ -63,7 +63,8 @@ struct Plan {
     int variant = 0;   // 1 direct, 2 fft
     int L = 0, logL = 0, V = 0;
     int whole = 0;     // FFT: 1 one transform per whole block (no overlap-save halo), two blocks
-                       // per CTA; 2 one block per CTA as an L/2-point complex transform
+                       // per CTA; 2 one block per CTA as an L/2-point complex transform; 3 the
+                       // same split by frequency over two CTAs (float64)
     FftPasses fp{};
     bool three = false;   // whole = 2, float32: the three-pass transform
     bool even = true;     // every segment starts at an even sample
@@ -321,6 +322,22 @@ bool fft_passes(int L, FftPasses* fp, int maxr = 16) {
 
 size_t smem_limit_bytes() { return 220 * 1024; }
 
+// Pass plan of a block split over two CTAs (k_filter_split): radix 4 first,
+// then the passes of M / 4 points.
+bool split_shape(int M) { return M == 2304 || M == 4608 || M == 9216; }
+void split_passes(int M, FftPasses* fp) {
+    FftPasses rest{};
+    fft_passes(M / 4, &rest, 8);
+    fp->L = M;
+    fp->npass = rest.npass + 1;
+    fp->radix[0] = 4;
+    fp->span[0] = M;
+    for (int i = 0; i < rest.npass; ++i) {
+        fp->radix[i + 1] = rest.radix[i];
+        fp->span[i + 1] = rest.span[i];
+    }
+}
+
 // FFT length and mode candidates: whole blocks (one block per transform, no
 // halo, when L >= n_b + lambda) or overlap-save segments of V = L - 2 lambda
 // outputs.  Cost model: transform points x passes plus gathered and
@@ -350,7 +367,12 @@ std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, i
                 const double ctash = c->n_blocks;
                 const double per_ctah = (double)(L / 2) * fh.npass * 44.0 + 2.0 * (double)c->n_samples / ctash * 45.0;
                 const double wavesh = std::ceil(ctash / (152.0 * per_smh));
-                out.push_back({L, 2, wavesh * per_ctah + 1e-3 * ((double)c->n_blocks * (L / 2) * fh.npass * 44.0)});
+                const double cost = wavesh * per_ctah + 1e-3 * ((double)c->n_blocks * (L / 2) * fh.npass * 44.0);
+                out.push_back({L, 2, cost});
+                // float64 blocks split by frequency over two CTAs, where one CTA each leaves SMs idle; timed, or
+                // asked for by "half_transform" = 2
+                if (f64 == 1 && split_shape(L / 2) && (c->opt_half == 2 || c->n_blocks < 152))
+                    out.push_back({L, 3, c->opt_half == 2 ? 0.0 : 1.001 * cost});
             }
             const size_t sm = fft_smem_bytes(L, f64 != 0);
             if (sm > smem_limit_bytes()) continue;
@@ -510,8 +532,9 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     FftPasses fp{};
     int logL = 0;
     if (variant == 2) {
-        fft_passes(whole == 2 ? L / 2 : L, &fp, f64 ? 8 : 16);
-        logL = ilog2(whole == 2 ? L / 2 : L);
+        if (whole == 3) split_passes(L / 2, &fp);
+        else fft_passes(whole == 2 ? L / 2 : L, &fp, f64 ? 8 : 16);
+        logL = ilog2(whole >= 2 ? L / 2 : L);
     }
     for (auto& p : ctx->plans)
         if (p->variant == variant && p->L == L && p->V == V && p->whole == whole && p->f64 == f64 &&
@@ -520,7 +543,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
             return MM_OK;
         }
     std::vector<Seg> segs;
-    const bool single = (variant == 2 && whole == 2);   // one segment per CTA
+    const bool single = (variant == 2 && whole >= 2);   // segments one by one, not in pairs
     auto push = [&](const Seg& s) {
         if (!single && segs.size() % 2 == 1 && (segs.back().band != s.band || segs.back().shift != s.shift)) {
             Seg e{};
@@ -577,7 +600,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     p->lens = lens;
     p->starts = starts;
     int r0 = 0, r1 = 0;
-    p->three = single && f64 == 0 && half3_shape(L / 2, &r0, &r1);
+    p->three = single && f64 == 0 && half3_shape(L / 2, &r0, &r1);   // whole = 2
     for (const Seg& sg : segs) p->even = p->even && sg.out0 % 2 == 0;
     p->n_work = (int)(single ? segs.size() : segs.size() / 2);
     CK(p->segs.ensure(std::max<size_t>(1, segs.size()) * sizeof(Seg)));
@@ -585,7 +608,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
         CK(cudaMemcpyAsync(p->segs.p, segs.data(), segs.size() * sizeof(Seg), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (p->three) TRY(build_half3_tables(ctx, p->ft, L));
-    else if (variant == 2 && whole == 2) TRY(build_half_tables(ctx, p->ft, fp, L, f64));
+    else if (variant == 2 && whole >= 2) TRY(build_half_tables(ctx, p->ft, fp, L, f64));
     else if (variant == 2) TRY(build_fft_tables(ctx, p->ft, fp, f64));
     if (f64 == 2 && !ctx->have_csdf) {
         CK(ctx->d_csdf.ensure((size_t)ctx->n_samples * 16));
@@ -663,7 +686,7 @@ std::vector<std::pair<TuneKey, TuneVal>>& tune_cache() {
 bool tune_lookup(const TuneKey& k, bool allow_half, TuneVal* v) {
     std::lock_guard<std::mutex> lock(tune_mutex());
     for (auto& kv : tune_cache())
-        if (kv.first == k && (allow_half || kv.second.whole != 2)) {
+        if (kv.first == k && (allow_half || kv.second.whole < 2)) {
             *v = kv.second;
             return true;
         }
@@ -704,7 +727,7 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
         const bool short_half = cands[i].whole == 2 && !half.empty() && cands[i].L <= half[std::min<size_t>(1, half.size() - 1)];
         int r0 = 0, r1 = 0;
         const bool three = f64 == 0 && cands[i].whole == 2 && half3_shape(cands[i].L / 2, &r0, &r1);
-        if (i < 6 || short_half || three)
+        if (i < 6 || short_half || three || cands[i].whole == 3)
             opts.push_back(
                 {2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
     }
@@ -846,8 +869,9 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
         FftTables& ft = plan->ft;
         a.H = ft.H.p;
         a.tw = ft.tw.p;
-        if (plan->whole == 2) {
+        if (plan->whole >= 2) {
             a.half = 1;
+            a.split = plan->whole == 3 ? 1 : 0;
             a.three = plan->three ? 1 : 0;
             a.even = plan->even ? 1 : 0;
             a.L = plan->L / 2;
@@ -2568,7 +2592,7 @@ mm_status mm_set_option(mm_ctx* ctx, const char* name, double value) {
     } else if (n == "autotune") {
         ctx->opt_autotune = v ? 1 : 0;
     } else if (n == "half_transform") {
-        ctx->opt_half = v ? 1 : 0;
+        ctx->opt_half = v == 2 ? 2 : (v ? 1 : 0);
     } else if (n == "coarse_prefix") {
         ctx->opt_coarse_prefix = v ? 1 : 0;
     } else if (n == "coarse_fallback") {

@@ -124,6 +124,7 @@ struct FilterArgs {
     const void* Hi;        // half, fused last pass: [n_bands][items][R] coefficients (alpha_k, alpha_{L-k}, beta_k)
     const void* twp;       // half: per-pass twiddles W_S^(j q), pass by pass, [q - 1][j] within a pass; may be null
     int half;              // 1: one whole block per CTA as L = N/2 complex points
+    int split;             // half, float64: a block over two CTAs (k_filter_split)
     int three;             // half, float32: three passes of radix r0, r1, 9 (half3_shape)
     int even;              // every segment starts at an even sample
     int* fault;            // set to 1 by a bounded wait that gave up

@@ -4,7 +4,10 @@
 namespace mm {
 
 void launch_filter_fft_f64(const FilterArgs& a, bool from_tod, cudaStream_t s) {
-    if (a.half) {
+    if (a.split) {
+        if (from_tod) launch_split_t<true>(a, s);
+        else launch_split_t<false>(a, s);
+    } else if (a.half) {
         if (from_tod) launch_half_t<double, true>(a, s);
         else launch_half_t<double, false>(a, s);
     } else {

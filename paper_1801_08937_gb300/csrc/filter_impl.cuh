@@ -1448,16 +1448,21 @@ __device__ __forceinline__ void half_scatter_t(const FilterArgs& a, const Seg& S
 // the spectrum step of every pair (k, M - k), written conjugated, and the
 // first conjugate-domain pass (DFT_R, no twiddles), so the spectrum step
 // costs no shared-memory round trip and no barrier of its own.
-template <typename T, int M, int NT, int R>
+// Place of butterfly c in the CTA's buffer (negative: another CTA's).
+struct AllButterflies {
+    __device__ __forceinline__ int operator()(int c) const { return c; }
+};
+template <typename T, int M, int NT, int R, typename Place = AllButterflies>
 __device__ __forceinline__ void ct_fused_spectrum(C2<T>* s, const uint32_t* __restrict__ items, const void* Hi,
-                                                  int64_t cb) {
+                                                  int64_t cb, Place place = Place()) {
     constexpr int NB = M / R;
     constexpr int NI = NB / 2 + 1;
     static_assert(NB % 2 == 0 && 16 % R == 0, "fused spectrum pass: butterfly pairs inside padding groups");
 #pragma unroll 1
     for (int i = threadIdx.x; i < NI; i += NT) {
         const uint32_t pr = __ldg(items + i);
-        const int c = (int)(pr & 0xffffu), c2 = (int)((pr >> 16) & 0x7fffu);
+        const int c = place((int)(pr & 0xffffu)), c2 = place((int)((pr >> 16) & 0x7fffu));
+        if (c < 0) continue;   // a pair lies in one CTA
         T aa[R], ab[R], be[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) ld_coef(Hi, cb + (int64_t)i * R + q, aa[q], ab[q], be[q]);
@@ -1561,6 +1566,114 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 512 / NT) k_filter_ha
     else fft_dit_conj<T>(s, tw, a.fp);
     if constexpr (std::is_same<T, float>::value) half_scatter_f32<NT>(a, S, s, M);
     else half_scatter_t<T, NT>(a, S, s);
+}
+
+// ---------------- whole block split by frequency over two CTAs, float64 ----------------
+// With fewer blocks than SMs one CTA per block leaves float64 pipes idle (64
+// blocks of 4096 samples: 64 of 152 SMs).  The first pass of the half-length
+// transform (radix 4) sorts the frequencies into classes k mod 4; classes 0 and 2
+// pair with themselves in the spectrum step, 1 and 3 with each other, and the
+// last inverse pass and P^T are linear in the classes.  So two CTAs take a block:
+// both gather it, fold it into their two classes (M / 4 points each), transform,
+// filter and transform back those, and scatter their parts of the filtered
+// timeline; they exchange nothing.  Gather and scatter are done twice (five
+// float64 operations a sample), the transform, some forty, once.  Measured on
+// that problem: 67 us in 2048-point overlap-save segments (128 CTAs) -> 51 us,
+// the float64 pipes of the 128 SMs 62 % busy (passes of 128 and 144 butterflies
+// on four SM partitions are what is left).
+template <int M> struct SplitPlan {
+    static constexpr int SR = M / 4;
+    static constexpr CtPlan pl = make_ct_plan(SR, 8);
+    static constexpr int R = pl.r[pl.np - 1];
+};
+// Passes P .. END - 1 (forward) or P .. 0 (inverse) of both classes, twiddles from the tables behind the radix-4 pass's.
+template <typename T, int M, int NT, int P, bool DIT>
+__device__ __forceinline__ void split_passes(C2<T>* s, const C2<T>* tt) {
+    using SP = SplitPlan<M>;
+    constexpr int END = SP::pl.np - 1;
+    if constexpr (P >= 0 && P < END) {
+        ct_pass<T, SP::pl.r[P], SP::pl.s[P], 2 * SP::SR, NT, DIT, true>(s, nullptr, tt + 3 * SP::SR + SP::pl.toff[P]);
+        __syncthreads();
+        split_passes<T, M, NT, DIT ? P - 1 : P + 1, DIT>(s, tt);
+    }
+}
+
+template <typename T, bool FROM_TOD, int NT, int M>
+__global__ void __launch_bounds__(NT, 2) k_filter_split(const FilterArgs a) {
+    using SP = SplitPlan<M>;
+    constexpr int SR = SP::SR, R = SP::R, NBC = SR / R;   // butterflies of the last pass per class
+    static_assert(SR % 16 == 0 && 16 % R == 0, "classes and butterflies keep to the padding groups");
+    extern __shared__ __align__(16) unsigned char smraw[];
+    C2<T>* s = reinterpret_cast<C2<T>*>(smraw);
+    const Seg S = a.segs[blockIdx.x >> 1];
+    const int odd = blockIdx.x & 1;   // classes 0 and 2, or 1 and 3
+    if (!seg_active<T>(a, S)) return;
+    const C2<T>* tt = reinterpret_cast<const C2<T>*>(a.twp);
+    const bool with_map = !FROM_TOD || a.xmap != nullptr;
+    const V4<T>* map =
+        with_map ? reinterpret_cast<const V4<T>*>(FROM_TOD ? a.xmap : a.src) + (int64_t)S.rhs * a.n_pix : nullptr;
+    auto sample = [&](int i) -> T {   // one value of the block's timeline
+        if (i >= S.n_out) return T(0);
+        const int64_t t = S.out0 + i;
+        T v = T(0);
+        if (FROM_TOD)
+            v = a.tod_is_float ? T(__ldg(reinterpret_cast<const float*>(a.src) + S.rhs * a.n_samples + t))
+                               : from64<T>(__ldg(reinterpret_cast<const double*>(a.src) + S.rhs * a.n_samples + t));
+        if (with_map) {
+            const int p = __ldg(a.pix + t);
+            if (p >= 0) {
+                T c, sn;
+                weights(a, t, c, sn);
+                const V4<T> m = ldmap<T>(map + p);
+                const T px = m.x + c * m.y + sn * m.z;
+                v = FROM_TOD ? v - px : px;
+            }
+        }
+        return v;
+    };
+    for (int j = threadIdx.x; j < SR; j += NT) {
+        C2<T> z[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) z[r] = C2<T>{sample(2 * (j + SR * r)), sample(2 * (j + SR * r) + 1)};
+        C2<T> u, v;
+        if (!odd) {
+            const C2<T> e = cadd(z[0], z[2]), f = cadd(z[1], z[3]);
+            u = cadd(e, f);
+            v = cmul(csub(e, f), ldtw(tt, SR + j));
+        } else {
+            const C2<T> e = csub(z[0], z[2]), f = csub(z[1], z[3]);
+            u = cmul(C2<T>{e.x + f.y, e.y - f.x}, ldtw(tt, j));            // e - i f
+            v = cmul(C2<T>{e.x - f.y, e.y + f.x}, ldtw(tt, 2 * SR + j));   // e + i f
+        }
+        s[sidx(j)] = u;
+        s[sidx(SR + j)] = v;
+    }
+    __syncthreads();
+    split_passes<T, M, NT, 0, false>(s, tt);
+    ct_fused_spectrum<T, M, NT, R>(s, a.items, a.Hi, (int64_t)S.band * ((M / R) / 2 + 1) * R, [&](int c) {
+        const int d = c / NBC;
+        return (d & 1) == odd ? (d >> 1) * NBC + c % NBC : -1;
+    });
+    __syncthreads();
+    split_passes<T, M, NT, SP::pl.np - 2, true>(s, tt);
+    // this CTA's part of the filtered timeline at point j + SR r is u or v times a power of i (conjugate domain)
+    for (int j = threadIdx.x; j < SR; j += NT) {
+        const C2<T> e = odd ? cmul(s[sidx(j)], ldtw(tt, j)) : s[sidx(j)];
+        const C2<T> f = cmul(s[sidx(SR + j)], ldtw(tt, (odd ? 2 * SR : SR) + j));
+        s[sidx(j)] = cadd(e, f);
+        s[sidx(SR + j)] = csub(e, f);
+    }
+    __syncthreads();
+    scatter8_t<T, NT / 32>(a, S, true, [&](int i) {
+        const int m = i >> 1, r = m / SR;
+        const C2<T> w = s[sidx((r & 1) * SR + m - r * SR)];
+        // odd classes: 1, -i, -1, i; even ones: 1 throughout.  An even sample is the real part, an odd one minus
+        // the imaginary part.
+        T v;
+        if (odd && (r & 1)) v = (i & 1) ? w.x : w.y;   // of -i w
+        else v = (i & 1) ? -w.y : w.x;
+        return odd && r >= 2 ? -v : v;
+    });
 }
 
 // ---------------- direct band variant, float32, four samples per thread ----------------
@@ -1828,6 +1941,26 @@ inline void launch_half_t(const FilterArgs& a, cudaStream_t s) {
             default: break;
         }
         return launch_half_nt<T, FROM_TOD, 256, 0>(a, sm, s);
+    }
+}
+
+// Whole blocks split over two CTAs (a.L = M of split_shape), float64.
+template <bool FROM_TOD, int M>
+inline void launch_split_m(const FilterArgs& a, cudaStream_t s) {
+    constexpr int NT = 256;
+    const size_t sm = fft_smem_bytes(M / 2, true);
+    static std::atomic<size_t> configured{0};
+    raise_smem_once(configured, sm, [](size_t v) { configure_smem(k_filter_split<double, FROM_TOD, NT, M>, v, NT); });
+    k_filter_split<double, FROM_TOD, NT, M><<<2 * a.n_work, NT, sm, s>>>(a);
+    count_launches(1);
+}
+template <bool FROM_TOD>
+inline void launch_split_t(const FilterArgs& a, cudaStream_t s) {
+    if (a.n_work <= 0) return;
+    switch (a.L) {
+        case 9216: return launch_split_m<FROM_TOD, 9216>(a, s);
+        case 4608: return launch_split_m<FROM_TOD, 4608>(a, s);
+        default: return launch_split_m<FROM_TOD, 2304>(a, s);
     }
 }
 

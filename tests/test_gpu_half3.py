@@ -97,3 +97,34 @@ def test_float64_scatter_of_every_fill(prec, L, pixels, nx):
     d = np.random.default_rng(1).standard_normal((1, scan.n_samples)).astype(c.tod_dtype)
     assert_close(c.rhs(d)[0], O.rhs(prob, d[0].astype(np.float64)), 1e-11)
     c.close()
+
+
+@pytest.mark.parametrize("L", [4608, 9216, 18432])
+@pytest.mark.parametrize("pixels,nx", [("raster", 16), ("random", 8), ("steps", 16)])
+def test_float64_block_split_over_two_ctas(L, pixels, nx):
+    """A x and b of blocks split by frequency, every fill of the transform: 1e-11; a whole solve with it
+    reaches the map of the unsplit plan (1e-7 at a tolerance of 1e-11: pixels with three hits and an rcond
+    of 1e-3 amplify the residual)."""
+    full = L - LAM
+    scan = scan_with([full, 1, 2, 3, full - 1, 255, 257, full // 2, L // 4, L // 4 + 1, 7], pixels, nx, L + nx)
+    maps = []
+    for half in (2, 1):
+        c = MM.Context(0, None, MM.MM_FP64)
+        c.set_option("filter", 2)
+        c.set_option("half_transform", half)
+        c.set_option("fft_len", L)
+        c.setup_scan(scan)
+        x = np.random.default_rng(L).standard_normal((2, scan.n_pix, 3))
+        y = c.apply_A(x)
+        assert c.get_option("plan_whole") == (3 if half == 2 else 2)
+        prob = O.Problem.from_scan(scan)
+        for r in range(2):
+            assert_close(y[r], O.apply_A(prob, x[r]), 1e-11)
+        d = np.random.default_rng(1).standard_normal((1, scan.n_samples))
+        assert_close(c.rhs(d)[0], O.rhs(prob, d[0]), 1e-11)
+        c.build_bd(1e-3)
+        m, info = c.solve(d, tol=1e-11, max_iter=1000)
+        assert info[0]["status"] == "MM_OK"
+        maps.append(m[0])
+        c.close()
+    assert_close(maps[0], maps[1], 1e-7)
