@@ -1019,8 +1019,18 @@ void precond_step(mm_ctx* ctx, const PcgArgs& a, int finalize_beta) {
     }
 }
 
+// With M_BD on a small map an iteration is the product and one kernel.
+bool pcg_stepped(const mm_ctx* ctx, const PcgArgs& a) { return ctx->precond == MM_PRECOND_BD && pcg_step_fits(a); }
+
 mm_status pcg_iteration(mm_ctx* ctx) {
     PcgArgs a = pcg_args(ctx);
+    if (pcg_stepped(ctx, a)) {   // the search direction is ready, from pcg_start or the last step
+        TRY(run_filter(ctx, ctx->plan_op, false, ctx->s_src.p, ctx->s_q.p, a.st, 0));
+        launch_pcg_step(a, ctx->stream);
+        if (ctx->harvest_on) launch_harvest(a, ctx->stream);
+        CKL();
+        return MM_OK;
+    }
     launch_pcg_src(a, 0, ctx->stream);
     TRY(run_filter(ctx, ctx->plan_op, false, ctx->s_src.p, ctx->s_q.p, a.st, 0));
     launch_pcg_pq(a, ctx->stream);
@@ -1048,6 +1058,7 @@ mm_status pcg_start(mm_ctx* ctx, const V4<double>* b, const std::vector<double>&
     launch_pcg_init(a, b, ctx->stream);
     precond_step(ctx, a, 0);
     if (ctx->harvest_on && ctx->precond == MM_PRECOND_BD) launch_harvest(a, ctx->stream);
+    if (pcg_stepped(ctx, a)) launch_pcg_src(a, 0, ctx->stream);
     CKL();
     return MM_OK;
 }

@@ -565,29 +565,30 @@ __global__ void k_bd_dot(const PcgArgs a, int finalize_beta) {
     }
 }
 
-// p = z + beta p (first: p = z); src = p in the operator precision; qacc = 0.
+// p = z + beta p; src = p in the operator precision; qacc = 0.
+__device__ __forceinline__ void pcg_direction(const PcgArgs& a, int64_t j, double beta) {
+    const V4<double> zv = a.z[j];
+    V4<double> pv = a.p[j];
+    pv = V4<double>{zv.x + beta * pv.x, zv.y + beta * pv.y, zv.z + beta * pv.z, 0.0};
+    a.p[j] = pv;
+    if (a.src_f32 == 1) {
+        reinterpret_cast<V4<float>*>(a.src)[j] = V4<float>{(float)pv.x, (float)pv.y, (float)pv.z, 0.0f};
+        reinterpret_cast<V4<float>*>(a.qacc)[j] = V4<float>{0.f, 0.f, 0.f, 0.f};
+    } else if (a.src_f32 == 2) {
+        // double-float operator input, float64 accumulators
+        reinterpret_cast<V4<df>*>(a.src)[j] = V4<df>{df(pv.x), df(pv.y), df(pv.z), df(0.0)};
+        reinterpret_cast<V4<double>*>(a.qacc)[j] = V4<double>{0, 0, 0, 0};
+    } else {
+        reinterpret_cast<V4<double>*>(a.src)[j] = pv;
+        reinterpret_cast<V4<double>*>(a.qacc)[j] = V4<double>{0, 0, 0, 0};
+    }
+}
 __global__ void k_pcg_src(const PcgArgs a, int first) {
     const int rhs = blockIdx.y;
     if (!a.st[rhs].active) return;
     const double beta = first ? 0.0 : a.st[rhs].beta;
     const int64_t off = (int64_t)rhs * a.n_pix;
-    PIX_LOOP(i) {
-        const V4<double> zv = a.z[off + i];
-        V4<double> pv = a.p[off + i];
-        pv = first ? zv : V4<double>{zv.x + beta * pv.x, zv.y + beta * pv.y, zv.z + beta * pv.z, 0.0};
-        a.p[off + i] = pv;
-        if (a.src_f32 == 1) {
-            reinterpret_cast<V4<float>*>(a.src)[off + i] = V4<float>{(float)pv.x, (float)pv.y, (float)pv.z, 0.0f};
-            reinterpret_cast<V4<float>*>(a.qacc)[off + i] = V4<float>{0.f, 0.f, 0.f, 0.f};
-        } else if (a.src_f32 == 2) {
-            // double-float operator input, float64 accumulators
-            reinterpret_cast<V4<df>*>(a.src)[off + i] = V4<df>{df(pv.x), df(pv.y), df(pv.z), df(0.0)};
-            reinterpret_cast<V4<double>*>(a.qacc)[off + i] = V4<double>{0, 0, 0, 0};
-        } else {
-            reinterpret_cast<V4<double>*>(a.src)[off + i] = pv;
-            reinterpret_cast<V4<double>*>(a.qacc)[off + i] = V4<double>{0, 0, 0, 0};
-        }
-    }
+    PIX_LOOP(i) pcg_direction(a, off + i, beta);
 }
 
 __device__ __forceinline__ V4<double> load_q(const PcgArgs& a, int64_t j) {
@@ -676,6 +677,141 @@ __global__ void k_pcg_update(const PcgArgs a) {
             a.counter[rhs] = 0;
         }
     }
+}
+
+// The whole of a PCG iteration behind the product, with M_BD, for small maps:
+// alpha from p^T q; x, r and z = M_BD r with ||r|| and r^T z; beta; the next
+// search direction, the operator's input and cleared accumulators.  One cluster
+// of eight CTAs per right-hand side sums over its CTAs through distributed
+// shared memory (rank order), so the three launches and their last-CTA
+// reductions (21 us an iteration at 1024 pixels) become one of 11 us.  Used up to
+// STEP_MAX_PIX pixels: beyond, eight SMs take longer than the launches cost.
+constexpr int STEP_CL = 8;
+constexpr int STEP_MAX_PIX = 4096;
+// Scalars are formed by one warp each: a float64 division is some twenty
+// instructions of 64 cycles, and every warp doing its own cost 4 us a step.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The sum over the cluster's CTAs of *slot, in a fixed order, for a whole warp (behind a cluster barrier).
+__device__ __forceinline__ double ranks_sum(const double* slot) {
+    uint32_t ra;
+    double x;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(ra)
+                 : "r"((uint32_t)__cvta_generic_to_shared(slot)), "r"(threadIdx.x & (STEP_CL - 1)));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(ra) : "memory");
+#pragma unroll
+    for (int d = 1; d < STEP_CL; d <<= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+    return x;
+}
+__global__ void __cluster_dims__(STEP_CL, 1, 1) __launch_bounds__(VT) k_pcg_step(const PcgArgs a) {
+    __shared__ double red[2][VT / 32], slot[3], scal[3];   // scal: pq, relres, r^T z
+    const int rhs = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const RhsState st0 = a.st[rhs];   // read before rank 0 updates it (behind the first cluster barrier)
+    if (!st0.active) return;          // the whole cluster
+    const int64_t off = (int64_t)rhs * a.n_pix;
+    double acc = 0.0;
+    PIX_LOOP(i) acc += dot3(a.p[off + i], load_q(a, off + i));
+    acc = warp_sum(acc);
+    if (lane == 0) red[0][warp] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < VT / 32; ++w) t += red[0][w];
+        slot[0] = t;
+    }
+    cluster_barrier();
+    __shared__ double s_alpha, s_beta;
+    __shared__ bool s_broken;
+    if (warp == 0) {
+        const double pq = ranks_sum(slot);
+        if (lane == 0) {
+            s_broken = !(pq > 0.0) || !isfinite(pq) || !isfinite(st0.rz);
+            s_alpha = s_broken ? 0.0 : st0.rz / pq;
+            scal[0] = pq;
+        }
+    }
+    __syncthreads();
+    const bool broken = s_broken;
+    const double alpha = s_alpha;
+    double rr = 0.0, rz = 0.0;
+    if (!broken) {
+        PIX_LOOP(i) {
+            const V4<double> pv = a.p[off + i];
+            const V4<double> qv = load_q(a, off + i);
+            V4<double> xv = a.x[off + i], rv = a.r[off + i];
+            xv.x += alpha * pv.x;
+            xv.y += alpha * pv.y;
+            xv.z += alpha * pv.z;
+            rv.x -= alpha * qv.x;
+            rv.y -= alpha * qv.y;
+            rv.z -= alpha * qv.z;
+            a.x[off + i] = xv;
+            a.r[off + i] = rv;
+            rr += dot3(rv, rv);
+            const V4<double> zv = bd_mul(bd_of(a, rhs, i), rv);
+            a.z[off + i] = zv;
+            rz += dot3(rv, zv);
+        }
+    }
+    rr = warp_sum(rr);
+    rz = warp_sum(rz);
+    if (lane == 0) {
+        red[0][warp] = rr;
+        red[1][warp] = rz;
+    }
+    __syncthreads();
+    if (lane == 0 && warp < 2) {
+        double t = 0.0;
+        for (int w = 0; w < VT / 32; ++w) t += red[warp][w];
+        slot[1 + warp] = t;
+    }
+    cluster_barrier();
+    if (warp == 0) {
+        const double t = ranks_sum(slot + 1);
+        if (lane == 0) scal[1] = broken ? st0.relres : sqrt(t) / st0.bnorm;
+    } else if (warp == 1) {
+        const double t = ranks_sum(slot + 2);
+        if (lane == 0) {
+            scal[2] = t;
+            s_beta = broken ? st0.beta : t / st0.rz;
+        }
+    }
+    __syncthreads();
+    RhsState st = st0;
+    st.pq = scal[0];
+    st.alpha = alpha;
+    if (broken) {
+        st.status = 6;
+        st.active = 0;
+    } else {
+        st.iters += 1;
+        st.relres = scal[1];
+        st.beta = s_beta;
+        st.rz = scal[2];
+        if (!isfinite(st.relres)) {
+            st.status = 6;
+            st.active = 0;
+        } else if (st.relres <= st.tol) {
+            st.active = 0;
+        } else if (st.iters >= st.max_iter) {
+            st.status = 5;
+            st.active = 0;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.st[rhs] = st;
+        if (a.ahist) a.ahist[(int64_t)rhs * a.hist_stride + st0.iters] = alpha;
+        if (!broken) {
+            a.hist[(int64_t)rhs * a.hist_stride + st.iters] = st.relres;
+            if (a.bhist) a.bhist[(int64_t)rhs * a.hist_stride + st.iters - 1] = st.beta;
+        }
+    }
+    if (st.active) {
+        PIX_LOOP(i) pcg_direction(a, off + i, st.beta);
+    }
+    cluster_barrier();   // no CTA leaves while another may still read its sums
 }
 
 // t = Z^T v for the k coarse vectors (one warp per coarse vector per pass),
@@ -863,6 +999,11 @@ void launch_pcg_init(const PcgArgs& a, const V4<double>* b, cudaStream_t s) {
 }
 void launch_pcg_src(const PcgArgs& a, int first, cudaStream_t s) {
     k_pcg_src<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, first);
+    count_launches(1);
+}
+bool pcg_step_fits(const PcgArgs& a) { return a.n_pix <= STEP_MAX_PIX; }
+void launch_pcg_step(const PcgArgs& a, cudaStream_t s) {
+    k_pcg_step<<<dim3(STEP_CL, a.nrhs), VT, 0, s>>>(a);
     count_launches(1);
 }
 void launch_pcg_pq(const PcgArgs& a, cudaStream_t s) {
