@@ -543,6 +543,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
             return MM_OK;
         }
     std::vector<Seg> segs;
+    segs.reserve((size_t)nrhs * (whole ? ctx->n_blocks + 1 : ctx->n_samples / std::max(1, V) + ctx->n_blocks + 1) + 2);
     const bool single = (variant == 2 && whole >= 2);   // segments one by one, not in pairs
     auto push = [&](const Seg& s) {
         if (!single && segs.size() % 2 == 1 && (segs.back().band != s.band || segs.back().shift != s.shift)) {

@@ -711,58 +711,6 @@ __device__ __forceinline__ void scatter_warp(int p, T c, T s, T z, V4<typename A
     scatter_vals<T>(p, z, z * c, z * s, q);
 }
 
-// Scatter of four consecutive outputs per lane: runs of equal pixels are
-// summed in registers first, a lane's leading run joins the previous lane's
-// trailing run when they share a pixel, runs strictly inside a lane's four
-// samples go out directly, and the trailing runs go through the
-// warp-segmented reduction.  Every output is counted once.
-template <typename T>
-__device__ __forceinline__ void scatter4_vals(const int (&p)[4], const T (&v0)[4], const T (&v1)[4],
-                                              const T (&v2)[4], V4<typename AccT<T>::type>* q) {
-    const unsigned FULL = 0xffffffffu;
-    const unsigned lane = threadIdx.x & 31u;
-    int kf = p[0], cur = p[0];
-    T f0 = v0[0], f1 = v1[0], f2 = v2[0];
-    T c0 = v0[0], c1 = v1[0], c2 = v2[0];
-    bool first_done = false;
-#pragma unroll
-    for (int j = 1; j < 4; ++j) {
-        if (p[j] == cur) {
-            c0 += v0[j];
-            c1 += v1[j];
-            c2 += v2[j];
-        } else {
-            if (!first_done) {
-                kf = cur;
-                f0 = c0;
-                f1 = c1;
-                f2 = c2;
-                first_done = true;
-            } else if (cur >= 0) {
-                atomic_add3(q + cur, c0, c1, c2);   // a run strictly inside the lane
-            }
-            cur = p[j];
-            c0 = v0[j];
-            c1 = v1[j];
-            c2 = v2[j];
-        }
-    }
-    const bool multi = first_done;
-    const int prev_last = __shfl_up_sync(FULL, cur, 1);
-    const bool give = multi && lane > 0 && kf == prev_last;
-    const T r0 = shfl_down_t(f0, 1);
-    const T r1 = shfl_down_t(f1, 1);
-    const T r2 = shfl_down_t(f2, 1);
-    const int rgive = __shfl_down_sync(FULL, (int)give, 1);
-    if (lane < 31 && rgive) {
-        c0 += r0;
-        c1 += r1;
-        c2 += r2;
-    }
-    if (multi && !give && kf >= 0) atomic_add3(q + kf, f0, f1, f2);
-    scatter_vals<T>(cur, c0, c1, c2, q);
-}
-
 // Pixel indices of four consecutive samples t0..t0+3 (a vector load past L1
 // when aligned); samples at or beyond the segment end come back flagged.
 __device__ __forceinline__ void load4_pix(const FilterArgs& a, int64_t t0, bool act, int count, int (&p)[4]) {
@@ -804,28 +752,6 @@ __device__ __forceinline__ void load4(const FilterArgs& a, int64_t t0, bool act,
     }
 }
 
-__device__ __forceinline__ void scatter4_f32(const FilterArgs& a, const Seg& S, bool act, int i0, const C2<float>* sm,
-                                             int lam, int L, bool imag, V4<float>* q) {
-    int p[4];
-    float ps[4];
-    const int64_t t0 = S.out0 + i0;
-    load4(a, t0, act, S.n_out - i0, p, ps);
-    float v0[4], v1[4], v2[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        float z = 0.0f, c = 0.0f, sn = 0.0f;
-        if (p[j] >= 0) {
-            const C2<float> v = sm[sidx(min(lam + i0 + j, L - 1))];
-            z = imag ? -v.y : v.x;
-            weights_from(a, t0 + j, ps[j], c, sn);
-        }
-        v0[j] = z;
-        v1[j] = z * c;
-        v2[j] = z * sn;
-    }
-    scatter4_vals(p, v0, v1, v2, q);
-}
-
 template <typename T>
 __device__ __forceinline__ void scatter_one(const FilterArgs& a, const Seg& S, bool act, int i, T zval) {
     int p = -1;
@@ -844,6 +770,113 @@ __device__ __forceinline__ void scatter_one(const FilterArgs& a, const Seg& S, b
 template <typename T>
 __device__ __forceinline__ bool seg_active(const FilterArgs& a, const Seg& S) {
     return S.n_out > 0 && (a.state == nullptr || a.state[S.rhs].active);
+}
+
+// cos 2psi, sin 2psi as -cos(2psi - pi), -sin(2psi - pi): __sincosf on [-pi, pi)
+__device__ __forceinline__ void neg_cs(float psi, float& nc, float& ns) {
+    __sincosf(fmaf(2.0f, psi, -3.14159265358979323846f), &ns, &nc);
+}
+
+// pix and psi of eight consecutive samples as one 256-bit load each (32-byte aligned)
+__device__ __forceinline__ void ld8_pointing(const int32_t* pp, const float* pf, int (&p)[8], float (&f)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]), "=r"(p[4]), "=r"(p[5]), "=r"(p[6]), "=r"(p[7])
+                 : "l"(pp));
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7])
+                 : "l"(pf));
+}
+
+// P^T of a warp's 256 consecutive outputs, eight per lane in order (real
+// samples z).  A raster that stays on a pixel for several samples gives a lane
+// at most two pixels, that of its first and that of its last sample: two sums
+// per lane, the first handed to the lane before it when that lane ends on the
+// same pixel (a lane on one pixel keeps its sum), then one atomic per pixel
+// left.  A warp with a lane that sees a third pixel (short runs, single flagged
+// samples) flushes every run of a lane from registers instead.  Every sample is
+// counted once.
+// weight(j, nc, ns) gives minus the pointing weights of sample j (formed where
+// they are used: arrays of sixteen would cost the transforms' kernels registers).
+template <typename W>
+__device__ __forceinline__ void warp_run8_scatter(const int (&p)[8], const float (&z)[8], V4<float>* q, W weight) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;   // the last sample's pixel
+    float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f;   // the first sample's, if it is another one
+    bool third = false;
+#pragma unroll
+    for (int j = 1; j < 7; ++j) third = third || (p[j] != p[0] && p[j] != p[7]);
+    bool two = p[0] != p[7];
+    if (!__any_sync(FULL, third)) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float nc, ns;
+            weight(j, nc, ns);
+            if (j == 7 || p[j] == p[7]) {
+                a0 += z[j];
+                a1 = fmaf(z[j], nc, a1);
+                a2 = fmaf(z[j], ns, a2);
+            } else {
+                b0 += z[j];
+                b1 = fmaf(z[j], nc, b1);
+                b2 = fmaf(z[j], ns, b2);
+            }
+        }
+    } else {
+        two = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j > 0 && p[j] != p[j - 1]) {
+                if (two && p[j - 1] >= 0) atomic_add3(q + p[j - 1], a0, -a1, -a2);
+                if (!two) {
+                    b0 = a0;
+                    b1 = a1;
+                    b2 = a2;
+                }
+                two = true;
+                a0 = a1 = a2 = 0.0f;
+            }
+            float nc, ns;
+            weight(j, nc, ns);
+            a0 += z[j];
+            a1 = fmaf(z[j], nc, a1);
+            a2 = fmaf(z[j], ns, a2);
+        }
+    }
+    const int plast = __shfl_up_sync(FULL, p[7], 1);
+    const bool give = two && lane > 0 && p[0] == plast;
+    const float r0 = __shfl_down_sync(FULL, b0, 1);
+    const float r1 = __shfl_down_sync(FULL, b1, 1);
+    const float r2 = __shfl_down_sync(FULL, b2, 1);
+    if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
+        a0 += r0;
+        a1 += r1;
+        a2 += r2;
+    }
+    if (two && !give && p[0] >= 0) atomic_add3(q + p[0], b0, -b1, -b2);
+    if (p[7] >= 0) atomic_add3(q + p[7], a0, -a1, -a2);
+}
+
+// The same with the angles.
+__device__ __forceinline__ void warp_run8_scatter_psi(const int (&p)[8], const float (&f)[8], const float (&z)[8],
+                                                      V4<float>* q) {
+    warp_run8_scatter(p, z, q, [&](int j, float& nc, float& ns) { neg_cs(f[j], nc, ns); });
+}
+
+// Pixel and angle of eight consecutive samples from i0 of a segment of n
+// (256-bit loads where aligned); samples from n on come back flagged.
+__device__ __forceinline__ void load8_pointing(const int32_t* pix, const float* psi, bool aligned, int i0, int n,
+                                               int (&p)[8], float (&f)[8]) {
+    if (aligned && i0 + 8 <= n) {
+        ld8_pointing(pix + i0, psi + i0, p, f);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const bool ok = i0 + j < n;
+            p[j] = ok ? __ldg(pix + i0 + j) : -1;
+            f[j] = ok ? __ldg(psi + i0 + j) : 0.0f;
+        }
+    }
 }
 
 // a + b c with one rounding where the type has a fused operation
@@ -964,14 +997,25 @@ __global__ void __launch_bounds__(NT, NT == 256 ? (sizeof(T) == 4 ? 3 : 2) : 1) 
     else fft_dit_conj<T>(s, tw, a.fp);
 
     if constexpr (std::is_same<T, float>::value) {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-        const int vmax = max(actA ? A.n_out : 0, actB ? B.n_out : 0);
-        V4<float>* qA = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)(actA ? A.rhs : 0) * a.n_pix;
-        V4<float>* qB = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)(actB ? B.rhs : 0) * a.n_pix;
-        for (int base = warp * 128; base < vmax; base += nwarp * 128) {
-            const int i0 = base + 4 * lane;
-            scatter4_f32(a, A, actA, i0, s, lam, L, false, qA);
-            scatter4_f32(a, B, actB, i0, s, lam, L, true, qB);
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const Seg& S = half ? B : A;
+            if (!(half ? actB : actA)) continue;
+            V4<float>* q = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)S.rhs * a.n_pix;
+#pragma unroll 1
+            for (int base = warp * 256; base < S.n_out; base += NT * 8) {
+                const int i0 = base + 8 * lane;
+                int p[8];
+                float f[8], z[8];
+                load8_pointing(a.pix + S.out0, a.psi + S.out0, (S.out0 & 7) == 0, i0, S.n_out, p, f);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const C2<float> v = s[sidx(min(lam + i0 + j, L - 1))];
+                    z[j] = half ? -v.y : v.x;
+                }
+                warp_run8_scatter_psi(p, f, z, q);
+            }
         }
     } else {
         scatter8_t<T, NT / 32>(a, A, actA, [&](int i) { return s[sidx(lam + i)].x; });
@@ -1056,11 +1100,6 @@ __device__ __forceinline__ void ld4_pointing(const int32_t* pp, const float* pf,
     asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(fv.x), "=f"(fv.y), "=f"(fv.z), "=f"(fv.w)
                  : "l"(pf));
-}
-
-// cos 2psi, sin 2psi as -cos(2psi - pi), -sin(2psi - pi): __sincosf on [-pi, pi)
-__device__ __forceinline__ void neg_cs(float psi, float& nc, float& ns) {
-    __sincosf(fmaf(2.0f, psi, -3.14159265358979323846f), &ns, &nc);
 }
 
 // y_t = I_p + Q_p cos 2psi + U_p sin 2psi (Sect. 2, Eq. datamodel), 0 for a flagged sample
@@ -1295,84 +1334,6 @@ __device__ __forceinline__ void half_gather_t(const FilterArgs& a, const Seg& S,
     }
 }
 
-// pix and psi of eight consecutive samples as one 256-bit load each (32-byte aligned)
-__device__ __forceinline__ void ld8_pointing(const int32_t* pp, const float* pf, int (&p)[8], float (&f)[8]) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]), "=r"(p[4]), "=r"(p[5]), "=r"(p[6]), "=r"(p[7])
-                 : "l"(pp));
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7])
-                 : "l"(pf));
-}
-
-// P^T of a warp's 256 consecutive outputs, eight per lane in order (real
-// samples z).  A raster that stays on a pixel for several samples gives a lane
-// at most two pixels, that of its first and that of its last sample: two sums
-// per lane, the first handed to the lane before it when that lane ends on the
-// same pixel (a lane on one pixel keeps its sum), then one atomic per pixel
-// left.  A warp with a lane that sees a third pixel (short runs, single flagged
-// samples) flushes every run of a lane from registers instead.  Every sample is
-// counted once.
-__device__ __forceinline__ void warp_run8_scatter(const int (&p)[8], const float (&f)[8], const float (&z)[8],
-                                                  V4<float>* q) {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;   // the last sample's pixel
-    float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f;   // the first sample's, if it is another one
-    bool third = false;
-#pragma unroll
-    for (int j = 1; j < 7; ++j) third = third || (p[j] != p[0] && p[j] != p[7]);
-    bool two = p[0] != p[7];
-    if (!__any_sync(FULL, third)) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float nc, ns;
-            neg_cs(f[j], nc, ns);
-            if (j == 7 || p[j] == p[7]) {
-                a0 += z[j];
-                a1 = fmaf(z[j], nc, a1);
-                a2 = fmaf(z[j], ns, a2);
-            } else {
-                b0 += z[j];
-                b1 = fmaf(z[j], nc, b1);
-                b2 = fmaf(z[j], ns, b2);
-            }
-        }
-    } else {
-        two = false;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (j > 0 && p[j] != p[j - 1]) {
-                if (two && p[j - 1] >= 0) atomic_add3(q + p[j - 1], a0, -a1, -a2);
-                if (!two) {
-                    b0 = a0;
-                    b1 = a1;
-                    b2 = a2;
-                }
-                two = true;
-                a0 = a1 = a2 = 0.0f;
-            }
-            float nc, ns;
-            neg_cs(f[j], nc, ns);
-            a0 += z[j];
-            a1 = fmaf(z[j], nc, a1);
-            a2 = fmaf(z[j], ns, a2);
-        }
-    }
-    const int plast = __shfl_up_sync(FULL, p[7], 1);
-    const bool give = two && lane > 0 && p[0] == plast;
-    const float r0 = __shfl_down_sync(FULL, b0, 1);
-    const float r1 = __shfl_down_sync(FULL, b1, 1);
-    const float r2 = __shfl_down_sync(FULL, b2, 1);
-    if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
-        a0 += r0;
-        a1 += r1;
-        a2 += r2;
-    }
-    if (two && !give && p[0] >= 0) atomic_add3(q + p[0], b0, -b1, -b2);
-    if (p[7] >= 0) atomic_add3(q + p[7], a0, -a1, -a2);
-}
-
 // After the conjugate-domain inverse, point m holds conj(z'_m):
 // y'_{2m} = Re, y'_{2m+1} = -Im.  Each warp takes 256 consecutive samples per
 // step, eight per lane.
@@ -1405,7 +1366,7 @@ __device__ __forceinline__ void half_scatter_f32(const FilterArgs& a, const Seg&
                 z[2 * j] = e.x;
                 z[2 * j + 1] = -e.y;
             }
-            warp_run8_scatter(p, f, z, q);
+            warp_run8_scatter_psi(p, f, z, q);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 p[j] = pn[j];
@@ -1426,7 +1387,7 @@ __device__ __forceinline__ void half_scatter_f32(const FilterArgs& a, const Seg&
             const C2<float> e = s[sidx(min(4 * u + j / 2, M - 1))];
             z[j] = (j & 1) ? -e.y : e.x;
         }
-        warp_run8_scatter(p, f, z, q);
+        warp_run8_scatter_psi(p, f, z, q);
     }
 }
 
@@ -1676,123 +1637,95 @@ __global__ void __launch_bounds__(NT, 2) k_filter_split(const FilterArgs a) {
     });
 }
 
-// ---------------- direct band variant, float32, four samples per thread ----------------
+// ---------------- direct band variant, float32, eight samples per thread ----------------
 // For narrow bands the product is gather + scatter bound: each thread owns
-// four consecutive outputs in both phases, so the pixel indices and pointing
-// weights loaded for the gather stay in registers for the scatter.  The
-// gathered y (with its lambda halo) is staged in shared memory for the band.
-template <bool FROM_TOD, int GPT, int LMAX>
-__global__ void __launch_bounds__(DIRECT_NT) k_filter_direct4(const FilterArgs a) {
+// eight consecutive outputs in both phases, so the pixel indices and pointing
+// weights loaded for the gather stay in registers for the scatter, whose runs
+// are summed in the thread (warp_run8_scatter).  The gathered y (with its
+// lambda halo) is staged in shared memory for the band, a register window of 8 +
+// 2 LMAX values per thread.  Bound by issue: 3.4e7 samples, lambda 16, the
+// product 187 us with four samples per thread and shuffled sums, 148 us now.
+template <bool FROM_TOD, int NT, int LMAX>
+__global__ void __launch_bounds__(NT) k_filter_direct8(const FilterArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int lam = a.lam;   // <= LMAX
     float* c = reinterpret_cast<float*>(smraw);                    // LMAX + 1 (zero beyond lam), padded to 4
-    float* y = c + ((LMAX + 1 + 3) & ~3);                          // [LMAX + 4*NT*GPT + LMAX], aligned to 16 B
+    float* y = c + ((LMAX + 1 + 3) & ~3);                          // [LMAX + 8 NT + LMAX], aligned to 16 B
+    const int i0 = 8 * threadIdx.x;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
         const Seg S = a.segs[2 * blockIdx.x + half];
         if (!seg_active<float>(a, S)) continue;   // uniform across the CTA
         const float* band = reinterpret_cast<const float*>(a.band) + (int64_t)S.band * (lam + 1);
-        for (int k = threadIdx.x; k <= LMAX; k += blockDim.x) c[k] = k <= lam ? band[k] : 0.0f;
+        for (int k = threadIdx.x; k <= LMAX; k += NT) c[k] = k <= lam ? band[k] : 0.0f;
         V4<float>* q = reinterpret_cast<V4<float>*>(a.dst) + (int64_t)S.rhs * a.n_pix;
-        const V4<float>* xm = reinterpret_cast<const V4<float>*>(a.src) + (int64_t)S.rhs * a.n_pix;
-        int p[GPT][4];
-        float cw[GPT][4], sw[GPT][4], yv[GPT][4];
-        // outputs of this thread: groups g = threadIdx.x + k * NT, samples out0 + 4g .. +3
+        const float4* xm = reinterpret_cast<const float4*>(a.src) + (int64_t)S.rhs * a.n_pix;
+        int p[8];
+        float nc[8], ns[8], z[8];
+        {
+            float f[8];
+            load8_pointing(a.pix + S.out0, a.psi + S.out0, (S.out0 & 7) == 0, i0, S.n_out, p, f);
 #pragma unroll
-        for (int k = 0; k < GPT; ++k) {
-            const int i0 = 4 * (threadIdx.x + k * DIRECT_NT);
-            float ps[4];
-            load4(a, S.out0 + i0, i0 < S.n_out, S.n_out - i0, p[k], ps);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                cw[k][j] = 0.0f;
-                sw[k][j] = 0.0f;
-                yv[k][j] = 0.0f;
-                if (p[k][j] >= 0) weights_from(a, S.out0 + i0 + j, ps[j], cw[k][j], sw[k][j]);
-            }
+            for (int j = 0; j < 8; ++j) neg_cs(f[j], nc[j], ns[j]);
         }
+        if (FROM_TOD) {
 #pragma unroll
-        for (int k = 0; k < GPT; ++k) {
-            const int i0 = 4 * (threadIdx.x + k * DIRECT_NT);
-            if (FROM_TOD) {
+            for (int j = 0; j < 8; ++j) {
+                const int64_t t = S.rhs * a.n_samples + S.out0 + i0 + j;
+                z[j] = i0 + j >= S.n_out ? 0.0f
+                       : a.tod_is_float ? __ldg(reinterpret_cast<const float*>(a.src) + t)
+                                        : (float)__ldg(reinterpret_cast<const double*>(a.src) + t);
+            }
+        } else {
+            float4 m[8];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (i0 + j < S.n_out)
-                        yv[k][j] = a.tod_is_float
-                                       ? __ldg(reinterpret_cast<const float*>(a.src) + S.rhs * a.n_samples + S.out0 + i0 + j)
-                                       : (float)__ldg(reinterpret_cast<const double*>(a.src) + S.rhs * a.n_samples + S.out0 + i0 + j);
-            } else {
-                V4<float> m[4];
+            for (int j = 0; j < 8; ++j) m[j] = __ldg(xm + max(p[j], 0));
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (p[k][j] >= 0) m[j] = ldmap<float>(xm + p[k][j]);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (p[k][j] >= 0) yv[k][j] = m[j].x + cw[k][j] * m[j].y + sw[k][j] * m[j].z;
+            for (int j = 0; j < 8; ++j) {
+                const float v = fmaf(-ns[j], m[j].z, fmaf(-nc[j], m[j].y, m[j].x));
+                z[j] = p[j] >= 0 ? v : 0.0f;
             }
         }
         if constexpr (LMAX > 0) {
             // stage y with its halo, then each thread slides over a register window
-#pragma unroll
-            for (int k = 0; k < GPT; ++k) {
-                const int i0 = 4 * (threadIdx.x + k * DIRECT_NT);
-                *reinterpret_cast<float4*>(y + LMAX + i0) = make_float4(yv[k][0], yv[k][1], yv[k][2], yv[k][3]);
-            }
+            float4* yv = reinterpret_cast<float4*>(y + LMAX + i0);
+            yv[0] = make_float4(z[0], z[1], z[2], z[3]);
+            yv[1] = make_float4(z[4], z[5], z[6], z[7]);
             __syncthreads();   // the right halo overlaps the stores of tile positions past the segment end
-            for (int h = threadIdx.x; h < 2 * LMAX; h += blockDim.x) {
+            for (int h = threadIdx.x; h < 2 * LMAX; h += NT) {
                 // left halo y[0 .. LMAX), right halo after the segment's outputs
                 const int i = h < LMAX ? h : LMAX + S.n_out + (h - LMAX);
                 const int64_t t = S.out0 - LMAX + i;
                 y[i] = (t >= S.lo && t < S.hi && (h < LMAX ? LMAX - h <= lam : h - LMAX < lam))
                            ? sample_value<float, FROM_TOD>(a, t, S.rhs) : 0.0f;
             }
-            // outputs inside the tile but past the segment end read zeros
-            for (int i = S.n_out + threadIdx.x; i < 4 * DIRECT_NT * GPT; i += blockDim.x)
-                if (i >= S.n_out + LMAX) y[LMAX + i] = 0.0f;
             __syncthreads();
-            float cr[LMAX + 1];
+            float w[8 + 2 * LMAX];
 #pragma unroll
-            for (int kk = 0; kk <= LMAX; ++kk) cr[kk] = c[kk];
+            for (int e = 0; e < (8 + 2 * LMAX) / 4; ++e) {
+                const float4 v = *reinterpret_cast<const float4*>(y + i0 + 4 * e);
+                w[4 * e] = v.x;
+                w[4 * e + 1] = v.y;
+                w[4 * e + 2] = v.z;
+                w[4 * e + 3] = v.w;
+            }
 #pragma unroll
-            for (int k = 0; k < GPT; ++k) {
-                const int i0 = 4 * (threadIdx.x + k * DIRECT_NT);
-                float w[4 + 2 * LMAX];
+            for (int j = 0; j < 8; ++j) z[j] = c[0] * w[LMAX + j];
 #pragma unroll
-                for (int e = 0; e < (4 + 2 * LMAX) / 4; ++e) {
-                    const float4 v = *reinterpret_cast<const float4*>(y + i0 + 4 * e);
-                    w[4 * e] = v.x;
-                    w[4 * e + 1] = v.y;
-                    w[4 * e + 2] = v.z;
-                    w[4 * e + 3] = v.w;
-                }
+            for (int kk = 1; kk <= LMAX; ++kk) {
+                const float ck = c[kk];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float z = cr[0] * w[LMAX + j];
-#pragma unroll
-                    for (int kk = 1; kk <= LMAX; ++kk) z += cr[kk] * (w[LMAX + j - kk] + w[LMAX + j + kk]);
-                    yv[k][j] = z;
-                }
+                for (int j = 0; j < 8; ++j) z[j] += ck * (w[LMAX + j - kk] + w[LMAX + j + kk]);
             }
         } else {
             __syncthreads();
-            const float c0 = c[0];
 #pragma unroll
-            for (int k = 0; k < GPT; ++k)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) yv[k][j] *= c0;
+            for (int j = 0; j < 8; ++j) z[j] *= c[0];
         }
-#pragma unroll
-        for (int k = 0; k < GPT; ++k) {
-            float v0[4], v1[4], v2[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float z = p[k][j] >= 0 ? yv[k][j] : 0.0f;
-                v0[j] = z;
-                v1[j] = z * cw[k][j];
-                v2[j] = z * sw[k][j];
-            }
-            scatter4_vals(p[k], v0, v1, v2, q);
-        }
+        warp_run8_scatter(p, z, q, [&](int j, float& c2, float& s2) {
+            c2 = nc[j];
+            s2 = ns[j];
+        });
         __syncthreads();
     }
 }
@@ -1968,25 +1901,24 @@ template <typename T, bool FROM_TOD>
 inline void launch_direct_t(const FilterArgs& a, cudaStream_t s) {
     if (a.n_work <= 0) return;
     if constexpr (std::is_same<T, float>::value) {
-        // lean kernel: tile = 4 * DIRECT_NT * GPT outputs, bands up to 16 taps each side
-        if ((a.V == 4 * DIRECT_NT * 2 || a.V == 4 * DIRECT_NT) && a.lam <= 16) {
-            const int gpt = a.V / (4 * DIRECT_NT);
+        // lean kernel: tiles of 1024 or 2048 outputs, eight per thread, bands up to 16 taps each side
+        if ((a.V == 1024 || a.V == 2048) && a.lam <= 16) {
             const int lmax = a.lam == 0 ? 0 : (a.lam <= 4 ? 4 : (a.lam <= 8 ? 8 : 16));
             const size_t sm = (size_t)(((lmax + 1 + 3) & ~3) + a.V + 2 * lmax + 4) * sizeof(float);
             auto go = [&](auto kern) {
-                kern<<<a.n_work, DIRECT_NT, sm, s>>>(a);
+                kern<<<a.n_work, a.V / 8, sm, s>>>(a);
                 count_launches(1);
             };
-            if (gpt == 2) {
-                if (lmax == 0) go(k_filter_direct4<FROM_TOD, 2, 0>);
-                else if (lmax == 4) go(k_filter_direct4<FROM_TOD, 2, 4>);
-                else if (lmax == 8) go(k_filter_direct4<FROM_TOD, 2, 8>);
-                else go(k_filter_direct4<FROM_TOD, 2, 16>);
+            if (a.V == 2048) {
+                if (lmax == 0) go(k_filter_direct8<FROM_TOD, 256, 0>);
+                else if (lmax == 4) go(k_filter_direct8<FROM_TOD, 256, 4>);
+                else if (lmax == 8) go(k_filter_direct8<FROM_TOD, 256, 8>);
+                else go(k_filter_direct8<FROM_TOD, 256, 16>);
             } else {
-                if (lmax == 0) go(k_filter_direct4<FROM_TOD, 1, 0>);
-                else if (lmax == 4) go(k_filter_direct4<FROM_TOD, 1, 4>);
-                else if (lmax == 8) go(k_filter_direct4<FROM_TOD, 1, 8>);
-                else go(k_filter_direct4<FROM_TOD, 1, 16>);
+                if (lmax == 0) go(k_filter_direct8<FROM_TOD, 128, 0>);
+                else if (lmax == 4) go(k_filter_direct8<FROM_TOD, 128, 4>);
+                else if (lmax == 8) go(k_filter_direct8<FROM_TOD, 128, 8>);
+                else go(k_filter_direct8<FROM_TOD, 128, 16>);
             }
             return;
         }

@@ -128,3 +128,23 @@ def test_float64_block_split_over_two_ctas(L, pixels, nx):
         maps.append(m[0])
         c.close()
     assert_close(maps[0], maps[1], 1e-7)
+
+
+@pytest.mark.parametrize("lam", [0, 3, 4, 8, 9, 16])
+@pytest.mark.parametrize("tile", [1024, 2048])
+@pytest.mark.parametrize("pixels,nx", [("raster", 16), ("random", 8), ("steps", 16)])
+def test_narrow_bands_of_every_fill(lam, tile, pixels, nx):
+    """The direct filter's eight outputs per thread: every padded band width, tiles that end inside a
+    thread's outputs or inside the halo, blocks shorter than the halo; 1e-5."""
+    scan = scan_with([2048, 1, 2, 7, 8, 9, 15, 17, 1023, 1025, 2047, 2049, 4099, 64], pixels, nx, lam + nx)
+    scan.band = np.stack([synth.scan.toeplitz_band(lam, 1.0)])
+    c = MM.Context(0, None, MM.MM_FP32_MIXED)
+    c.set_option("filter", 1)
+    c.set_option("direct_tile", tile)
+    c.setup_scan(scan)
+    x = np.random.default_rng(tile).standard_normal((2, scan.n_pix, 3))
+    y = c.apply_A(x)
+    prob = O.Problem.from_scan(scan)
+    for r in range(2):
+        assert_close(y[r], O.apply_A(prob, x[r]), TOL32)
+    c.close()
