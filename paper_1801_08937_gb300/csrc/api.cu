@@ -429,20 +429,30 @@ mm_status band_spectra_dev(mm_ctx* ctx, int N, DevBuf& H) {
     CK(H.ensure(all * 8));
     CK(ctx->w_tw64.ensure((size_t)N * 16));
     launch_twiddles64(ctx->w_tw64.as<double2>(), N, ctx->stream);
-    if ((double)ctx->n_bands * ctx->lam * (N / 2) < 1.5e8) {
-        launch_band_cosines(ctx->d_band64.as<double>(), ctx->lam, ctx->n_bands, N, ctx->w_tw64.as<double2>(),
-                            H.as<double>(), ctx->stream);
-        CKL();
-        return MM_OK;
-    }
+    const bool cosines = (double)ctx->n_bands * ctx->lam * (N / 2) < 1.5e8;
+    // Many bands go in groups: a grid holds 65535 rows, and the transforms' scratch (about 33 bytes a point) stays
+    // within 256 MB.
+    const int group = cosines ? 8 * 65535 : std::max(1, std::min(65535, (1 << 28) / (33 * N)));
+    const size_t wide = (size_t)std::min(group, ctx->n_bands) * (N + (N >> 4));
     DevBuf h, Hp, work;
-    CK(h.ensure(all * 8));
-    CK(Hp.ensure(all * 8));
-    CK(work.ensure((size_t)ctx->n_bands * (N + (N >> 4)) * 16));
-    launch_band_circle(ctx->d_band64.as<double>(), ctx->lam, ctx->n_bands, N, h.as<double>(), ctx->stream);
-    launch_fft_spectrum(h.as<double>(), Hp.as<double>(), work.as<double2>(), ctx->w_tw64.as<double2>(), ctx->n_bands, fpN,
-                        ctx->stream);
-    launch_spectrum_order(Hp.as<double>(), H.as<double>(), ctx->n_bands, fpN, ctx->stream);
+    if (!cosines) {
+        CK(h.ensure(wide * 8));
+        CK(Hp.ensure(wide * 8));
+        CK(work.ensure(wide * 16));
+    }
+    for (int b0 = 0; b0 < ctx->n_bands; b0 += group) {
+        const int nb = std::min(group, ctx->n_bands - b0);
+        const double* band = ctx->d_band64.as<double>() + (size_t)b0 * (ctx->lam + 1);
+        double* out = H.as<double>() + (size_t)b0 * N;
+        if (cosines) {
+            launch_band_cosines(band, ctx->lam, nb, N, ctx->w_tw64.as<double2>(), out, ctx->stream);
+        } else {
+            launch_band_circle(band, ctx->lam, nb, N, h.as<double>(), ctx->stream);
+            launch_fft_spectrum(h.as<double>(), Hp.as<double>(), work.as<double2>(), ctx->w_tw64.as<double2>(), nb, fpN,
+                                ctx->stream);
+            launch_spectrum_order(Hp.as<double>(), out, nb, fpN, ctx->stream);
+        }
+    }
     CKL();
     return MM_OK;   // the buffers' release waits for the kernels
 }
@@ -619,6 +629,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
         ctx->have_csdf = true;
     }
     if (f64 == 1) TRY(ensure_weights64(ctx));
+    if (ctx->w_spec.bytes > (size_t)1 << 28) ctx->w_spec.release();   // many bands: not kept beside the plan's own tables
     ctx->plans.push_back(std::move(p));
     *out = ctx->plans.back().get();
     return MM_OK;

@@ -230,11 +230,12 @@ __global__ void k_plan_twiddles(const FftPasses fp, void* tw, void* twp, int64_t
 }
 // Spectrum of a two-segment plan: position p holds H at its frequency.
 template <int KIND>
-__global__ void k_plan_spectrum(const double* __restrict__ S, const FftPasses fp, void* H) {
+__global__ void k_plan_spectrum(const double* __restrict__ S, const FftPasses fp, int n_bands, void* H) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= fp.L) return;
     const int k = dif_freq(fp, p);
-    Tab<KIND>::put(H, (int64_t)blockIdx.y * fp.L + p, S[(int64_t)blockIdx.y * fp.L + min(k, fp.L - k)]);
+    for (int64_t b = blockIdx.y; b < n_bands; b += gridDim.y)
+        Tab<KIND>::put(H, b * fp.L + p, S[b * fp.L + min(k, fp.L - k)]);
 }
 // Index tables of a half-length plan (one CTA).  Pairs (k, M - k), k = 0 ..
 // M/2, in the order of the position of k: neighbouring threads then touch
@@ -353,8 +354,6 @@ __global__ void __launch_bounds__(256) k_block_windows(const int32_t* __restrict
                                                        int n_pix, int2* win, int* bad) {
     const int b = blockIdx.x;
     const int64_t o1 = off[b + 1];
-    const int64_t t0 = off[b] + (int64_t)blockIdx.y * WIN_SLICE, t1 = t0 + WIN_SLICE < o1 ? t0 + WIN_SLICE : o1;
-    if (t0 >= t1) return;
     int lo = 0x7fffffff, hi = -1;
     bool ok = true;
     auto take = [&](int p) {
@@ -362,15 +361,18 @@ __global__ void __launch_bounds__(256) k_block_windows(const int32_t* __restrict
         if (p >= 0) lo = min(lo, p);
         hi = max(hi, p);
     };
-    int64_t t = t0 + threadIdx.x;
-    for (; t + 3 * 256 < t1; t += 4 * 256) {
-        int p[4];
+    for (int64_t t0 = off[b] + (int64_t)blockIdx.y * WIN_SLICE; t0 < o1; t0 += (int64_t)gridDim.y * WIN_SLICE) {
+        const int64_t t1 = t0 + WIN_SLICE < o1 ? t0 + WIN_SLICE : o1;
+        int64_t t = t0 + threadIdx.x;
+        for (; t + 3 * 256 < t1; t += 4 * 256) {
+            int p[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) p[j] = __ldg(pix + t + j * 256);
+            for (int j = 0; j < 4; ++j) p[j] = __ldg(pix + t + j * 256);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) take(p[j]);
+            for (int j = 0; j < 4; ++j) take(p[j]);
+        }
+        for (; t < t1; t += 256) take(__ldg(pix + t));
     }
-    for (; t < t1; t += 256) take(__ldg(pix + t));
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     if ((threadIdx.x & 31) == 0 && hi >= 0) {
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(256) k_block_windows(const int32_t* __restrict
 void launch_block_windows(const int32_t* pix, const int64_t* block_off, int n_blocks, int64_t max_block, int n_pix,
                           int2* win, int* bad, cudaStream_t s) {
     k_window_init<<<(n_blocks + 255) / 256, 256, 0, s>>>(win, n_blocks);
-    k_block_windows<<<dim3(n_blocks, (unsigned)((max_block + WIN_SLICE - 1) / WIN_SLICE)), 256, 0, s>>>(
+    k_block_windows<<<dim3(n_blocks, (unsigned)std::min<int64_t>(65535, (max_block + WIN_SLICE - 1) / WIN_SLICE)), 256, 0, s>>>(
         pix, block_off, n_pix, win, bad);
     count_launches(2);
 }
@@ -422,7 +424,7 @@ void launch_spectrum_order(const double* Hp, double* H, int n_bands, const FftPa
 template <int KIND>
 static void plan_tables(const double* S, int n_bands, const FftPasses& fp, void* tw, void* H, cudaStream_t s) {
     k_plan_twiddles<KIND><<<(fp.L + 255) / 256, 256, 0, s>>>(fp, tw, nullptr, 0);
-    k_plan_spectrum<KIND><<<dim3((fp.L + 255) / 256, n_bands), 256, 0, s>>>(S, fp, H);
+    k_plan_spectrum<KIND><<<dim3((fp.L + 255) / 256, std::min(n_bands, 64)), 256, 0, s>>>(S, fp, n_bands, H);
     count_launches(2);
 }
 void launch_plan_tables(const double* S, int n_bands, const FftPasses& fp, int kind, void* tw, void* H, cudaStream_t s) {

@@ -87,3 +87,22 @@ def test_spectra_of_few_and_many_bands(n_bands):
     assert_close(c.apply_A(x)[0], O.apply_A(O.Problem.from_scan(scan), x), 1e-5)
     assert (1e8 > n_bands * lam * 9216) == (n_bands == 1)
     c.close()
+
+
+@pytest.mark.parametrize("n_bands,length,lam,n_fft", [(5600, 1024, 256, 1536), (70000, 16, 2, 256)])
+@pytest.mark.parametrize("half", [0, 2])
+def test_tables_of_very_many_bands(n_bands, length, lam, n_fft, half):
+    """A band per block: more bands than one group of transforms (2^28 / (33 * 1536) = 5295) and than the
+    65535 rows of a grid; float64, 1e-11."""
+    scan = odd_scan("random", [length] * n_bands, "hwp", 3)
+    rng = np.random.default_rng(4)
+    scan.band = rng.standard_normal((n_bands, lam + 1)) * np.exp(-np.arange(lam + 1) / (lam / 4 + 1))
+    scan.block_band = np.arange(n_bands, dtype=np.int32)
+    c = MM.Context(0, None, MM.MM_FP64)
+    c.set_option("filter", 2)
+    c.set_option("half_transform", half)
+    c.set_option("fft_len", n_fft)
+    c.setup_scan(scan)
+    x = rng.standard_normal((scan.n_pix, 3))
+    assert_close(c.apply_A(x)[0], O.apply_A(O.Problem.from_scan(scan), x), TOL)
+    c.close()
