@@ -31,8 +31,7 @@
 
 namespace mm {
 
-// Threads per block: the float64 and double-float timelines of long blocks fill
-// an SM's shared memory, so one block of 32 warps; float32 ones share it.
+// Most threads per block (tmpl_threads picks).
 template <typename T> struct TmplThreads { static constexpr int value = sizeof(T) == 4 ? 512 : 1024; };
 
 // Place of sample i in the block's shared timeline: permuted within groups of
@@ -110,7 +109,7 @@ __device__ __forceinline__ df mulf(df a, float f) {
 constexpr int POLY_UNITS = 64;   // units of one round of the parts' shared sums
 template <typename T, int K>
 __device__ void project_poly(T* y, T (*part)[4], const TmplArgs& t, int blk, int64_t b0) {
-    constexpr int nw = TmplThreads<T>::value / 32;
+    const int nw = blockDim.x >> 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sb0 = t.blk_sub[blk], sb1 = t.blk_sub[blk + 1];
     const int parts = sb1 - sb0 >= 2 * nw ? 1 : (sb1 - sb0 >= nw ? 2 : (sb1 - sb0 >= nw / 2 ? 4 : 6));
@@ -313,7 +312,7 @@ __device__ __forceinline__ void bin_sums8(const int (&g)[8], const T (&v)[8], Ac
 
 template <typename T, bool FROM_TOD, int K, int ST>
 __global__ void __launch_bounds__(TmplThreads<T>::value) k_filter_tmpl(const FilterArgs a, const TmplArgs t) {
-    constexpr int TMPL_NT = TmplThreads<T>::value;
+    const int TMPL_NT = blockDim.x;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int blk = blockIdx.x, rhs = blockIdx.y;
     if (a.state && !a.state[rhs].active) return;
@@ -488,6 +487,22 @@ size_t tmpl_smem_bytes(int64_t max_block, int n_bins, bool f64) {
     return (size_t)((max_block + 1) & ~1LL) * e + (size_t)n_bins * (e + 4);
 }
 
+// Threads of a CTA.  At 64 registers an SM holds 1024 threads of the 8-byte
+// types, in as many CTAs as the blocks' timelines leave shared memory for:
+// several small CTAs hide one another's barriers and serial parts.  Double-float,
+// order 1 + ground, ms with 256 / 512 / 1024 threads: blocks of 16384 (one CTA
+// fits) 1.199 / 0.887 / 0.825, of 12000 (two) 0.095 / 0.093 / 0.124, of 8192
+// 0.155 / 0.160 / 0.223; order 3, blocks of 4096 0.094 / 0.114 / 0.156; 24 blocks
+// of 7000, fewer than SMs, 0.054 / 0.049 / 0.050.  Native float64 is bound by the
+// float64 pipe, which few warps keep busy: blocks of 16384 0.296 / 0.292 / 0.380,
+// of 8192 0.339 / 0.398 / 0.529, 24 blocks of 7000 0.087 / 0.093 / 0.117.
+template <typename T> static int tmpl_threads(size_t smem, int64_t ctas) {
+    if (sizeof(T) == 4) return 512;
+    const size_t fit = (228 * 1024) / (smem + 2048);
+    if (std::is_same<T, double>::value) return fit >= 2 ? 256 : 512;
+    return fit < 2 ? 1024 : (fit == 2 || ctas <= 152 ? 512 : 256);
+}
+
 template <typename T, bool FROM_TOD, int K, int ST>
 static void launch_tmpl_ks(const FilterArgs& a, const TmplArgs& t, int nrhs, cudaStream_t s) {
     const size_t sm = tmpl_smem_bytes(t.max_block, t.n_bins, sizeof(T) == 8) + 64;   // whole groups of eight samples
@@ -495,7 +510,8 @@ static void launch_tmpl_ks(const FilterArgs& a, const TmplArgs& t, int nrhs, cud
     raise_smem_once(configured, sm, [](size_t v) {
         cudaFuncSetAttribute(k_filter_tmpl<T, FROM_TOD, K, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
     });
-    k_filter_tmpl<T, FROM_TOD, K, ST><<<dim3(t.n_blocks, nrhs), TmplThreads<T>::value, sm, s>>>(a, t);
+    const int threads = tmpl_threads<T>(sm, t.n_blocks * (int64_t)nrhs);
+    k_filter_tmpl<T, FROM_TOD, K, ST><<<dim3(t.n_blocks, nrhs), threads, sm, s>>>(a, t);
     count_launches(1);
 }
 template <typename T, bool FROM_TOD, int K>

@@ -816,6 +816,7 @@ __global__ void __cluster_dims__(STEP_CL, 1, 1) __launch_bounds__(VT) k_pcg_step
 
 // t = Z^T v for the k coarse vectors (one warp per coarse vector per pass),
 // then u = E^-1 t in the last CTA.
+template <bool F32>
 __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
     const int rhs = blockIdx.y;
     if (a.st && !a.st[rhs].active) return;
@@ -827,9 +828,9 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
     const int i0 = blockIdx.x * chunk, i1 = min(a.n_pix, i0 + chunk);
     // float32: the residual of the chunk is converted once and shared by the warps (each coarse vector's warp
     // converted it anew: 32 -> 14 us at 65536 pixels, k = 32)
-    constexpr int STAGE = 1024;
+    constexpr int STAGE = F32 ? 1024 : 1;
     __shared__ float vx[3][STAGE];
-    const bool staged = a.Z32 && chunk <= STAGE;
+    const bool staged = F32 && chunk <= STAGE;
     if (staged) {
         for (int i = i0 + threadIdx.x; i < i1; i += VT) {
             const V4<double> x = v[off + i];
@@ -850,7 +851,7 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
                 sf = fmaf(z.x, vx[0][i - i0], fmaf(z.y, vx[1][i - i0], fmaf(z.z, vx[2][i - i0], sf)));
             }
             s = f2d_exact(sf);
-        } else if (a.Z32) {
+        } else if (F32) {
             // float32 products summed per lane in float32 (a few dozen terms), the lanes in float64
             const V4<float>* zc = a.Z32 + (int64_t)c * a.n_pix;
             float sf = 0.0f;
@@ -887,6 +888,8 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
 
 // out = M_BD (v - AZ u) + Z u  (Sect. 3.2, Eq. m2l); with finalize_beta >= 0
 // it also forms v^T out and updates rz/beta like k_bd_dot.
+// G lanes per pixel, each 1/G of the coarse vectors.
+template <int G>
 __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* out, int finalize_beta) {
     const int rhs = blockIdx.y;
     if (a.st && !a.st[rhs].active) return;
@@ -900,19 +903,17 @@ __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* ou
     __syncthreads();
     double acc[1] = {0.0};
     const V4<double>* AZ = a.AZ + (int64_t)rhs * a.az_stride;
-    // four lanes per pixel, each a quarter of the coarse vectors: a small map still fills the SMs' float64 pipes
-    // and the loads of a pixel's vectors are in flight together
-    const int g = threadIdx.x & 3;
-    for (int base = blockIdx.x * (VT / 4); base < a.n_pix; base += gridDim.x * (VT / 4)) {
-        const int i = base + (threadIdx.x >> 2);
+    const int g = threadIdx.x % G;
+    for (int base = blockIdx.x * (VT / G); base < a.n_pix; base += gridDim.x * (VT / G)) {
+        const int i = base + threadIdx.x / G;
         const bool in = i < a.n_pix;
         double yx = 0.0, yy = 0.0, yz = 0.0, zx = 0.0, zy = 0.0, zz = 0.0;
         if (in) {
             if (a.Z32) {
                 // the coarse sums AZ u and Z u in float32 (mixed precision), the rest in float64
                 float fx = 0.0f, fy = 0.0f, fz = 0.0f, hx = 0.0f, hy = 0.0f, hz = 0.0f;
-#pragma unroll 4
-                for (int c = g; c < a.k; c += 4) {
+#pragma unroll(G == 1 ? 8 : 4)
+                for (int c = g; c < a.k; c += G) {
                     const V4<float> azc = a.AZ32[(int64_t)c * a.n_pix + i];
                     const V4<float> zc = a.Z32[(int64_t)c * a.n_pix + i];
                     const float uc = uf[c];
@@ -931,7 +932,7 @@ __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* ou
                 zz = f2d_exact(hz);
             } else {
 #pragma unroll 4
-                for (int c = g; c < a.k; c += 4) {
+                for (int c = g; c < a.k; c += G) {
                     const V4<double> azc = AZ[(int64_t)c * a.n_pix + i];
                     const V4<double> zc = a.Z[(int64_t)c * a.n_pix + i];
                     const double uc = u[c];
@@ -945,7 +946,7 @@ __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* ou
             }
         }
 #pragma unroll
-        for (int d = 1; d < 4; d <<= 1) {
+        for (int d = 1; d < G; d <<= 1) {
             yx += __shfl_xor_sync(0xffffffffu, yx, d);
             yy += __shfl_xor_sync(0xffffffffu, yy, d);
             yz += __shfl_xor_sync(0xffffffffu, yz, d);
@@ -1024,15 +1025,29 @@ void launch_precond_bd_dot(const PcgArgs& a, int finalize_beta, cudaStream_t s) 
     k_bd_dot<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, finalize_beta);
     count_launches(1);
 }
-// CTAs of k_m2l_ztr: a small map is cut into 64-pixel chunks so that its k vectors spread over more SMs (the
-// partials then hold this many entries per value).
+// CTAs of k_m2l_ztr at most (the partials hold this many entries per value).
 int m2l_ztr_grid(int n_pix) { return std::min(304, (n_pix + 63) / 64); }
+// A small map is cut into chunks down to 64 pixels, so that its k vectors spread over more SMs, until all
+// right-hand sides together have 304 CTAs; from there on chunks of 256, whose warp sums weigh less (64 right-hand
+// sides, 10^4 pixels, k = 8, float64: 325 us a call in chunks of 64 with four lanes a pixel below, 208 so).
+static int m2l_grid(int n_pix, int nrhs) {
+    return std::min(304, std::max((n_pix + VT - 1) / VT, std::min((n_pix + 63) / 64, 304 / std::max(1, nrhs))));
+}
 void launch_m2l_ztr(const PcgArgs& a, const V4<double>* v, cudaStream_t s) {
-    k_m2l_ztr<<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v);
+    const dim3 grid(m2l_grid(a.n_pix, a.nrhs), a.nrhs);
+    if (a.Z32) k_m2l_ztr<true><<<grid, VT, 0, s>>>(a, v);
+    else k_m2l_ztr<false><<<grid, VT, 0, s>>>(a, v);
     count_launches(1);
 }
+// Four lanes per pixel while they all fit on the device at once (152 x 2048 threads): a small map still fills the
+// SMs' float64 pipes and the loads of a pixel's vectors are in flight together.  Beyond that one lane per pixel
+// spares the lanes' sums, which are float64 adds (8 right-hand sides of 14400 pixels, k = 64: 268 -> 244 us a call with
+// the chunks above; 90000 pixels, k = 32, alone: 142 and 141).
 void launch_m2l_apply(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, cudaStream_t s) {
-    k_m2l_apply<<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+    if ((int64_t)a.n_pix * a.nrhs <= 152 * 2048 / 4)
+        k_m2l_apply<4><<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+    else
+        k_m2l_apply<1><<<dim3(std::min(304, (a.n_pix + VT - 1) / VT), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
     count_launches(1);
 }
 

@@ -69,3 +69,20 @@ def test_tensor_core_path_reads_and_writes_three_wide_maps(nx, nrhs, k):
         c.apply_precond(MM.MM_PRECOND_2L, xs, out=ys)
         assert_close(ys.cpu().numpy().reshape(-1, 3), ref.reshape(-1, 3), 2e-5)
     c.close()
+
+
+@pytest.mark.parametrize("k", [1, 13])
+def test_batch_past_four_lanes_a_pixel(k):
+    """40 right-hand sides of 2304 pixels (one lane a pixel, chunks of 256) against each alone (four lanes,
+    chunks of 64): the same sums in another order, E's condition below 1e4."""
+    scan = synth.make_scan(nx=48, ny=48, n_det=2, n_t=40 * 2304, n_int=2, half_bw=16, f_knee=1.0, seed=8)
+    c = MM.Context(0, None, MM.MM_FP64)
+    c.setup_scan(scan)
+    assert c.build_bd(1e-6) == 0
+    rng = np.random.default_rng(k)
+    c.set_coarse(rng.standard_normal((k, scan.n_pix, 3)))
+    x = rng.standard_normal((40, scan.n_pix, 3))
+    y = c.apply_precond(MM.MM_PRECOND_2L, x)
+    for r in (0, 17, 39):
+        assert_close(y[r], c.apply_precond(MM.MM_PRECOND_2L, x[r:r + 1])[0], 1e-9)
+    c.close()

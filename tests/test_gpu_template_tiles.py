@@ -46,3 +46,24 @@ def test_every_subscan_and_bin_length(prec, order, stokes, bins):
     for r in range(2):
         assert_close(y[r], O.apply_A_T(tp, x[r]), 1e-5 if prec == "f32" else 1e-11)
     c.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "df"])
+@pytest.mark.parametrize("block,n_blocks", [(16384, 2), (12000, 3), (1024, 8), (1000, 160)])
+def test_every_thread_count(prec, block, n_blocks):
+    """Blocks of which an SM holds one, two or many, fewer and more of them than SMs."""
+    rng = np.random.default_rng(12)
+    n = block * n_blocks
+    s = synth.make_scan(nx=9, ny=9, n_det=1, n_t=n, n_int=n_blocks, half_bw=0, f_knee=0.0, seed=6, hwp=False)
+    s.psi[:] = rng.uniform(0, np.pi, n).astype(np.float32)
+    sub = np.unique(np.concatenate([s.block_off, np.arange(0, n, 397)])).astype(np.int64)
+    az = (np.arange(n) // 50 % 23).astype(np.int32)
+    tp = O.TemplateProblem(s.pix, s.psi, s.block_off, s.band[s.block_band, 0], s.n_pix, sub, 1, az, 23, 1)
+    c = MM.Context(0, None, MM.MM_FP64)
+    c.setup_scan(s)
+    c.set_templates(1, sub, az, 23, 1)
+    if prec == "df":
+        c.set_option("fp64_products", 2)
+    x = rng.standard_normal((s.n_pix, 3))
+    assert_close(c.apply_A(x)[0], O.apply_A_T(tp, x), 1e-11)
+    c.close()
