@@ -168,11 +168,18 @@ def fft_passes(L):
     return rs
 
 
-# real flops per point of one pass (butterfly + pass twiddles), as the kernel computes them
+# real flops per point of one pass (butterfly + pass twiddles), as the kernel computes them; the
+# three-pass kernel's radix 9 is its last pass and has no twiddles
 FLOPS_PER_POINT = {16: 266 / 16, 9: 168 / 9, 8: 102 / 8, 4: 34 / 4, 3: 28 / 3, 2: 10 / 2}
 
 
-def fft_flops_per_point(L):
+# passes of the float32 whole-block transforms of these many complex points
+THREE_PASS = {9216: [32, 32, 9], 4608: [32, 16, 9], 2304: [16, 16, 9]}
+
+
+def fft_flops_per_point(L, three=False):
+    if three:
+        return sum({32: 674 / 32, 16: 266 / 16, 9: 120 / 9}[r] for r in THREE_PASS[L])
     return sum(FLOPS_PER_POINT[r] for r in fft_passes(L))
 
 
@@ -473,11 +480,11 @@ def main():
     whole = int(ctx.get_option("plan_whole"))
     lam = scan.half_bw
     n_work = 0
-    T = L // 2 if whole == 2 else L          # complex points per transform
+    T = L // 2 if whole >= 2 else L          # complex points per transform
     if L:
         blen = scan.n_t // scan.n_int
         segs_per_block = 1 if whole else -(-blen // (L - 2 * lam))
-        n_work = scan.n_blocks if whole == 2 else -(-(scan.n_blocks * segs_per_block) // 2)
+        n_work = scan.n_blocks if whole >= 2 else -(-(scan.n_blocks * segs_per_block) // 2)
     xin = torch.randn((1, scan.n_pix, 3), dtype=torch.float64, device=dev)
     yout = torch.empty_like(xin)
     for _ in range(3):
@@ -491,7 +498,8 @@ def main():
     ctx.set_option("time_filter", 0)
     # forward + inverse transform, plus the spectrum step (2 flop per point; 8 per point for the
     # paired real-spectrum step of half-length transforms)
-    flops_per_launch = n_work * (2 * fft_flops_per_point(T) * T + (8 if whole == 2 else 2) * T) if L else 0.0
+    three = whole == 2 and prec == M.MM_FP32_MIXED and T in THREE_PASS
+    flops_per_launch = n_work * (2 * fft_flops_per_point(T, three) * T + (8 if whole >= 2 else 2) * T) if L else 0.0
     bytes_per_launch = 8.0 * scan.n_samples
     peaks = {}
     try:
@@ -522,11 +530,12 @@ def main():
                 "traffic_note": ("dram__bytes_read.sum + dram__bytes_write.sum per sample from one ncu capture "
                                  "(16-detector cut), scaled by samples to this launch") if traffic else None,
                 "kernel": "%s<%s> (gather + FFT Toeplitz + scatter)"
-                          % ("k_filter_half" if whole == 2 else "k_filter_fft",
+                          % ("k_filter_half3" if three else "k_filter_half" if whole == 2 else
+                             "k_filter_split" if whole == 3 else "k_filter_fft",
                              "float" if prec == M.MM_FP32_MIXED else "double"),
                 "avg_launch_ms": ax_ms, "fft_len": L,
-                "fft_radices": fft_passes(T) if L else None, "whole_blocks": bool(whole),
-                "half_length_transform": whole == 2,
+                "fft_radices": (THREE_PASS[T] if three else fft_passes(T)) if L else None, "whole_blocks": bool(whole),
+                "half_length_transform": whole >= 2,
                 "alu_view": {"achieved_tflops": achieved_tf, "peak_tflops": alu_peak,
                              "frac": achieved_tf / alu_peak if alu_peak else None,
                              "flops_per_launch": flops_per_launch,
