@@ -304,8 +304,11 @@ mm_status mm_solve(mm_ctx* ctx, const void* tod, double* map_out, int32_t nrhs,
  * in high and low parts, about 21 bits) when 8 <= nrhs <= 128, k <= 64, the
  * right-hand sides share one coarse space and the map has at least 16384
  * pixels (smaller maps are faster in float64 on the CUDA cores); 2 does so
- * for every eligible batch whatever the map size; 0 keeps them in float64.  A bounded wait of the tensor-core kernels that gives up is
- * reported as MM_ERR_TIMEOUT.  Errors: MM_ERR_ARG for an unknown name or
+ * for every eligible batch whatever the map size; 0 keeps them in float64;
+ * "wait_limit_ns": how long the float32 whole-block filter waits for a copy
+ * to shared memory, in nanoseconds (default and most 1e9; 0 gives up at once).
+ * A bounded wait of that filter or of the tensor-core kernels that gives up is
+ * reported as MM_ERR_TIMEOUT by the call whose products it belongs to.  Errors: MM_ERR_ARG for an unknown name or
  * value. */
 mm_status mm_set_option(mm_ctx* ctx, const char* name, double value);
 

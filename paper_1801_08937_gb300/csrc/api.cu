@@ -193,6 +193,7 @@ struct mm_ctx {
     // set by a bounded wait of a filter kernel that gave up (pinned host memory the kernels write to)
     int* h_fault = nullptr;
     int* d_fault = nullptr;
+    unsigned opt_wait_ns = WAIT_NS;   // limit of those waits (0: they give up at once)
     // asynchronous stepping
     RhsState* h_st_pinned = nullptr;
     int h_st_pinned_n = 0;
@@ -861,6 +862,7 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
     }
     a.csdf = ctx->d_csdf.as<float4>();
     a.fault = ctx->d_fault;
+    a.wait_ns = ctx->opt_wait_ns;
     if (ctx->tmpl_on) {
         if (!plan->lens.empty() || !plan->starts.empty())
             return fail(ctx, MM_ERR_ARG, "template filters: right-hand sides of uneven length are not supported");
@@ -2637,6 +2639,9 @@ mm_status mm_set_option(mm_ctx* ctx, const char* name, double value) {
     } else if (n == "harvest") {
         if (v < 0 || v > 4096) return fail(ctx, MM_ERR_ARG, "harvest must lie in [0, 4096]");
         ctx->opt_harvest = v;
+    } else if (n == "wait_limit_ns") {
+        if (!(value >= 0.0) || value > (double)WAIT_NS) return fail(ctx, MM_ERR_ARG, "wait_limit_ns must lie in [0, 1e9]");
+        ctx->opt_wait_ns = (unsigned)value;
     } else if (n == "time_filter") {
         ctx->opt_time_filter = v ? 1 : 0;
         ctx->fev_used = 0;
@@ -2658,6 +2663,7 @@ mm_status mm_get_option(mm_ctx* ctx, const char* name, double* value) {
     else if (n == "last_apply_ms") *value = ctx->last_apply_ms;
     else if (n == "kernel_launches") *value = (double)launches_total();
     else if (n == "time_filter") *value = ctx->opt_time_filter;
+    else if (n == "wait_limit_ns") *value = ctx->opt_wait_ns;
     else if (n == "autotune") *value = ctx->opt_autotune;
     else if (n == "half_transform") *value = ctx->opt_half;
     else if (n == "coarse_prefix") *value = ctx->opt_coarse_prefix;

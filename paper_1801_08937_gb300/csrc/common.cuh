@@ -128,6 +128,7 @@ struct FilterArgs {
     int three;             // half, float32: three passes of radix r0, r1, 9 (half3_shape)
     int even;              // every segment starts at an even sample
     int* fault;            // set to 1 by a bounded wait that gave up
+    unsigned wait_ns;      // its limit
     int ahead;             // CTAs on the device at a time: the pointing of the CTA so many later goes to L2
     const void* band;      // direct: [n_bands][lambda+1]
     int L, logL, lam, V;
@@ -162,6 +163,8 @@ void launch_filter_fft_f32(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_fft_f64(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_f32(const FilterArgs& a, bool from_tod, cudaStream_t s);
 void launch_filter_direct_f64(const FilterArgs& a, bool from_tod, cudaStream_t s);
+// Limit of the filter kernels' waits, nanoseconds ("wait_limit_ns" sets a context's own).
+constexpr unsigned WAIT_NS = 1000000000u;
 // Spare bytes behind pix and psi: the chunked copies of the three-pass filter read past the last sample.
 constexpr size_t POINTING_SPARE = 16384;
 // Spectra of the bands for circular products of N points by the cosine sum, on the device: H[b][k] / N for

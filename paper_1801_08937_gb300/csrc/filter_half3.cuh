@@ -79,15 +79,16 @@ __device__ __forceinline__ bool h3_bar_try(uint32_t bar, uint32_t parity) {
                  : "memory");
     return done != 0;
 }
-// false if the copy has not landed after a second
-__device__ __forceinline__ bool h3_bar_wait(uint32_t bar, uint32_t parity) {
+// false if the copy has not landed after `limit` nanoseconds (0: without a look)
+__device__ __forceinline__ bool h3_bar_wait(uint32_t bar, uint32_t parity, unsigned limit) {
+    if (limit == 0) return false;
     if (h3_bar_try(bar, parity)) return true;
     unsigned long long t0, t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
     for (;;) {
         if (h3_bar_try(bar, parity)) return true;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        if (t - t0 > 1000000000ull) return false;
+        if (t - t0 > limit) return false;
     }
 }
 
@@ -255,19 +256,24 @@ __global__ void __launch_bounds__(H::NT, H::MINB) k_filter_half3(const FilterArg
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * i), "l"(map + S.win0 + i) : "memory");
             asm volatile("cp.async.wait_all;" ::: "memory");
             bool ok = true;
+            int issued = min(NS, nch);   // thread 0: chunks asked for
             auto rows = [&](auto entry) {
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                     int32_t* lc = reinterpret_cast<int32_t*>(smraw + H::BUF - (NS - c % NS) * H::CHB) + d;
                     __syncthreads();   // everyone is done with chunk c - 1 (and has staged its map entries)
-                    if (c > 0 && c + NS - 1 < nch && j == 0)
+                    // (behind a wait that gave up the buffer's barrier still counts its last copy: no new one then)
+                    if (c > 0 && c + NS - 1 < nch && j == 0 && ok) {
                         h3_fetch<H>(a.pix + base, a.psi + base, c + NS - 1, cb + ((c - 1) % NS) * H::CHB,
                                     fb + 8 * ((c - 1) % NS));
+                        issued = c + NS;
+                    }
                     if (c < nch) {
-                        ok = ok && h3_bar_wait(fb + 8 * (c % NS), (c / NS) & 1);
+                        ok = ok && h3_bar_wait(fb + 8 * (c % NS), (c / NS) & 1, a.wait_ns);
                         if (S.n_out < (c + 1) * H::CH) {   // the end of the block: what follows is flagged
-                            for (int k = S.n_out - c * H::CH + j; k < H::CH; k += H::NT) lc[k] = -1;
-                            __syncthreads();
+                            if (ok)   // (not while the copy may still land on it)
+                                for (int k = S.n_out - c * H::CH + j; k < H::CH; k += H::NT) lc[k] = -1;
+                            ok = __syncthreads_and(ok);
                         }
                     }
                     if (c < nch && ok) {
@@ -297,9 +303,8 @@ __global__ void __launch_bounds__(H::NT, H::MINB) k_filter_half3(const FilterArg
             else rows([&](int p) { return __ldg(map + max(p, 0)); });
             if (!ok) {
                 *reinterpret_cast<volatile int*>(a.fault) = 1;
-#pragma unroll
-                for (int c = 0; c < NS; ++c)   // let copies in flight land before the buffer is reused
-                    if (c < nch) h3_bar_wait(fb + 8 * c, ((nch - 1 - c) / NS) & 1);
+                if (j == 0)   // let the copies in flight land before the buffer is reused
+                    for (int c = max(0, issued - NS); c < issued; ++c) h3_bar_wait(fb + 8 * (c % NS), (c / NS) & 1, WAIT_NS);
             }
             __syncthreads();   // the buffer becomes the transform's
         }
