@@ -638,6 +638,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
 
 mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, void* dst, const RhsState* st,
                      int tod_is_float, const void* xmap = nullptr);
+mm_status filter_fault_check(mm_ctx* ctx);
 
 // Process-wide record of tuned choices, keyed by problem shape.
 struct TuneKey {
@@ -754,13 +755,24 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
     CK(src.ensure(nv * esz));
     CK(dst.ensure(nv * esz));
     CK(cudaMemsetAsync(src.p, 0, nv * esz, ctx->stream));
-    cudaEvent_t e0, e1;
-    CK(cudaEventCreate(&e0));
-    CK(cudaEventCreate(&e1));
+    struct Tuning {   // whatever way the tuner is left, the context's products are reduced and timed again
+        mm_ctx* c;
+        int time_filter;
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        explicit Tuning(mm_ctx* ctx) : c(ctx), time_filter(ctx->opt_time_filter) {
+            c->opt_time_filter = 0;
+            c->tuning = true;
+        }
+        ~Tuning() {
+            c->opt_time_filter = time_filter;
+            c->tuning = false;
+            if (e0) cudaEventDestroy(e0);
+            if (e1) cudaEventDestroy(e1);
+        }
+    } t(ctx);
+    CK(cudaEventCreate(&t.e0));
+    CK(cudaEventCreate(&t.e1));
     best->ms = 1e300;
-    const int saved_time = ctx->opt_time_filter;
-    ctx->opt_time_filter = 0;
-    ctx->tuning = true;
     for (const Opt& o : opts) {
         Plan* p = nullptr;
         TRY(make_plan(ctx, f64, nrhs, lens, o.variant, o.L, o.whole, o.V, &p));
@@ -768,21 +780,18 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
         // best of up to three timed launches (one when a launch is long)
         double ms_best = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
-            CK(cudaEventRecord(e0, ctx->stream));
+            CK(cudaEventRecord(t.e0, ctx->stream));
             TRY(run_filter(ctx, p, false, src.p, dst.p, nullptr, 0));
-            CK(cudaEventRecord(e1, ctx->stream));
-            CK(cudaEventSynchronize(e1));
+            CK(cudaEventRecord(t.e1, ctx->stream));
+            CK(cudaEventSynchronize(t.e1));
+            TRY(filter_fault_check(ctx));
             float ms = 0.f;
-            CK(cudaEventElapsedTime(&ms, e0, e1));
+            CK(cudaEventElapsedTime(&ms, t.e0, t.e1));
             ms_best = std::min(ms_best, (double)ms);
             if (ms > 2.0) break;
         }
         if (ms_best < best->ms) *best = TuneVal{o.variant, o.L, o.whole, o.V, ms_best};
     }
-    ctx->opt_time_filter = saved_time;
-    ctx->tuning = false;
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     return MM_OK;
 }
 
@@ -1246,6 +1255,11 @@ mm_status finish_coarse(mm_ctx* ctx) {
     std::vector<double> G((size_t)k * k), E((size_t)k * k);
     CK(cudaMemcpyAsync(G.data(), dG.p, G.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    const mm_status wait = filter_fault_check(ctx);
+    if (wait != MM_OK) {
+        ctx->k = 0;
+        return wait;
+    }
     for (int i = 0; i < k; ++i)
         for (int j = 0; j < k; ++j) E[(size_t)i * k + j] = 0.5 * (G[(size_t)j * k + i] + G[(size_t)i * k + j]);
     std::vector<double> L = E, Einv;
@@ -1410,6 +1424,7 @@ mm_status coarse_products_for_lens(mm_ctx* ctx, int f64) {
                                ctx->d_Tpref.as<double>() + (size_t)m * k * n, (int64_t)k * n, 1, nullptr, ctx->stream);
         CKL();
         CK(cudaStreamSynchronize(ctx->stream));
+        TRY(filter_fault_check(ctx));
         ctx->tpref_valid = true;
     }
     DevBuf zrep;
@@ -1446,6 +1461,7 @@ mm_status coarse_for_lens(mm_ctx* ctx, const std::vector<uint8_t>& deflate) {
     std::vector<double> G((size_t)R * k * k), Einv_all((size_t)R * k * k);
     CK(cudaMemcpyAsync(G.data(), dG.p, G.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    TRY(filter_fault_check(ctx));
     // A prefix of the scan may leave part of the map unobserved, and with it directions of span Z
     // on which A_i vanishes: E_i is then only semi-definite.  Its inverse is taken on the columns a
     // pivoted Cholesky keeps (all of them when E_i is well conditioned; otherwise the coarse
@@ -1995,6 +2011,7 @@ mm_status mm_build_coarse(mm_ctx* ctx, const double* b_or_null, int32_t m_max, d
         std::vector<double> h2(2 * (size_t)(m_max + 2));
         CK(cudaMemcpyAsync(h2.data(), h, h2.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
+        TRY(filter_fault_check(ctx));
         for (int i = 0; i <= j; ++i) H[(size_t)i * m_max + j] = h2[i] + h2[(size_t)(m_max + 2) + i];
         const double hn = std::sqrt(std::max(0.0, h2[m_max + 1]));
         H[(size_t)(j + 1) * m_max + j] = hn;
