@@ -2513,7 +2513,6 @@ mm_status mm_solve_launch(mm_ctx* ctx, int32_t n_iter) {
     TRY(launch_iters(ctx, n_iter));
     if (!ctx->h_st_pinned || ctx->h_st_pinned_n < ctx->nrhs) {
         if (ctx->h_st_pinned) cudaFreeHost(ctx->h_st_pinned);
-    if (ctx->reduce_host) cudaFreeHost(ctx->reduce_host);
         ctx->h_st_pinned = nullptr;
         CK(cudaMallocHost(reinterpret_cast<void**>(&ctx->h_st_pinned), ctx->nrhs * sizeof(RhsState)));
         ctx->h_st_pinned_n = ctx->nrhs;
