@@ -213,7 +213,8 @@ void launch_zero(void* p, size_t bytes, cudaStream_t s) {
 // the float64 pipe (17 operations a sample, 0.9 ms on 3.4e7 samples at its
 // measured rate): 4433 -> 1191 us there against one sample per lane with the
 // general sincos and seven five-step shuffled sums.
-constexpr int BD_SLICE = 8192;   // samples per CTA: long blocks spread over the device
+constexpr int BD_SLICE = 8192;   // samples per CTA and step: long blocks spread over the device
+constexpr int BD_SLICES = 1024;  // CTAs per block at most (a grid holds 65535 rows): longer blocks are walked
 
 struct BdSums {
     double c, s, cc, cs, ss;
@@ -242,85 +243,86 @@ __global__ void __launch_bounds__(VT) k_bd_accumulate(const int32_t* __restrict_
     const int b = blockIdx.x;
     const int64_t o1 = block_off[b + 1];
     const int64_t det0 = block_off[b] / n_t * n_t;   // a block lies in one detector's timeline
-    const int64_t s0 = block_off[b] + (int64_t)blockIdx.y * BD_SLICE;
-    const int64_t s1 = s0 + BD_SLICE < o1 ? s0 + BD_SLICE : o1;
     const double c0 = band[(int64_t)block_band[b] * lam1];
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    for (int64_t w0 = s0 + (threadIdx.x >> 5) * 256; w0 < s1; w0 += VT * 8) {
-        const int64_t t0 = w0 + 8 * lane;
-        using Key = typename std::conditional<LENS, int64_t, int>::type;
-        Key key[8];
-        BdSums a{0, 0, 0, 0, 0, 0}, f{0, 0, 0, 0, 0, 0};
-        bool multi = false;
-        int j = 0;
-        if (LENS && t0 < s1) {   // lengths up to the first sample's position
-            const int64_t pos = t0 - det0;
-            int hi = nrhs;
-            while (j < hi) {
-                const int mid = (j + hi) >> 1;
-                if (sorted_len[mid] <= pos) j = mid + 1;
-                else hi = mid;
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int64_t t = t0 + e;
-            key[e] = -1;
-            double cs = 0.0, sn = 0.0;
-            if (t < s1) {
-                const int p = __ldg(pix + t);
-                if (LENS) {
-                    while (j < nrhs && sorted_len[j] <= t - det0) ++j;
-                    if (p >= 0 && j < nrhs) key[e] = (Key)j * n_pix + p;
-                } else {
-                    key[e] = p;
+    for (int64_t s0 = block_off[b] + (int64_t)blockIdx.y * BD_SLICE; s0 < o1; s0 += (int64_t)gridDim.y * BD_SLICE) {
+        const int64_t s1 = s0 + BD_SLICE < o1 ? s0 + BD_SLICE : o1;
+        for (int64_t w0 = s0 + (threadIdx.x >> 5) * 256; w0 < s1; w0 += VT * 8) {
+            const int64_t t0 = w0 + 8 * lane;
+            using Key = typename std::conditional<LENS, int64_t, int>::type;
+            Key key[8];
+            BdSums a{0, 0, 0, 0, 0, 0}, f{0, 0, 0, 0, 0, 0};
+            bool multi = false;
+            int j = 0;
+            if (LENS && t0 < s1) {   // lengths up to the first sample's position
+                const int64_t pos = t0 - det0;
+                int hi = nrhs;
+                while (j < hi) {
+                    const int mid = (j + hi) >> 1;
+                    if (sorted_len[mid] <= pos) j = mid + 1;
+                    else hi = mid;
                 }
-                if (key[e] >= 0) {
-                    if (cs64) {
-                        const double2 w = __ldg(cs64 + t);
-                        cs = w.x;
-                        sn = w.y;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t t = t0 + e;
+                key[e] = -1;
+                double cs = 0.0, sn = 0.0;
+                if (t < s1) {
+                    const int p = __ldg(pix + t);
+                    if (LENS) {
+                        while (j < nrhs && sorted_len[j] <= t - det0) ++j;
+                        if (p >= 0 && j < nrhs) key[e] = (Key)j * n_pix + p;
                     } else {
-                        sincos_2psi(__ldg(psi + t), trig, cs, sn);
+                        key[e] = p;
+                    }
+                    if (key[e] >= 0) {
+                        if (cs64) {
+                            const double2 w = __ldg(cs64 + t);
+                            cs = w.x;
+                            sn = w.y;
+                        } else {
+                            sincos_2psi(__ldg(psi + t), trig, cs, sn);
+                        }
                     }
                 }
-            }
-            if (e > 0 && key[e] != key[e - 1]) {
-                if (multi) {
-                    if (key[e - 1] >= 0) bd_flush(sums, key[e - 1], c0, a);
-                } else {
-                    f = a;
-                    multi = true;
+                if (e > 0 && key[e] != key[e - 1]) {
+                    if (multi) {
+                        if (key[e - 1] >= 0) bd_flush(sums, key[e - 1], c0, a);
+                    } else {
+                        f = a;
+                        multi = true;
+                    }
+                    a = BdSums{0, 0, 0, 0, 0, 0};
                 }
-                a = BdSums{0, 0, 0, 0, 0, 0};
+                a.c += cs;
+                a.s += sn;
+                a.cc = fma(cs, cs, a.cc);
+                a.cs = fma(cs, sn, a.cs);
+                a.ss = fma(sn, sn, a.ss);
+                a.n += 1;
             }
-            a.c += cs;
-            a.s += sn;
-            a.cc = fma(cs, cs, a.cc);
-            a.cs = fma(cs, sn, a.cs);
-            a.ss = fma(sn, sn, a.ss);
-            a.n += 1;
+            const Key klast = __shfl_up_sync(FULL, key[7], 1);
+            const bool give = multi && lane > 0 && key[0] == klast;
+            BdSums r;
+            r.c = __shfl_down_sync(FULL, f.c, 1);
+            r.s = __shfl_down_sync(FULL, f.s, 1);
+            r.cc = __shfl_down_sync(FULL, f.cc, 1);
+            r.cs = __shfl_down_sync(FULL, f.cs, 1);
+            r.ss = __shfl_down_sync(FULL, f.ss, 1);
+            r.n = __shfl_down_sync(FULL, f.n, 1);
+            if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
+                a.c += r.c;
+                a.s += r.s;
+                a.cc += r.cc;
+                a.cs += r.cs;
+                a.ss += r.ss;
+                a.n += r.n;
+            }
+            if (multi && !give && key[0] >= 0) bd_flush(sums, key[0], c0, f);
+            if (key[7] >= 0) bd_flush(sums, key[7], c0, a);
         }
-        const Key klast = __shfl_up_sync(FULL, key[7], 1);
-        const bool give = multi && lane > 0 && key[0] == klast;
-        BdSums r;
-        r.c = __shfl_down_sync(FULL, f.c, 1);
-        r.s = __shfl_down_sync(FULL, f.s, 1);
-        r.cc = __shfl_down_sync(FULL, f.cc, 1);
-        r.cs = __shfl_down_sync(FULL, f.cs, 1);
-        r.ss = __shfl_down_sync(FULL, f.ss, 1);
-        r.n = __shfl_down_sync(FULL, f.n, 1);
-        if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
-            a.c += r.c;
-            a.s += r.s;
-            a.cc += r.cc;
-            a.cs += r.cs;
-            a.ss += r.ss;
-            a.n += r.n;
-        }
-        if (multi && !give && key[0] >= 0) bd_flush(sums, key[0], c0, f);
-        if (key[7] >= 0) bd_flush(sums, key[7], c0, a);
     }
 }
 
@@ -340,7 +342,7 @@ void launch_bd_accumulate(const int32_t* pix, const float* psi, const double2* c
                           int64_t max_block, int64_t n_t, const int64_t* sorted_len, int nrhs, double* sums, int n_pix,
                           cudaStream_t s) {
     if (n_blocks <= 0) return;
-    const dim3 g(n_blocks, (unsigned)((max_block + BD_SLICE - 1) / BD_SLICE));
+    const dim3 g(n_blocks, (unsigned)std::min<int64_t>(BD_SLICES, (max_block + BD_SLICE - 1) / BD_SLICE));
     if (sorted_len)
         k_bd_accumulate<true><<<g, VT, 0, s>>>(pix, psi, cs64, trig, block_off, block_band, band, lam1, n_t, sorted_len,
                                                nrhs, sums, n_pix);
