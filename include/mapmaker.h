@@ -269,7 +269,8 @@ mm_status mm_solve(mm_ctx* ctx, const void* tod, double* map_out, int32_t nrhs,
  * "fft_log2": FFT length 2^v (0 = choose); "autotune": 1 (default) times the
  * candidate filter plans on first use of a problem shape and keeps the
  * fastest (cached per process, and in the JSON-lines file named by the
- * environment variable MM_TUNE_CACHE when set); "direct_tile": outputs per
+ * environment variable MM_TUNE_CACHE when set; lines chosen from another
+ * build's set of plans are passed over); "direct_tile": outputs per
  * CTA of the direct filter; "check_every": PCG iterations between host
  * convergence checks; "graphs": 1 to replay a captured CUDA graph of
  * check_every PCG iterations (only on a created stream, not the legacy

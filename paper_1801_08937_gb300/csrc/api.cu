@@ -655,7 +655,11 @@ struct TuneVal {
     double ms;
 };
 // Optional persistence: when MM_TUNE_CACHE names a file, tuned choices are
-// read from it at first use and appended to it as JSON lines.
+// read from it at first use and appended to it as JSON lines.  A line names the
+// set of plans it was chosen from: one of another set is passed over (a choice
+// made before a faster plan existed would hide that plan for good).  Raised with
+// every change of the candidates or of which of them is fast.
+constexpr int TUNE_VERSION = 2;
 const char* tune_file() { return std::getenv("MM_TUNE_CACHE"); }
 
 // The plan cache is shared by every context of the process (contexts may be
@@ -678,12 +682,14 @@ std::vector<std::pair<TuneKey, TuneVal>>& tune_cache() {
                     TuneKey k{};
                     TuneVal v{};
                     long long ns = 0, mb = 0, ls = 0;
+                    int version = 0;
                     if (std::sscanf(line,
-                                    "{\"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
+                                    "{\"v\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
                                     "\"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
                                     "\"whole\": %d, \"V\": %d, \"ms\": %lf}",
-                                    &k.f64, &k.lam, &k.n_blocks, &k.nrhs, &ns, &mb, &ls, &k.n_pix, &v.variant, &v.L,
-                                    &v.whole, &v.V, &v.ms) == 13) {
+                                    &version, &k.f64, &k.lam, &k.n_blocks, &k.nrhs, &ns, &mb, &ls, &k.n_pix, &v.variant,
+                                    &v.L, &v.whole, &v.V, &v.ms) == 14 &&
+                        version == TUNE_VERSION) {
                         k.n_samples = ns;
                         k.max_block = mb;
                         k.lens_sum = ls;
@@ -713,10 +719,10 @@ void tune_record(const TuneKey& k, const TuneVal& v) {
     if (const char* path = tune_file()) {
         if (FILE* f = std::fopen(path, "a")) {
             std::fprintf(f,
-                         "{\"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
+                         "{\"v\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
                          "\"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
                          "\"whole\": %d, \"V\": %d, \"ms\": %.6f}\n",
-                         k.f64, k.lam, k.n_blocks, k.nrhs, (long long)k.n_samples, (long long)k.max_block,
+                         TUNE_VERSION, k.f64, k.lam, k.n_blocks, k.nrhs, (long long)k.n_samples, (long long)k.max_block,
                          (long long)k.lens_sum, k.n_pix, v.variant, v.L, v.whole, v.V, v.ms);
             std::fclose(f);
         }
