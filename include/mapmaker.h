@@ -287,7 +287,7 @@ mm_status mm_solve(mm_ctx* ctx, const void* tod, double* map_out, int32_t nrhs,
  * PCG run between float64-accurate refinements (default 2e-6);
  * "half_transform": 1 (default) lets a whole block of N real samples run as
  * one N/2-point complex transform per CTA (paired real-spectrum step), 2
- * prefers such a block split by frequency over two CTAs where native float64
+ * takes such a block split by frequency over two CTAs wherever native float64
  * products have that form (with 1 it is used where it times faster), 0
  * keeps two blocks per N-point transform; "coarse_prefix": 1 (default) forms
  * the per-RHS coarse products A_i Z of an uneven-length two-level batch from

@@ -645,8 +645,9 @@ struct TuneKey {
     int f64, lam, n_blocks, nrhs;
     int64_t n_samples, max_block, lens_sum;
     int n_pix;
+    int half;   // "half_transform": each of its values has candidates of its own
     bool operator==(const TuneKey& o) const {
-        return f64 == o.f64 && lam == o.lam && n_blocks == o.n_blocks && nrhs == o.nrhs && n_samples == o.n_samples &&
+        return half == o.half && f64 == o.f64 && lam == o.lam && n_blocks == o.n_blocks && nrhs == o.nrhs && n_samples == o.n_samples &&
                max_block == o.max_block && lens_sum == o.lens_sum && n_pix == o.n_pix;
     }
 };
@@ -684,11 +685,11 @@ std::vector<std::pair<TuneKey, TuneVal>>& tune_cache() {
                     long long ns = 0, mb = 0, ls = 0;
                     int version = 0;
                     if (std::sscanf(line,
-                                    "{\"v\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
-                                    "\"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
+                                    "{\"v\": %d, \"half\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, "
+                                    "\"n_samples\": %lld, \"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
                                     "\"whole\": %d, \"V\": %d, \"ms\": %lf}",
-                                    &version, &k.f64, &k.lam, &k.n_blocks, &k.nrhs, &ns, &mb, &ls, &k.n_pix, &v.variant,
-                                    &v.L, &v.whole, &v.V, &v.ms) == 14 &&
+                                    &version, &k.half, &k.f64, &k.lam, &k.n_blocks, &k.nrhs, &ns, &mb, &ls, &k.n_pix,
+                                    &v.variant, &v.L, &v.whole, &v.V, &v.ms) == 15 &&
                         version == TUNE_VERSION) {
                         k.n_samples = ns;
                         k.max_block = mb;
@@ -703,10 +704,10 @@ std::vector<std::pair<TuneKey, TuneVal>>& tune_cache() {
     return c;
 }
 
-bool tune_lookup(const TuneKey& k, bool allow_half, TuneVal* v) {
+bool tune_lookup(const TuneKey& k, TuneVal* v) {
     std::lock_guard<std::mutex> lock(tune_mutex());
     for (auto& kv : tune_cache())
-        if (kv.first == k && (allow_half || kv.second.whole < 2)) {
+        if (kv.first == k) {
             *v = kv.second;
             return true;
         }
@@ -719,10 +720,10 @@ void tune_record(const TuneKey& k, const TuneVal& v) {
     if (const char* path = tune_file()) {
         if (FILE* f = std::fopen(path, "a")) {
             std::fprintf(f,
-                         "{\"v\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, \"n_samples\": %lld, "
-                         "\"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
+                         "{\"v\": %d, \"half\": %d, \"f64\": %d, \"lam\": %d, \"n_blocks\": %d, \"nrhs\": %d, "
+                         "\"n_samples\": %lld, \"max_block\": %lld, \"lens_sum\": %lld, \"n_pix\": %d, \"variant\": %d, \"L\": %d, "
                          "\"whole\": %d, \"V\": %d, \"ms\": %.6f}\n",
-                         TUNE_VERSION, k.f64, k.lam, k.n_blocks, k.nrhs, (long long)k.n_samples, (long long)k.max_block,
+                         TUNE_VERSION, k.half, k.f64, k.lam, k.n_blocks, k.nrhs, (long long)k.n_samples, (long long)k.max_block,
                          (long long)k.lens_sum, k.n_pix, v.variant, v.L, v.whole, v.V, v.ms);
             std::fclose(f);
         }
@@ -751,7 +752,11 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
             opts.push_back(
                 {2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
     }
-    if (ctx->lam <= 256)
+    // "half_transform" = 2 asks for blocks split over two CTAs wherever they have that form
+    auto split = [](const Opt& o) { return o.whole == 3; };
+    const bool only_split = ctx->opt_half == 2 && std::any_of(opts.begin(), opts.end(), split);
+    if (only_split) opts.erase(std::remove_if(opts.begin(), opts.end(), [&](const Opt& o) { return !split(o); }), opts.end());
+    if (ctx->lam <= 256 && !only_split)
         for (int tile : {1024, 2048})
             if (direct_smem_bytes(tile, ctx->lam, f64 != 0) <= 200 * 1024) opts.push_back({1, 0, 0, tile});
     if (opts.empty()) return fail(ctx, MM_ERR_ARG, "no filter plan fits this band");
@@ -814,9 +819,9 @@ mm_status get_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& l
         int tn = 1;
         if (ctx->n_blocks < 304)
             while (tn < 16 && 2 * tn <= nrhs) tn *= 2;
-        TuneKey key{f64, ctx->lam, ctx->n_blocks, tn, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix};
+        TuneKey key{f64, ctx->lam, ctx->n_blocks, tn, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix, ctx->opt_half};
         TuneVal hit{};
-        if (tune_lookup(key, ctx->opt_half != 0, &hit))
+        if (tune_lookup(key, &hit))
             return make_plan(ctx, f64, nrhs, lens, hit.variant, hit.L, hit.whole, hit.V, out, starts);
         TuneVal best{};
         TRY(autotune_plan(ctx, f64, tn, {}, &best));

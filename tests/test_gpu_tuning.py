@@ -52,3 +52,24 @@ def test_lines_of_another_set_of_plans_are_passed_over(tmp_path):
     # others, and those from before lines carried a version: tuned again, recorded beside the old line
     assert lines_after(dict(forced, v=entry["v"] - 1))[1] == 2
     assert lines_after({k: v for k, v in forced.items() if k != "v"})[1] == 2
+
+
+# 64 blocks have fewer CTAs than the device has SMs, 256 blocks more (one CTA a block is then usual)
+@pytest.mark.parametrize("n_det", [8, 32])
+def test_half_transform_is_part_of_what_a_choice_is_reused_for(n_det):
+    """0 keeps half-length plans out, 2 takes blocks split over two CTAs, whatever was tuned before for the
+    other values; native float64, all tuned in one process."""
+    import numpy as np
+    import synth
+    scan = synth.make_scan(nx=16, ny=16, n_det=n_det, n_t=8 * 4096, n_int=8, half_bw=500, f_knee=1.0, seed=8)
+    got = []
+    for half in (0, 1, 2, 1, 0, 2):
+        c = MM.Context(0, None, MM.MM_FP64)
+        c.set_option("half_transform", half)
+        c.setup_scan(scan)
+        c.apply_A(np.zeros((1, scan.n_pix, 3)))
+        got.append(c.get_option("plan_whole"))
+        c.close()
+    assert got[0] in (0, 1) and got[4] == got[0]
+    assert got[2] == got[5] == 3
+    assert got[3] == got[1]
