@@ -811,6 +811,8 @@ mm_status get_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& l
     int variant = ctx->opt_filter;
     int L = 0, V = 0, whole = 0;
     if (variant == 0 && ctx->opt_fft_len == 0 && ctx->opt_fft_log2 == 0 && ctx->opt_autotune && !ctx->capturing) {
+        // template products read nothing of a plan but its type and right-hand sides: none is timed or recorded
+        if (ctx->tmpl_on) return make_plan(ctx, f64, nrhs, lens, 1, 0, 0, (int)max_block_len(ctx), out, starts);
         // tuned once per precision and geometry, on a single right-hand side where that fills the device (the
         // per-CTA work of a plan does not depend on how many right-hand sides share it).  With fewer blocks than
         // two per SM one right-hand side wants short segments on many SMs and a batch the least work per sample

@@ -73,3 +73,24 @@ def test_half_transform_is_part_of_what_a_choice_is_reused_for(n_det):
     assert got[0] in (0, 1) and got[4] == got[0]
     assert got[2] == got[5] == 3
     assert got[3] == got[1]
+
+
+def test_template_products_record_no_plan(tmp_path):
+    """The template kernel is one for every plan: its times say nothing about an unfiltered scan of the same shape."""
+    cache = tmp_path / "tune"
+    body = f"""
+        scan = synth.make_scan(**{dict(SCAN, half_bw=0, f_knee=0.0, hwp=False)!r})
+        sub, az, bins = synth.make_templates(scan)
+        c = MM.Context(0, None, MM.MM_FP32_MIXED)
+        c.setup_scan(scan)
+        x = np.random.default_rng(1).standard_normal((1, scan.n_pix, 3))
+        for on in (True, False):
+            if on: c.set_templates(1, sub, az, bins)
+            else: c.set_templates()
+            c.apply_A(x)
+            c.rhs(np.zeros((1, scan.n_samples), dtype=np.float32))
+            if on: assert not __import__("os").path.exists({str(cache)!r})
+        print(json.dumps(c.get_option("plan_whole")))
+    """
+    child(cache, body)
+    assert len(cache.read_text().splitlines()) == 2   # the unfiltered float32 and double-float products
