@@ -59,7 +59,7 @@ struct FftTables {
 };
 
 struct Plan {
-    FftTables ft;      // twiddles and band spectra for this plan's L
+    std::shared_ptr<FftTables> ft;   // twiddles and band spectra, shared by the scan's plans of one type and length
     int variant = 0;   // 1 direct, 2 fft
     int L = 0, logL = 0, V = 0;
     int whole = 0;     // FFT: 1 one transform per whole block (no overlap-save halo), two blocks
@@ -342,10 +342,11 @@ void split_passes(int M, FftPasses* fp) {
 // FFT length and mode candidates: whole blocks (one block per transform, no
 // halo, when L >= n_b + lambda) or overlap-save segments of V = L - 2 lambda
 // outputs.  Cost model: transform points x passes plus gathered and
-// scattered samples, with a penalty when the grid cannot fill the GPU.
+// scattered samples, with a penalty when the grid cannot fill the GPU; `work`
+// is the same without it, what a batch that fills the GPU pays per map.
 struct FftCand {
     int L, whole;
-    double cost;
+    double cost, work;
 };
 
 std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, int forced_len) {
@@ -369,11 +370,11 @@ std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, i
                 const double per_ctah = (double)(L / 2) * fh.npass * 44.0 + 2.0 * (double)c->n_samples / ctash * 45.0;
                 const double wavesh = std::ceil(ctash / (152.0 * per_smh));
                 const double cost = wavesh * per_ctah + 1e-3 * ((double)c->n_blocks * (L / 2) * fh.npass * 44.0);
-                out.push_back({L, 2, cost});
+                out.push_back({L, 2, cost, ctash * per_ctah});
                 // float64 blocks split by frequency over two CTAs, where one CTA each leaves SMs idle; timed, or
                 // asked for by "half_transform" = 2
                 if (f64 == 1 && split_shape(L / 2) && (c->opt_half == 2 || c->n_blocks < 152))
-                    out.push_back({L, 3, c->opt_half == 2 ? 0.0 : 1.001 * cost});
+                    out.push_back({L, 3, c->opt_half == 2 ? 0.0 : 1.001 * cost, 1.1 * ctash * per_ctah});
             }
             const size_t sm = fft_smem_bytes(L, f64 != 0);
             if (sm > smem_limit_bytes()) continue;
@@ -404,7 +405,7 @@ std::vector<FftCand> fft_candidates(const mm_ctx* c, int f64, int forced_log2, i
             const double per_cta = (double)L * fp.npass * 44.0 + (gathered + (double)c->n_samples) / std::max(1.0, ctas) * 45.0;
             const double waves = std::ceil(std::max(1.0, ctas) / slots);
             double cost = waves * per_cta + 1e-3 * (points * fp.npass * 44.0);
-            out.push_back({L, whole, cost});
+            out.push_back({L, whole, cost, std::max(1.0, ctas) * per_cta});
         }
     }
     std::sort(out.begin(), out.end(), [](const FftCand& a, const FftCand& b) { return a.cost < b.cost; });
@@ -598,7 +599,13 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     }
     auto p = std::move(ctx->spare);
     if (!p) p = std::make_unique<Plan>();
-    p->ft.L = 0;   // its tables are another scan's
+    std::shared_ptr<FftTables> tables;
+    if (variant == 2)
+        for (auto& o : ctx->plans)
+            if (o->variant == 2 && o->L == L && o->whole == whole && o->f64 == f64) tables = o->ft;
+    if (tables) p->ft = tables;
+    else if (!p->ft || p->ft.use_count() > 1) p->ft = std::make_shared<FftTables>();
+    if (!tables) p->ft->L = 0;   // a kept plan's are another scan's
     p->three = false;
     p->even = true;
     p->variant = variant;
@@ -619,9 +626,9 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     if (!segs.empty())
         CK(cudaMemcpyAsync(p->segs.p, segs.data(), segs.size() * sizeof(Seg), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    if (p->three) TRY(build_half3_tables(ctx, p->ft, L));
-    else if (variant == 2 && whole >= 2) TRY(build_half_tables(ctx, p->ft, fp, L, f64));
-    else if (variant == 2) TRY(build_fft_tables(ctx, p->ft, fp, f64));
+    if (p->three) TRY(build_half3_tables(ctx, *p->ft, L));
+    else if (variant == 2 && whole >= 2) TRY(build_half_tables(ctx, *p->ft, fp, L, f64));
+    else if (variant == 2) TRY(build_fft_tables(ctx, *p->ft, fp, f64));
     if (f64 == 2 && !ctx->have_csdf) {
         CK(ctx->d_csdf.ensure((size_t)ctx->n_samples * 16));
         launch_weights_df(ctx->d_psi.as<float>(), ctx->have_cs64 ? ctx->d_cs64.as<double2>() : nullptr, trig_of(ctx),
@@ -732,12 +739,22 @@ void tune_record(const TuneKey& k, const TuneVal& v) {
 
 // Time each candidate plan once (after one warm-up launch) on the current
 // pointing and keep the fastest.  Candidates: the six cheapest FFT plans of
-// the cost model, the two shortest half-length and every three-pass plan of
-// whole blocks and, for narrow bands, the direct band at two tile sizes.
-mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& lens, TuneVal* best) {
+// the cost model, the two shortest half-length, every three-pass and every
+// split plan of whole blocks and, for narrow bands, the direct band at two
+// tile sizes.  A batch (`single`: the plan of one right-hand side) chooses
+// between that one, the plan of least work and the shortest half-length and
+// three-pass ones: its launches are long, and timing all plans four times, 16
+// right-hand sides each, cost the first coarse space of a small scan (c1, k =
+// 16) 40 ms: 46.2 ms against 7.7 so.  Two or three right-hand sides, which may
+// want any of the plans, time all of them, mostly once.
+mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& lens, TuneVal* best,
+                        const TuneVal* single = nullptr) {
     struct Opt { int variant, L, whole, V; };
     std::vector<Opt> opts;
     auto cands = fft_candidates(ctx, f64, 0, 0);
+    auto opt_of = [&](const FftCand& c) {
+        return Opt{2, c.L, c.whole, c.whole ? c.L - ctx->lam : c.L - 2 * ctx->lam};
+    };
     // the cost model underrates whole blocks as half-length transforms (no halo, half the points): the two
     // shortest of them are always timed
     std::vector<int> half;
@@ -749,8 +766,7 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
         int r0 = 0, r1 = 0;
         const bool three = f64 == 0 && cands[i].whole == 2 && half3_shape(cands[i].L / 2, &r0, &r1);
         if (i < 6 || short_half || three || cands[i].whole == 3)
-            opts.push_back(
-                {2, cands[i].L, cands[i].whole, cands[i].whole ? cands[i].L - ctx->lam : cands[i].L - 2 * ctx->lam});
+            opts.push_back(opt_of(cands[i]));
     }
     // "half_transform" = 2 asks for blocks split over two CTAs wherever they have that form
     auto split = [](const Opt& o) { return o.whole == 3; };
@@ -759,6 +775,28 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
     if (ctx->lam <= 256 && !only_split)
         for (int tile : {1024, 2048})
             if (direct_smem_bytes(tile, ctx->lam, f64 != 0) <= 200 * 1024) opts.push_back({1, 0, 0, tile});
+    if (single && nrhs > 2 && !only_split) {
+        opts.assign(1, Opt{single->variant, single->L, single->whole, single->V});
+        auto add = [&](const FftCand& c) {
+            const Opt o = opt_of(c);
+            for (const Opt& p : opts)
+                if (p.variant == 2 && p.L == o.L && p.whole == o.whole) return;
+            opts.push_back(o);
+        };
+        const FftCand *least = nullptr, *shortest = nullptr, *three = nullptr;
+        for (const FftCand& c : cands) {
+            int r0 = 0, r1 = 0;
+            if (!least || c.work < least->work) least = &c;
+            if (c.whole == 2 && (!shortest || c.L < shortest->L)) shortest = &c;
+            if (f64 == 0 && c.whole == 2 && half3_shape(c.L / 2, &r0, &r1) && (!three || c.L < three->L)) three = &c;
+        }
+        for (const FftCand* c : {least, shortest, three})
+            if (c) add(*c);
+        if (opts.size() == 1) {
+            *best = *single;
+            return MM_OK;
+        }
+    }
     if (opts.empty()) return fail(ctx, MM_ERR_ARG, "no filter plan fits this band");
     const size_t esz = f64 ? sizeof(V4<double>) : sizeof(V4<float>);   // V4<df> is 32 bytes too
     const size_t nv = (size_t)ctx->n_pix * nrhs;
@@ -787,7 +825,12 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
     for (const Opt& o : opts) {
         Plan* p = nullptr;
         TRY(make_plan(ctx, f64, nrhs, lens, o.variant, o.L, o.whole, o.V, &p));
-        TRY(run_filter(ctx, p, false, src.p, dst.p, nullptr, 0));
+        // (a batch's warm-up is one CTA: it loads the kernel)
+        const int n_work = p->n_work;
+        if (single) p->n_work = std::min(1, n_work);
+        const mm_status warm = run_filter(ctx, p, false, src.p, dst.p, nullptr, 0);
+        p->n_work = n_work;
+        TRY(warm);
         // best of up to three timed launches (one when a launch is long)
         double ms_best = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
@@ -799,7 +842,7 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
             float ms = 0.f;
             CK(cudaEventElapsedTime(&ms, t.e0, t.e1));
             ms_best = std::min(ms_best, (double)ms);
-            if (ms > 2.0) break;
+            if (ms > (single ? 0.3 : 2.0)) break;
         }
         if (ms_best < best->ms) *best = TuneVal{o.variant, o.L, o.whole, o.V, ms_best};
     }
@@ -817,18 +860,23 @@ mm_status get_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& l
         // per-CTA work of a plan does not depend on how many right-hand sides share it).  With fewer blocks than
         // two per SM one right-hand side wants short segments on many SMs and a batch the least work per sample
         // (64 blocks of 4096 samples, float64: 67 us alone in 2048-point segments, but 32 together 1.59 ms
-        // against 1.15 ms in whole blocks), so batches there are tuned on up to 16.
+        // against 1.15 ms in whole blocks), so batches there choose again, on up to 16, between a few plans.
+        auto tuned = [&](int tn, const TuneVal* single, TuneVal* v) -> mm_status {
+            const TuneKey key{f64, ctx->lam, ctx->n_blocks, tn, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix,
+                              ctx->opt_half};
+            if (tune_lookup(key, v)) return MM_OK;
+            TRY(autotune_plan(ctx, f64, tn, {}, v, single));
+            tune_record(key, *v);
+            return MM_OK;
+        };
         int tn = 1;
         if (ctx->n_blocks < 304)
             while (tn < 16 && 2 * tn <= nrhs) tn *= 2;
-        TuneKey key{f64, ctx->lam, ctx->n_blocks, tn, ctx->n_samples, max_block_len(ctx), 0, ctx->n_pix, ctx->opt_half};
-        TuneVal hit{};
-        if (tune_lookup(key, &hit))
-            return make_plan(ctx, f64, nrhs, lens, hit.variant, hit.L, hit.whole, hit.V, out, starts);
-        TuneVal best{};
-        TRY(autotune_plan(ctx, f64, tn, {}, &best));
-        tune_record(key, best);
-        return make_plan(ctx, f64, nrhs, lens, best.variant, best.L, best.whole, best.V, out, starts);
+        TuneVal one{}, val{};
+        TRY(tuned(1, nullptr, &one));
+        val = one;
+        if (tn > 1) TRY(tuned(tn, &one, &val));
+        return make_plan(ctx, f64, nrhs, lens, val.variant, val.L, val.whole, val.V, out, starts);
     }
     if (variant == 0) variant = (ctx->lam <= 32) ? 1 : 2;
     if (variant == 2) {
@@ -902,7 +950,7 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
         t.stokes = ctx->tmpl_qu;
         launch_filter_tmpl(a, t, plan->nrhs, plan->f64, from_tod, ctx->stream);
     } else if (plan->variant == 2) {
-        FftTables& ft = plan->ft;
+        const FftTables& ft = *plan->ft;
         a.H = ft.H.p;
         a.tw = ft.tw.p;
         if (plan->whole >= 2) {

@@ -94,3 +94,27 @@ def test_template_products_record_no_plan(tmp_path):
     """
     child(cache, body)
     assert len(cache.read_text().splitlines()) == 2   # the unfiltered float32 and double-float products
+
+
+@pytest.mark.parametrize("prec", [MM.MM_FP64, MM.MM_FP32_MIXED])
+def test_a_batch_chooses_between_few_plans(prec):
+    """The first batch on a scan of few blocks does not time every plan again: four at most, each with a
+    one-CTA warm-up and up to three timed launches, and tables (up to seven kernels) for those that are new;
+    the batch's product stays the single ones'."""
+    import numpy as np
+    import synth
+    from helpers import assert_close
+    scan = synth.make_scan(nx=16, ny=16, n_det=8, n_t=8 * 3001, n_int=8, half_bw=301, f_knee=1.0, seed=12)
+    c = MM.Context(0, None, prec)
+    c.setup_scan(scan)
+    x = np.random.default_rng(2).standard_normal((16, scan.n_pix, 3))
+    one = [c.apply_A(v[None])[0] for v in x]
+    n0 = c.get_option("kernel_launches")
+    y = c.apply_A(x)
+    n1 = c.get_option("kernel_launches")
+    c.apply_A(x)
+    n2 = c.get_option("kernel_launches")
+    assert (n1 - n0) - (n2 - n1) <= 4 * (1 + 3 + 7)
+    for a, b in zip(y, one):
+        assert_close(a, b, 1e-12 if prec == MM.MM_FP64 else 1e-5)
+    c.close()
