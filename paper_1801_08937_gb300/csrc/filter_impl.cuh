@@ -894,6 +894,77 @@ __device__ __forceinline__ void weights2(const FilterArgs& a, int64_t t, df (&c)
         : "l"(a.csdf + t));
 }
 
+// The sums of one run to the map, out of line: ten copies of it (six integer
+// conversions each) beside the transform's passes do not fit the instruction
+// cache of an SM whose 16 warps run them in step.
+static __device__ __noinline__ void flush_run(V4<double>* q, df a, df b, df c) { atomic_add3(q, a, b, c); }
+
+// scatter8_t in a loop over pairs of samples, for kernels of one 512-thread
+// double-float CTA per SM.  All its warps scatter at the same time, so nothing
+// hides instruction fetch: with the eight samples unrolled 1.39 of the 8 stall
+// cycles per instruction were missing instructions (0.69 with four samples and
+// shuffled sums).  A x, 1.34e8 samples, M = 9216: 3.93 ms with four samples and
+// shuffled sums, 4.17 unrolled, 3.84 so; b of it 4.50, 3.77, 3.64 ms.  CTAs of
+// 256 threads, two an SM, cover each other's fetches: 0.966 ms unrolled and
+// 0.976 so at M = 2304 and 3.4e7 samples.
+template <int NW, typename Z>
+__device__ __forceinline__ void scatter8_pairs(const FilterArgs& a, const Seg& S, bool act, Z z) {
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    V4<double>* q = reinterpret_cast<V4<double>*>(a.dst) + (int64_t)(act ? S.rhs : 0) * a.n_pix;
+    const int n = act ? S.n_out : 0;
+#pragma unroll 1
+    for (int base = warp * 256; base < n; base += NW * 256) {
+        const int i0 = base + 8 * lane;
+        const int64_t t0 = S.out0 + i0;
+        const bool pairs = (t0 & 1) == 0 && i0 + 8 <= n;
+        df a0(0), a1(0), a2(0), b0(0), b1(0), b2(0);
+        bool multi = false;
+        int first = -1, last = -1;
+#pragma unroll 1
+        for (int g = 0; g < 8; g += 2) {
+            int p[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) p[j] = i0 + g + j < n ? __ldg(a.pix + t0 + g + j) : -1;
+            df c[2], sn[2];
+            if (pairs) weights2(a, t0 + g, c, sn);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                if (!pairs && p[j] >= 0) weights(a, t0 + g + j, c[j], sn[j]);
+                if (j == 0 && g == 0) first = last = p[0];
+                if (p[j] != last) {
+                    if (multi) {
+                        if (last >= 0) flush_run(q + last, a0, a1, a2);
+                    } else {
+                        b0 = a0;
+                        b1 = a1;
+                        b2 = a2;
+                        multi = true;
+                    }
+                    a0 = a1 = a2 = df(0);
+                    last = p[j];
+                }
+                if (p[j] >= 0) {
+                    const df v = z(i0 + g + j);
+                    a0 += v;
+                    a1 = madd(v, c[j], a1);
+                    a2 = madd(v, sn[j], a2);
+                }
+            }
+        }
+        const int plast = __shfl_up_sync(FULL, last, 1);
+        const bool give = multi && lane > 0 && first == plast;
+        const df r0 = shfl_down_t(b0, 1), r1 = shfl_down_t(b1, 1), r2 = shfl_down_t(b2, 1);
+        if (__shfl_down_sync(FULL, (int)give, 1) && lane < 31) {
+            a0 += r0;
+            a1 += r1;
+            a2 += r2;
+        }
+        if (multi && !give && first >= 0) flush_run(q + first, b0, b1, b2);
+        if (last >= 0) flush_run(q + last, a0, a1, a2);
+    }
+}
+
 // P^T of a segment for float64 and double-float: eight consecutive outputs per
 // lane, z(i) the filtered sample i.  A lane sums its runs of equal pixels one
 // after the other (three operations per sample; a warp instruction of the
@@ -905,6 +976,7 @@ __device__ __forceinline__ void weights2(const FilterArgs& a, int64_t t, df (&c)
 // pipe 35 -> 4 % busy), A x in float64 on ragged blocks 0.833 -> 0.736 ms.
 template <typename T, int NW, typename Z>
 __device__ __forceinline__ void scatter8_t(const FilterArgs& a, const Seg& S, bool act, Z z) {
+    if constexpr (std::is_same<T, df>::value && NW >= 16) return scatter8_pairs<NW>(a, S, act, z);
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     V4<typename AccT<T>::type>* q = reinterpret_cast<V4<typename AccT<T>::type>*>(a.dst) + (int64_t)(act ? S.rhs : 0) * a.n_pix;
