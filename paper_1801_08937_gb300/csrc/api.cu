@@ -68,6 +68,7 @@ struct Plan {
     FftPasses fp{};
     bool three = false;   // whole = 2, float32: the three-pass transform
     bool even = true;     // every segment starts at an even sample
+    int tiles = 1;        // direct: tiles of V outputs per listed segment
     int f64 = 0;
     int nrhs = 0;
     std::vector<int64_t> lens;
@@ -554,8 +555,15 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
             *out = p.get();
             return MM_OK;
         }
+    // the eight-outputs-a-thread direct filter cuts its segments into tiles itself, up to eight: the list is filled on
+    // the host for every new scan, and with one entry per tile of 1024 that cost more than the small tiles gain
+    // (first product on 3.4e7 samples, lambda 16: 0.52 ms in tiles of 2048, 0.49 in tiles of 1024, 0.24 so; lambda 0:
+    // 0.30, 0.41, 0.16)
+    int tiles = 1;
+    if (variant == 1 && f64 == 0 && direct8_shape(V, ctx->lam))
+        while (tiles < 8 && 2 * (int64_t)tiles * V <= max_block_len(ctx)) tiles *= 2;
     std::vector<Seg> segs;
-    segs.reserve((size_t)nrhs * (whole ? ctx->n_blocks + 1 : ctx->n_samples / std::max(1, V) + ctx->n_blocks + 1) + 2);
+    segs.reserve((size_t)nrhs * (whole ? ctx->n_blocks + 1 : ctx->n_samples / std::max(1, V * tiles) + ctx->n_blocks + 1) + 2);
     const bool single = (variant == 2 && whole >= 2);   // segments one by one, not in pairs
     auto push = [&](const Seg& s) {
         if (!single && segs.size() % 2 == 1 && (segs.back().band != s.band || segs.back().shift != s.shift)) {
@@ -570,7 +578,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     for (int b = 0; b < ctx->n_blocks; ++b) {
         const int64_t o0 = ctx->block_off[b], o1 = ctx->block_off[b + 1];
         const int64_t det0 = (o0 / ctx->n_t) * ctx->n_t;
-        const int64_t step = whole ? (o1 - o0) : V;
+        const int64_t step = whole ? (o1 - o0) : (int64_t)V * tiles;
         for (int64_t c0 = o0; c0 < o1; c0 += step) {
             for (int r = 0; r < nrhs; ++r) {
                 int64_t hi = o1;
@@ -608,6 +616,7 @@ mm_status make_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_t>& 
     if (!tables) p->ft->L = 0;   // a kept plan's are another scan's
     p->three = false;
     p->even = true;
+    p->tiles = tiles;
     p->variant = variant;
     p->L = L;
     p->logL = logL;
@@ -968,6 +977,7 @@ mm_status run_filter(mm_ctx* ctx, Plan* plan, bool from_tod, const void* src, vo
         else if (plan->f64 == 1) launch_filter_fft_f64(a, from_tod, ctx->stream);
         else launch_filter_fft_f32(a, from_tod, ctx->stream);
     } else {
+        a.tiles_log = ilog2(plan->tiles);
         a.band = plan->f64 == 2 ? ctx->d_banddf.p : (plan->f64 ? ctx->d_band64.p : ctx->d_band32.p);
         if (plan->f64 == 2) launch_filter_direct_df(a, from_tod, ctx->stream);
         else if (plan->f64 == 1) launch_filter_direct_f64(a, from_tod, ctx->stream);

@@ -131,6 +131,7 @@ struct FilterArgs {
     unsigned wait_ns;      // its limit
     int ahead;             // CTAs on the device at a time: the pointing of the CTA so many later goes to L2
     const void* band;      // direct: [n_bands][lambda+1]
+    int tiles_log;         // direct, float32: log2 of the tiles of V outputs per listed segment (direct8_shape)
     int L, logL, lam, V;
     FftPasses fp;
     const RhsState* state; // may be null: all right-hand sides active
@@ -197,6 +198,8 @@ void launch_weights_df(const float* psi, const double2* cs64, const TrigTable& t
                        cudaStream_t s);   // from the stored float64 weights where there are any
 void launch_map_to_df(const V4<double>* src, void* dst, int64_t n, cudaStream_t s);
 size_t fft_smem_bytes(int L, bool f64);
+// float32 direct filters with eight outputs per thread: tiles of 1024 or 2048, bands up to 16 taps each side
+inline bool direct8_shape(int V, int lam) { return (V == 1024 || V == 2048) && lam <= 16; }
 size_t direct_smem_bytes(int V, int lam, bool f64);
 // H = DIF(h) for each band in float64 through global scratch; h [n_bands][L].
 void launch_fft_spectrum(const double* h, double* H_out, double2* work, const double2* tw,

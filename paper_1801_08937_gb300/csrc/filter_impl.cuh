@@ -1726,7 +1726,10 @@ __global__ void __launch_bounds__(NT) k_filter_direct8(const FilterArgs a) {
     const int i0 = 8 * threadIdx.x;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-        const Seg S = a.segs[2 * blockIdx.x + half];
+        const int u = 2 * blockIdx.x + half, tile = u & ((1 << a.tiles_log) - 1);
+        Seg S = a.segs[u >> a.tiles_log];
+        S.out0 += tile * (8 * NT);   // a tile of the segment (none behind its end)
+        S.n_out = min(8 * NT, S.n_out - tile * (8 * NT));
         if (!seg_active<float>(a, S)) continue;   // uniform across the CTA
         const float* band = reinterpret_cast<const float*>(a.band) + (int64_t)S.band * (lam + 1);
         for (int k = threadIdx.x; k <= LMAX; k += NT) c[k] = k <= lam ? band[k] : 0.0f;
@@ -1973,12 +1976,11 @@ template <typename T, bool FROM_TOD>
 inline void launch_direct_t(const FilterArgs& a, cudaStream_t s) {
     if (a.n_work <= 0) return;
     if constexpr (std::is_same<T, float>::value) {
-        // lean kernel: tiles of 1024 or 2048 outputs, eight per thread, bands up to 16 taps each side
-        if ((a.V == 1024 || a.V == 2048) && a.lam <= 16) {
+        if (direct8_shape(a.V, a.lam)) {
             const int lmax = a.lam == 0 ? 0 : (a.lam <= 4 ? 4 : (a.lam <= 8 ? 8 : 16));
             const size_t sm = (size_t)(((lmax + 1 + 3) & ~3) + a.V + 2 * lmax + 4) * sizeof(float);
             auto go = [&](auto kern) {
-                kern<<<a.n_work, a.V / 8, sm, s>>>(a);
+                kern<<<a.n_work << a.tiles_log, a.V / 8, sm, s>>>(a);
                 count_launches(1);
             };
             if (a.V == 2048) {
