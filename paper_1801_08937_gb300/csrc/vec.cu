@@ -866,6 +866,7 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
             s = f2d_exact(sf);
         } else {
             const V4<double>* zc = a.Z + (int64_t)c * a.n_pix;
+#pragma unroll 4
             for (int i = i0 + lane; i < i1; i += 32) s += dot3(zc[i], v[off + i]);
         }
         s = warp_sum(s);
@@ -890,8 +891,8 @@ __global__ void k_m2l_ztr(const PcgArgs a, const V4<double>* v) {
 
 // out = M_BD (v - AZ u) + Z u  (Sect. 3.2, Eq. m2l); with finalize_beta >= 0
 // it also forms v^T out and updates rz/beta like k_bd_dot.
-// G lanes per pixel, each 1/G of the coarse vectors.
-template <int G>
+// G lanes per pixel, each 1/G of the coarse vectors, U of them in flight in float64.
+template <int G, int U>
 __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* out, int finalize_beta) {
     const int rhs = blockIdx.y;
     if (a.st && !a.st[rhs].active) return;
@@ -933,7 +934,7 @@ __global__ void k_m2l_apply(const PcgArgs a, const V4<double>* v, V4<double>* ou
                 zy = f2d_exact(hy);
                 zz = f2d_exact(hz);
             } else {
-#pragma unroll 4
+#pragma unroll U
                 for (int c = g; c < a.k; c += G) {
                     const V4<double> azc = AZ[(int64_t)c * a.n_pix + i];
                     const V4<double> zc = a.Z[(int64_t)c * a.n_pix + i];
@@ -1029,11 +1030,16 @@ void launch_precond_bd_dot(const PcgArgs& a, int finalize_beta, cudaStream_t s) 
 }
 // CTAs of k_m2l_ztr at most (the partials hold this many entries per value).
 int m2l_ztr_grid(int n_pix) { return std::min(304, (n_pix + 63) / 64); }
-// A small map is cut into chunks down to 64 pixels, so that its k vectors spread over more SMs, until all
-// right-hand sides together have 304 CTAs; from there on chunks of 256, whose warp sums weigh less (64 right-hand
-// sides, 10^4 pixels, k = 8, float64: 325 us a call in chunks of 64 with four lanes a pixel below, 208 so).
+// Chunks of whole warps (a ragged last row of 32 pixels costs the float64 pipe a full one), at least 64 and at
+// most 256 pixels: one CTA per SM over all right-hand sides where that fits, else two.  Microseconds a call, one
+// right-hand side, k = 32, float64, with 304 chunks whatever their length / with chunks of 256 / so (all with four
+// lanes a pixel up to 16384 pixels and the loops unrolled below): 128 x 128 and 140 x 140 84 / 83 / 75, 180 x 180
+// 94 / 83 / 78, 220 x 220 105 / 121 / 104.
 static int m2l_grid(int n_pix, int nrhs) {
-    return std::min(304, std::max((n_pix + VT - 1) / VT, std::min((n_pix + 63) / 64, 304 / std::max(1, nrhs))));
+    auto chunk = [&](int ctas) { return std::max(64, ((n_pix + ctas - 1) / ctas + 31) / 32 * 32); };
+    const int w = std::max(2, 304 / std::max(1, nrhs)), c1 = chunk(w / 2), c2 = chunk(w);
+    const int c = std::min(256, c1 <= 256 ? c1 : c2);
+    return std::min(304, (n_pix + c - 1) / c);
 }
 void launch_m2l_ztr(const PcgArgs& a, const V4<double>* v, cudaStream_t s) {
     const dim3 grid(m2l_grid(a.n_pix, a.nrhs), a.nrhs);
@@ -1041,15 +1047,20 @@ void launch_m2l_ztr(const PcgArgs& a, const V4<double>* v, cudaStream_t s) {
     else k_m2l_ztr<false><<<grid, VT, 0, s>>>(a, v);
     count_launches(1);
 }
-// Four lanes per pixel while they all fit on the device at once (152 x 2048 threads): a small map still fills the
-// SMs' float64 pipes and the loads of a pixel's vectors are in flight together.  Beyond that one lane per pixel
-// spares the lanes' sums, which are float64 adds (8 right-hand sides of 14400 pixels, k = 64: 268 -> 244 us a call with
-// the chunks above; 90000 pixels, k = 32, alone: 142 and 141).
+// Four lanes per pixel on small maps: the SMs' float64 pipes are filled and the loads of a pixel's vectors are in
+// flight together.  From 16384 pixels on (over all right-hand sides) one lane per pixel spares the lanes' sums,
+// which are float64 adds, and eight vectors in flight take their place for a single right-hand side.  k = 32, float64,
+// us a call, four lanes / one: 100 x 100 72 / 78, 140 x 140 86 / 84, 180 x 180 101 / 93, 256 x 256 126 / 112.  One
+// lane, four / eight in flight: 300 x 300 144 / 139; eight right-hand sides of 120 x 120, k = 64: 223 / 252.  Float32
+// coarse sums (a.Z32) keep four lanes while all of them fit on the device at once.
 void launch_m2l_apply(const PcgArgs& a, const V4<double>* v, V4<double>* out, int finalize_beta, cudaStream_t s) {
-    if ((int64_t)a.n_pix * a.nrhs <= 152 * 2048 / 4)
-        k_m2l_apply<4><<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+    const int rows = std::min(304, (a.n_pix + VT - 1) / VT);
+    if ((int64_t)a.n_pix * a.nrhs < (a.Z32 ? 152 * 2048 / 4 : 16384))
+        k_m2l_apply<4, 4><<<dim3(m2l_ztr_grid(a.n_pix), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+    else if (a.nrhs == 1)
+        k_m2l_apply<1, 8><<<dim3(rows, a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
     else
-        k_m2l_apply<1><<<dim3(std::min(304, (a.n_pix + VT - 1) / VT), a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
+        k_m2l_apply<1, 4><<<dim3(rows, a.nrhs), VT, 0, s>>>(a, v, out, finalize_beta);
     count_launches(1);
 }
 
