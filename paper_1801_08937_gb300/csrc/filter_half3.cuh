@@ -79,9 +79,8 @@ __device__ __forceinline__ bool h3_bar_try(uint32_t bar, uint32_t parity) {
                  : "memory");
     return done != 0;
 }
-// false if the copy has not landed after `limit` nanoseconds (0: without a look)
+// false if the copy has not landed after `limit` nanoseconds
 __device__ __forceinline__ bool h3_bar_wait(uint32_t bar, uint32_t parity, unsigned limit) {
-    if (limit == 0) return false;
     if (h3_bar_try(bar, parity)) return true;
     unsigned long long t0, t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
@@ -255,7 +254,7 @@ __global__ void __launch_bounds__(H::NT, H::MINB) k_filter_half3(const FilterArg
                 for (int i = j; i < S.nwin; i += H::NT)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * i), "l"(map + S.win0 + i) : "memory");
             asm volatile("cp.async.wait_all;" ::: "memory");
-            bool ok = true;
+            bool ok = a.wait_ns != 0;   // a limit of zero gives up without a look
             int issued = min(NS, nch);   // thread 0: chunks asked for
             auto rows = [&](auto entry) {
 #pragma unroll
