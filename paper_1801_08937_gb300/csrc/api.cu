@@ -840,7 +840,8 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
         const mm_status warm = run_filter(ctx, p, false, src.p, dst.p, nullptr, 0);
         p->n_work = n_work;
         TRY(warm);
-        // best of up to three timed launches (one when a launch is long)
+        // best of up to three timed launches (one when a launch is long; of a batch one, or two when it comes
+        // within a tenth of the best so far: plans of nearly the same time are told apart by the second)
         double ms_best = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
             CK(cudaEventRecord(t.e0, ctx->stream));
@@ -851,7 +852,7 @@ mm_status autotune_plan(mm_ctx* ctx, int f64, int nrhs, const std::vector<int64_
             float ms = 0.f;
             CK(cudaEventElapsedTime(&ms, t.e0, t.e1));
             ms_best = std::min(ms_best, (double)ms);
-            if (ms > (single ? 0.3 : 2.0)) break;
+            if (ms > 2.0 || (single && ms > 0.3 && (rep == 1 || ms > 1.1 * best->ms))) break;
         }
         if (ms_best < best->ms) *best = TuneVal{o.variant, o.L, o.whole, o.V, ms_best};
     }
