@@ -1126,7 +1126,7 @@ mm_status pcg_iteration(mm_ctx* ctx) {
         CKL();
         return MM_OK;
     }
-    launch_pcg_src(a, 0, ctx->stream);
+    launch_pcg_src(a, ctx->stream);
     TRY(run_filter(ctx, ctx->plan_op, false, ctx->s_src.p, ctx->s_q.p, a.st, 0));
     launch_pcg_pq(a, ctx->stream);
     const int two = ctx->precond == MM_PRECOND_2L;
@@ -1153,7 +1153,7 @@ mm_status pcg_start(mm_ctx* ctx, const V4<double>* b, const std::vector<double>&
     launch_pcg_init(a, b, ctx->stream);
     precond_step(ctx, a, 0);
     if (ctx->harvest_on && ctx->precond == MM_PRECOND_BD) launch_harvest(a, ctx->stream);
-    if (pcg_stepped(ctx, a)) launch_pcg_src(a, 0, ctx->stream);
+    if (pcg_stepped(ctx, a)) launch_pcg_src(a, ctx->stream);
     CKL();
     return MM_OK;
 }

@@ -271,7 +271,7 @@ struct PcgArgs {
     int harvest_m;
 };
 void launch_pcg_init(const PcgArgs& a, const V4<double>* b, cudaStream_t s);
-void launch_pcg_src(const PcgArgs& a, int first, cudaStream_t s);
+void launch_pcg_src(const PcgArgs& a, cudaStream_t s);
 // the rest of an iteration with M_BD behind the product, in one launch (small maps): pq, update and the next src
 bool pcg_step_fits(const PcgArgs& a);
 void launch_pcg_step(const PcgArgs& a, cudaStream_t s);

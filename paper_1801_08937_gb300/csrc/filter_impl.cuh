@@ -1227,136 +1227,15 @@ __device__ __forceinline__ void half_gather_f32_map(const FilterArgs& a, const S
     }
 }
 
-// P^T of a warp's 128 consecutive samples, four per lane in order: one atomic
-// per run of equal pixels.  Within a lane, suffix sums over each run; the
-// lane's last run continues into the following lanes while their first
-// pixel is the same, and its continuation X(l) = a(l) + b(l) X(l + 1)
-// (a = the next lane's leading run when the run continues, b = that run fills
-// the next lane) is solved by doubling, taking only the steps the longest
-// chain needs.  Every sample is counted once: at the first sample of its run
-// inside this warp's 128.
-__device__ __forceinline__ void warp_run_scatter(const int (&p)[4], float (&v0)[4], float (&v1)[4], float (&v2)[4],
-                                                 V4<float>* q) {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const bool e01 = p[0] == p[1], e12 = p[1] == p[2], e23 = p[2] == p[3];
-    if (e23) { v0[2] += v0[3]; v1[2] += v1[3]; v2[2] += v2[3]; }
-    if (e12) { v0[1] += v0[2]; v1[1] += v1[2]; v2[1] += v2[2]; }
-    if (e01) { v0[0] += v0[1]; v1[0] += v1[1]; v2[0] += v2[1]; }
-    const bool whole = e01 && e12 && e23;
-    const int pnext = __shfl_down_sync(FULL, p[0], 1);
-    const bool cont = lane < 31 && pnext == p[3];
-    float x0 = __shfl_down_sync(FULL, v0[0], 1);
-    float x1 = __shfl_down_sync(FULL, v1[0], 1);
-    float x2 = __shfl_down_sync(FULL, v2[0], 1);
-    const bool wnext = __shfl_down_sync(FULL, (int)whole, 1) != 0;
-    if (!cont) { x0 = 0.0f; x1 = 0.0f; x2 = 0.0f; }
-    bool chain = cont && wnext;
-#pragma unroll 1
-    for (int d = 1; __any_sync(FULL, chain); d <<= 1) {
-        const float y0 = __shfl_down_sync(FULL, x0, d);
-        const float y1 = __shfl_down_sync(FULL, x1, d);
-        const float y2 = __shfl_down_sync(FULL, x2, d);
-        const bool cn = __shfl_down_sync(FULL, (int)chain, d) != 0;
-        if (chain) { x0 += y0; x1 += y1; x2 += y2; }
-        chain = chain && cn;
-    }
-    const int plast = __shfl_up_sync(FULL, p[3], 1);
-    // heads: the first sample of each run; a run reaching the lane end adds X
-    const bool h0 = lane == 0 || p[0] != plast;
-    if (h0 && p[0] >= 0) {
-        const float w = whole ? 1.0f : 0.0f;
-        atomic_add3(q + p[0], fmaf(w, x0, v0[0]), fmaf(w, x1, v1[0]), fmaf(w, x2, v2[0]));
-    }
-    if (!e01 && p[1] >= 0) {
-        const float w = (e12 && e23) ? 1.0f : 0.0f;
-        atomic_add3(q + p[1], fmaf(w, x0, v0[1]), fmaf(w, x1, v1[1]), fmaf(w, x2, v2[1]));
-    }
-    if (!e12 && p[2] >= 0) {
-        const float w = e23 ? 1.0f : 0.0f;
-        atomic_add3(q + p[2], fmaf(w, x0, v0[2]), fmaf(w, x1, v1[2]), fmaf(w, x2, v2[2]));
-    }
-    if (!e23 && p[3] >= 0) atomic_add3(q + p[3], v0[3] + x0, v1[3] + x1, v2[3] + x2);
-}
-
-// Loads in flight per thread in the float32 gather (groups of four samples)
-// and in the scatter (warp iterations of 128 samples).
-constexpr int HALF_GB = 1;
-constexpr int HALF_SU = 1;
-
-// float32 gather: each thread fills two complex points (four samples) per
-// group, GB groups per iteration.  The pointing of the next iteration is
-// requested before the map entries of the current one, so its DRAM latency
-// overlaps the L2 latency and arithmetic of this iteration.
-template <bool FROM_TOD, int NT>
-__device__ __forceinline__ void half_gather_f32(const FilterArgs& a, const Seg& S, C2<float>* s, int M) {
-    constexpr int GB = HALF_GB;
+// float32 gather from a timeline: each thread fills two complex points (four samples) per step.
+template <int NT>
+__device__ __forceinline__ void half_gather_f32_tod(const FilterArgs& a, const Seg& S, C2<float>* s, int M) {
     const int ng = M >> 1;
-    auto store = [&](int u0, const float (&y)[GB][4]) {
-#pragma unroll
-        for (int g = 0; g < GB; ++g) {
-            const int u = u0 + g * NT;
-            if (u < ng) {
-                s[sidx(2 * u)] = C2<float>{y[g][0], y[g][1]};
-                s[sidx(2 * u + 1)] = C2<float>{y[g][2], y[g][3]};
-            }
-        }
-    };
-    if constexpr (FROM_TOD) {
-        for (int u0 = threadIdx.x; u0 < ng; u0 += NT * GB) {
-            float y[GB][4];
-#pragma unroll
-            for (int g = 0; g < GB; ++g) {
-                const int u = u0 + g * NT;
-                load4_tod(a, S, 4 * u, u < ng && 4 * u < S.n_out, y[g]);
-            }
-            store(u0, y);
-        }
-    } else {
-        const V4<float>* map = reinterpret_cast<const V4<float>*>(a.src) + (int64_t)S.rhs * a.n_pix;
-        auto pointing = [&](int u0, int (&p)[GB][4], float (&ps)[GB][4]) {
-#pragma unroll
-            for (int g = 0; g < GB; ++g) {
-                const int u = u0 + g * NT;
-                const int i0 = 4 * u;
-                load4(a, S.out0 + i0, u < ng && i0 < S.n_out, S.n_out - i0, p[g], ps[g]);
-            }
-        };
-        int p[GB][4];
-        float ps[GB][4];
-        pointing(threadIdx.x, p, ps);
-        for (int u0 = threadIdx.x; u0 < ng; u0 += NT * GB) {
-            int pn[GB][4];
-            float psn[GB][4];
-            pointing(u0 + NT * GB, pn, psn);
-            V4<float> m[GB][4];
-#pragma unroll
-            for (int g = 0; g < GB; ++g)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (p[g][j] >= 0) m[g][j] = ldmap<float>(map + p[g][j]);
-            float y[GB][4];
-#pragma unroll
-            for (int g = 0; g < GB; ++g)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float v = 0.0f;
-                    if (p[g][j] >= 0) {
-                        float c, sn;
-                        weights_from(a, 0, ps[g][j], c, sn);
-                        v = m[g][j].x + c * m[g][j].y + sn * m[g][j].z;
-                    }
-                    y[g][j] = v;
-                }
-            store(u0, y);
-#pragma unroll
-            for (int g = 0; g < GB; ++g)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    p[g][j] = pn[g][j];
-                    ps[g][j] = psn[g][j];
-                }
-        }
+    for (int u = threadIdx.x; u < ng; u += NT) {
+        float y[4];
+        load4_tod(a, S, 4 * u, 4 * u < S.n_out, y);
+        s[sidx(2 * u)] = C2<float>{y[0], y[1]};
+        s[sidx(2 * u + 1)] = C2<float>{y[2], y[3]};
     }
 }
 
@@ -1548,7 +1427,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 512 / NT) k_filter_ha
     const int M = MCT > 0 ? MCT : a.L;
     const C2<T>* tw = reinterpret_cast<const C2<T>*>(a.tw);
     if constexpr (std::is_same<T, float>::value && !FROM_TOD) half_gather_f32_map<NT>(a, S, s, M);
-    else if constexpr (std::is_same<T, float>::value) half_gather_f32<FROM_TOD, NT>(a, S, s, M);
+    else if constexpr (std::is_same<T, float>::value) half_gather_f32_tod<NT>(a, S, s, M);
     else half_gather_t<T, FROM_TOD, NT>(a, S, s, M);
     __syncthreads();
     if constexpr (MCT > 0) {

@@ -585,10 +585,10 @@ __device__ __forceinline__ void pcg_direction(const PcgArgs& a, int64_t j, doubl
         reinterpret_cast<V4<double>*>(a.qacc)[j] = V4<double>{0, 0, 0, 0};
     }
 }
-__global__ void k_pcg_src(const PcgArgs a, int first) {
+__global__ void k_pcg_src(const PcgArgs a) {
     const int rhs = blockIdx.y;
     if (!a.st[rhs].active) return;
-    const double beta = first ? 0.0 : a.st[rhs].beta;
+    const double beta = a.st[rhs].beta;
     const int64_t off = (int64_t)rhs * a.n_pix;
     PIX_LOOP(i) pcg_direction(a, off + i, beta);
 }
@@ -1001,8 +1001,8 @@ void launch_pcg_init(const PcgArgs& a, const V4<double>* b, cudaStream_t s) {
     k_pcg_init<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, b);
     count_launches(1);
 }
-void launch_pcg_src(const PcgArgs& a, int first, cudaStream_t s) {
-    k_pcg_src<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a, first);
+void launch_pcg_src(const PcgArgs& a, cudaStream_t s) {
+    k_pcg_src<<<dim3(a.grid_x, a.nrhs), VT, 0, s>>>(a);
     count_launches(1);
 }
 bool pcg_step_fits(const PcgArgs& a) { return a.n_pix <= STEP_MAX_PIX; }
