@@ -314,7 +314,8 @@ mm_status mm_solve(mm_ctx* ctx, const void* tod, double* map_out, int32_t nrhs,
 mm_status mm_set_option(mm_ctx* ctx, const char* name, double value);
 
 /* Read back a tuning knob or statistic: any knob above, or "last_apply_ms"
- * (device time of the last mm_apply_A), "filter_launches" and "filter_ms"
+ * (device time of the last mm_apply_A from the conversion of its input to that
+ * of its output, without copies from and to the host), "filter_launches" and "filter_ms"
  * (filter launches timed since the last read of "filter_ms", and their total
  * device time; reading "filter_ms" resets both), "kernel_launches" (kernels
  * launched by the library since load), "plan_fft_len", "plan_fft_log2",
