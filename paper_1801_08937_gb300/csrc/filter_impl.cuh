@@ -901,9 +901,9 @@ static __device__ __noinline__ void flush_run(V4<double>* q, df a, df b, df c) {
 
 // scatter8_t in a loop over pairs of samples, for kernels of one 512-thread
 // double-float CTA per SM.  All its warps scatter at the same time, so nothing
-// hides instruction fetch: with the eight samples unrolled 1.39 of the 8 stall
-// cycles per instruction were missing instructions (0.69 with four samples and
-// shuffled sums).  A x, 1.34e8 samples, M = 9216: 3.93 ms with four samples and
+// hides instruction fetch: with the eight samples unrolled a warp waited 1.39
+// cycles per issued instruction for instructions (0.69 with four samples and
+// shuffled sums, 0.50 so).  A x, 1.34e8 samples, M = 9216: 3.93 ms with four samples and
 // shuffled sums, 4.17 unrolled, 3.84 so; b of it 4.50, 3.77, 3.64 ms.  CTAs of
 // 256 threads, two an SM, cover each other's fetches: 0.966 ms unrolled and
 // 0.976 so at M = 2304 and 3.4e7 samples.
